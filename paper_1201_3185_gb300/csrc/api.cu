@@ -839,12 +839,15 @@ BoxSet box_set(const qumond_ctx* c, const double* const* phis)
     memset(&bs, 0, sizeof(bs));
     bs.nboxes = c->p.nboxes;
     bs.n = c->p.n;
+    const double top = (double)(c->p.n - 1);
+    memcpy(&bs.top, &top, sizeof(top));
     for (int b = 0; b < c->p.nboxes; ++b) {
         const double L = box_side(c, b);
         bs.b[b].phi = phis[b];
         bs.b[b].L = L;
         bs.b[b].h = L / (double)c->p.n;
         bs.b[b].inv_h = (double)c->p.n / L;
+        bs.b[b].s = -0.5 / bs.b[b].h;
         bs.b[b].xlo = c->p.center[0] - 0.5 * L;
         bs.b[b].ylo = c->p.center[1] - 0.5 * L;
         bs.b[b].zlo = c->p.center[2] - 0.5 * L;

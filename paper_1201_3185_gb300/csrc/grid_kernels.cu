@@ -334,43 +334,90 @@ source_kernel(const double* __restrict__ phi, double* __restrict__ src, int n, f
 
 // ---------------------------------------------------------------------------
 // Forces at points: finest box whose containing cell has 8 interior corners.
-__device__ __forceinline__ bool find_cell(const BoxGeom& g, int n, double x, double y, double z, int* ijk, double* d)
+//
+// These kernels are bound by the FP64 pipe (2 operations a clock on each SM,
+// against 64 integer ones), so what is not arithmetic of the result runs on
+// the integer pipe, and a warp looks for every point's box first and
+// interpolates once: with the interpolation inside the search, the points of
+// a warp that lie in different boxes ran it one box after another.
+// Measured at 2e6 points in 3 boxes of 257^3: 336 us, 824 us with the search
+// around the interpolation and the 8 corners weighted one by one (222 FP64
+// instructions a point, that pipe 86% busy).  The rounding error against
+// extended precision is the same (1.05e-16 and 1.07e-16 of the rms force).
+
+// Index coordinates of (x, y, z) in box g, and whether the containing cell has
+// interior corners only: 1 <= t < n-1 on each axis.  `top` holds the bits of
+// (double)(n-1); positive doubles order as their bits do, negative ones and
+// NaNs with the sign bit are negative integers, other NaNs lie above.
+__device__ __forceinline__ bool in_cells(const BoxGeom& g, long long top, double x, double y, double z, double* t)
 {
-    const double t[3] = {(x - g.xlo) * g.inv_h, (y - g.ylo) * g.inv_h, (z - g.zlo) * g.inv_h};
+    t[0] = (x - g.xlo) * g.inv_h;
+    t[1] = (y - g.ylo) * g.inv_h;
+    t[2] = (z - g.zlo) * g.inv_h;
+    bool ok = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (!(t[a] >= 1.0 && t[a] < (double)(n - 1))) return false;
-        const double fl = floor(t[a]);
-        ijk[a] = (int)fl;
-        d[a] = t[a] - fl;
-        if (ijk[a] < 1 || ijk[a] > n - 2) return false;
+        const long long b = __double_as_longlong(t[a]);
+        ok = ok && b >= 0x3ff0000000000000LL && b < top;
     }
-    return true;
+    return ok;
 }
 
-// set: which of the context's sets (its potentials sit at set (n+1)^3 in every box)
-__device__ __forceinline__ void grad_at(const BoxGeom& g, int n, const int* ijk, const double* d, double* out,
-                                        int set = 0)
+// Integer part of 1 <= t < 2^20 and the offset t - floor(t): the integer part
+// is the top of the significand, and t without the bits below it is floor(t).
+__device__ __forceinline__ int cell_of(double t, double& d)
 {
-    const double* phi = g.phi + set * nat_elems(n);
-    const double s = -0.5 / g.h;
-    const long long P = n + 1, Q = P * P;
-    double gx = 0.0, gy = 0.0, gz = 0.0;
+    const int hi = __double2hiint(t);
+    const int sh = 1043 - (hi >> 20);  // 20 - exponent: fraction bits in the high word
+    d = t - __hiloint2double(hi & (int)(0xffffffffu << sh), 0);
+    return ((hi & 0xfffff) | 0x100000) >> sh;
+}
+
+// -grad Phi at index coordinates t of box g (in_cells): central differences at
+// the cell's corners with CIC weights.  Along each axis the differences of a
+// row are weighted first and the four rows after, 22 FP64 operations per
+// component where weighting the 8 corners one by one takes 24 and the weights.
+// set: which of the context's sets (its potentials sit at set (n+1)^3 in every box)
+__device__ __forceinline__ void grad_at(const double* __restrict__ phi, double s, int n, const double* t, double* out)
+{
+    double d[3], w[3];
+    int c[3];
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                const long long o = nat(n, ijk[0] + a, ijk[1] + b, ijk[2] + c);
-                const double w = (a ? d[0] : 1.0 - d[0]) * (b ? d[1] : 1.0 - d[1]) * (c ? d[2] : 1.0 - d[2]);
-                gx += w * ((phi[o + 1] - phi[o - 1]) * s);
-                gy += w * ((phi[o + P] - phi[o - P]) * s);
-                gz += w * ((phi[o + Q] - phi[o - Q]) * s);
-            }
-    out[0] = gx;
-    out[1] = gy;
-    out[2] = gz;
+    for (int a = 0; a < 3; ++a) {
+        c[a] = cell_of(t[a], d[a]);
+        w[a] = 1.0 - d[a];
+    }
+    const int P = n + 1;
+    const long long Q = (long long)P * P;
+    const double* p = phi + (c[0] + (long long)P * c[1] + Q * c[2]);
+    // rows along axis U (stride u) at the corners (0, v), (0, z): the weighted difference of the row
+    auto part = [&](long long u, long long v, long long z, int U, int V, int Z) {
+        auto row = [&](const double* r) {
+            return fma(r[2 * u] - r[0], d[U], (r[u] - r[-u]) * w[U]);
+        };
+        const double lo = fma(row(p + v), d[V], row(p) * w[V]);
+        const double hi = fma(row(p + v + z), d[V], row(p + z) * w[V]);
+        return fma(hi, d[Z], lo * w[Z]) * s;
+    };
+    out[0] = part(1, P, Q, 0, 1, 2);
+    out[1] = part(P, 1, Q, 1, 0, 2);
+    out[2] = part(Q, 1, P, 2, 0, 1);
+}
+
+// g = -grad Phi at (x, y, z) from the finest box b <= b0 whose cell is interior; 0 where there is none.
+__device__ __forceinline__ void force_at(const BoxSet& boxes, int b0, double x, double y, double z, int set, double* g)
+{
+    double t[3];
+    const double* phi = nullptr;
+    double s = 0.0;
+    for (int b = b0; b >= 0; --b)
+        if (in_cells(boxes.b[b], boxes.top, x, y, z, t)) {
+            phi = boxes.b[b].phi;
+            s = boxes.b[b].s;
+            break;
+        }
+    g[0] = g[1] = g[2] = 0.0;
+    if (phi) grad_at(phi + set * nat_elems(boxes.n), s, boxes.n, t, g);
 }
 
 __global__ void forces_kernel(BoxSet boxes, const double* __restrict__ qx, const double* __restrict__ qy,
@@ -384,16 +431,8 @@ __global__ void forces_kernel(BoxSet boxes, const double* __restrict__ qx, const
     }
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= nq) return;
-    const double x = qx[p], y = qy[p], z = qz[p];
-    double g[3] = {0.0, 0.0, 0.0};
-    for (int b = boxes.nboxes - 1; b >= 0; --b) {
-        int ijk[3];
-        double d[3];
-        if (find_cell(boxes.b[b], boxes.n, x, y, z, ijk, d)) {
-            grad_at(boxes.b[b], boxes.n, ijk, d, g, set);
-            break;
-        }
-    }
+    double g[3];
+    force_at(boxes, boxes.nboxes - 1, qx[p], qy[p], qz[p], set, g);
     gx[p] = g[0];
     gy[p] = g[1];
     gz[p] = g[2];
@@ -426,16 +465,8 @@ __global__ void rotation_curve_kernel(BoxSet boxes, double cx, double cy, double
         const double ph = 6.283185307179586476925286766559 * (double)m / (double)nphi;
         double s, c;
         sincos(ph, &s, &c);
-        const double x = cx + R * c, y = cy + R * s, z = cz;
-        double g[3] = {0.0, 0.0, 0.0};
-        for (int b = b0; b >= 0; --b) {
-            int ijk[3];
-            double d[3];
-            if (find_cell(boxes.b[b], boxes.n, x, y, z, ijk, d)) {
-                grad_at(boxes.b[b], boxes.n, ijk, d, g, set);
-                break;
-            }
-        }
+        double g[3];
+        force_at(boxes, b0, cx + R * c, cy + R * s, cz, set, g);
         dphidr[m] = -(g[0] * c + g[1] * s);
     }
     __syncthreads();
@@ -475,15 +506,8 @@ __global__ void profile_kernel(BoxSet boxes, double cx, double cy, double cz, in
         const double ph = 6.283185307179586476925286766559 * (double)m / (double)nphi;
         double s, c;
         sincos(ph, &s, &c);
-        double g[3] = {0.0, 0.0, 0.0};
-        for (int b = b0; b >= 0; --b) {
-            int ijk[3];
-            double d[3];
-            if (find_cell(boxes.b[b], boxes.n, cx + R * c, cy + R * s, zt, ijk, d)) {
-                grad_at(boxes.b[b], boxes.n, ijk, d, g, set);
-                break;
-            }
-        }
+        double g[3];
+        force_at(boxes, b0, cx + R * c, cy + R * s, zt, set, g);
         if (mode == 0) {
             const double gm = sqrt(g[0] * g[0] + g[1] * g[1] + g[2] * g[2]);
             const double nu = gm > 0.0 ? 0.5 + 0.5 * sqrt(1.0 + 4.0 * a0 / gm) : 0.0;

@@ -212,12 +212,14 @@ struct BoxGeom {
     double inv_h;
     double h;
     double L;
+    double s;  // -1/(2h): central differences to -grad
 };
 constexpr int kMaxBoxes = 16;
 struct BoxSet {
     BoxGeom b[kMaxBoxes];
     int nboxes;
     int n;
+    long long top;  // the bits of (double)(n-1)
 };
 // nq points per set; with several sets, set s's points, forces, radii and
 // curves follow set s-1's, and its potentials sit at s (n+1)^3 in every box

@@ -1,0 +1,41 @@
+"""Kernels at the sizes where their index arithmetic can go wrong, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_helpers import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def q():
+    import paper_1201_3185_gb300 as q
+    return q
+
+
+@pytest.mark.parametrize("n,nboxes", [(4, 3), (8, 1), (16, 4)])
+def test_forces_at_cell_edges(q, ora, n, nboxes):
+    # points on, just inside and just outside the first and last interior cells of every box, at the centre, and
+    # points that are no number: which box a point takes and its cell must be the oracle's
+    L0 = 64.0
+    rng = np.random.default_rng(n)
+    phis = [rng.uniform(-1.0, 1.0, (n + 1) ** 3) for _ in range(nboxes)]
+    axis = [0.0, -0.0, 1e-300, L0, -L0, np.nan, -np.nan, np.inf, -np.inf]
+    for b in range(nboxes):
+        h = L0 / 2 ** b / n
+        for i in (1.0, 1.5, n / 2 + 0.25, n - 1.25, n - 1.0):
+            x = -0.5 * L0 / 2 ** b + i * h
+            axis += [x, np.nextafter(x, -np.inf), np.nextafter(x, np.inf)]
+    pts = rng.choice(np.array(axis), size=(3, 20011))
+    pts[:, :len(axis)] = axis  # the diagonal too
+    ctx = q.Context(n=n, nboxes=nboxes, L0=L0)
+    d = [to_dev(a) for a in pts]
+    g = [torch.full_like(d[0], 7.0) for _ in range(3)]
+    ctx.qumond_forces([to_dev(p) for p in phis], *d, *g)
+    want = ora.forces(n, L0, (0.0, 0.0, 0.0), phis, *pts)[:3]
+    # each side weights differences of values <= 1 with at most 24 rounded products and sums, times 1/(2h)
+    tol = 2 * 24 * 2.0 ** -53 * 2.0 / (2.0 * L0 / 2 ** (nboxes - 1) / n)
+    for a, w in zip(g, want):
+        assert np.max(np.abs(a.cpu().numpy() - w)) <= tol
+    ctx.close()
