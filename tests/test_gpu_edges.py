@@ -39,3 +39,29 @@ def test_forces_at_cell_edges(q, ora, n, nboxes):
     for a, w in zip(g, want):
         assert np.max(np.abs(a.cpu().numpy() - w)) <= tol
     ctx.close()
+
+
+@pytest.mark.parametrize("n,center", [(2, 0.0), (8, 32.0), (64, -7.3), (1024, 32.0)])
+def test_deposit_at_cell_edges_and_rounding_ties(q, ora, n, center):
+    # coordinates on, just inside and just outside the box and cell faces (centre 32: the box starts at 0, and -0.0 is
+    # in it), masses whose shares are ties, below one unit, above 2^52 (the conversion instruction) and negative
+    L0, shift = 64.0, 24
+    rng = np.random.default_rng(n)
+    lo, h = center - 0.5 * L0, L0 / n
+    axis = [0.0, -0.0, np.nan, np.inf, -np.inf, 5e-324]
+    for i in (0.0, 0.5, 1.0, 1.25, n / 2, n - 1.0, n - 0.5, n):
+        x = lo + i * h
+        axis += [x, np.nextafter(x, -np.inf), np.nextafter(x, np.inf)]
+    x, y, z = rng.choice(np.array(axis), size=(3, 4999))
+    unit = 2.0 ** -shift
+    m = rng.choice(np.array([0.0, 4.0, 12.0, 20.0, 1.0, 0.3, 1e-9, -4.0, -12.0, 1e6 + 0.7, 2.0 ** 52, 2.0 ** 52 - 1.0,
+                             2.0 ** 53 + 2.0, 2.0 ** 40 + 0.5, -2.0 ** 54]) * unit, size=4999)
+    want, _ = ora.cic_deposit(n, L0, (center,) * 3, shift, x, y, z, m)
+    ctx = q.Context(n=n, nboxes=1, L0=L0, center=(center,) * 3, deposit_shift=shift)
+    qf = torch.empty(ctx.nodes, dtype=torch.int64, device="cuda")
+    rho = torch.empty(ctx.nodes, dtype=torch.float64, device="cuda")
+    ctx.qumond_deposit(0, *(to_dev(a) for a in (x, y, z, m)), qf, rho)
+    got = qf.cpu().numpy()
+    assert np.array_equal(got, want)
+    assert np.array_equal(rho.cpu().numpy(), got * (2.0 ** -shift * (n / L0) ** 3))
+    ctx.close()
