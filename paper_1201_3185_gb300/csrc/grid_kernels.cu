@@ -214,190 +214,204 @@ __global__ void boundary_from_parent_kernel(const double* __restrict__ parent, d
 // numbers hi + lo (hi: the top 24 significant bits, lo: the next 24), and a
 // difference is (hi_a - hi_b) + (lo_a - lo_b).
 //
-// Layout: a CTA owns a 32 x 8 tile of (i, j) and walks k through a chunk of
-// planes.  Three consecutive planes of the tile plus a one-node halo sit in
-// shared memory as hi/lo pairs; every node computes the fluxes through its
-// +x, +y and +z faces once, and its source is the difference of its own
-// fluxes and those of its -x, -y, -z neighbours (the -z one carried over from
-// the previous plane).
-constexpr int kSrcTX = 32, kSrcTY = 8, kSrcKC = 16;
-constexpr int kSrcPX = kSrcTX + 2, kSrcPY = kSrcTY + 2;
+// Layout: a warp owns 30 x 2 columns of (i, j) and walks k through a chunk of
+// planes on its own, without shared memory or block barriers.  Lane l holds
+// the column i = i0 - 1 + l of the two rows and of one halo row on each side
+// in registers, as hi/lo pairs of the planes k-1, k, k+1; neighbours in x come
+// by shuffles (the outer two lanes are halo), neighbours in y and z lie in the
+// thread's own registers.  The kernel is bound by instruction issue, so each
+// central difference is formed once per node and used by the four faces that
+// average it, and the arithmetic is packed in pairs (one instruction rounds
+// two sums or products).  Measured at 257^3: 150 us; forming the 15
+// differences of a node's three faces from shared-memory planes took 512
+// instructions a node and 277 us.  Four rows a warp (fewer halo rows, 119
+// registers) took 206 us: too few warps to cover the latencies.
 
 // x = hi + lo exactly up to the 48th significant bit, both FP32, integer ops
-// only.  |x| < 2^-126 gives (0, 0); lo is dropped below |x| < 2^-74.
-__device__ __forceinline__ void split_hi_lo(double x, float& hi, float& lo)
+// only.  |x| < 2^-126 gives (0, 0); lo is dropped below |x| < 2^-74; beyond
+// FP32's range (and for infinities and NaNs) there is no split.
+__device__ __noinline__ float2 split_hi_lo_ends(double x)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 63) << 31;
     const int E = (int)((b >> 52) & 0x7ffu);
-    if (E < 897) {
-        hi = 0.0f;
-        lo = 0.0f;
-        return;
-    }
-    if (E > 1150) {  // beyond FP32 range (or inf/nan): no split
-        hi = __double2float_rn(x);
-        lo = 0.0f;
-        return;
-    }
-    const unsigned long long M = b & 0xFFFFFFFFFFFFFull;
-    hi = __uint_as_float(sign | ((unsigned)(E - 896) << 23) | (unsigned)(M >> 29));
-    if (E < 949) {
-        lo = 0.0f;
-        return;
-    }
-    const float r = __uint2float_rn((unsigned)(M & 0x1FFFFFFFull));  // < 2^29
-    lo = __uint_as_float(sign | __float_as_uint(r * __uint_as_float((unsigned)(E - 948) << 23)));
+    if (E < 897) return make_float2(0.0f, 0.0f);
+    if (E > 1150) return make_float2(__double2float_rn(x), 0.0f);
+    const unsigned long long M = b & 0xFFFFFFFFFFFFFull;  // 897 <= E < 949
+    return make_float2(__uint_as_float(sign | ((unsigned)(E - 896) << 23) | (unsigned)(M >> 29)), 0.0f);
+}
+
+// for 949 <= exponent field <= 1150 (the caller's check)
+__device__ __forceinline__ unsigned split_field(double x) { return (unsigned)__double2hiint(x) & 0x7ff00000u; }
+__device__ __forceinline__ float2 split_hi_lo(double x)
+{
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned ex = h & 0x7ff00000u, sign = h & 0x80000000u;
+    // exponent E and the fraction's top 23 bits, rebiased by E - 896 (modulo 2^9, the bits that a shift by three
+    // leaves); then the fraction's other 29 bits times 2^(E - 948 - 127)
+    const float hi = __uint_as_float(sign | ((__funnelshift_l(l, h, 3) - (896u << 23)) & 0x7fffffffu));
+    const float r = __uint2float_rn(l & 0x1FFFFFFFu);
+    return make_float2(hi, r * __uint_as_float(sign | (((ex << 3) - (948u << 23)) & 0x7fffffffu)));
 }
 
 // Exact FP32 -> FP64 with integer ops (subnormals flushed to zero).
 __device__ __forceinline__ double f32_to_f64(float f)
 {
     const unsigned u = __float_as_uint(f);
-    const unsigned long long sign = (unsigned long long)(u >> 31) << 63;
-    const unsigned e = (u >> 23) & 0xffu;
-    if (e == 0) return __longlong_as_double((long long)sign);
-    const unsigned long long ed = e == 255 ? 2047ull : (unsigned long long)(e + 896);
-    return __longlong_as_double((long long)(sign | (ed << 52) | ((unsigned long long)(u & 0x7fffffu) << 29)));
+    const unsigned sign = u & 0x80000000u, e = u & 0x7f800000u;
+    unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20), lo = u << 29;
+    if (e == 0u) hi = 0u, lo = 0u;
+    if (e == 0x7f800000u) hi += 896u << 20;  // exponent 255 to 2047
+    return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
-struct SrcPlanes {
-    float hi[3][kSrcPY][kSrcPX];
-    float lo[3][kSrcPY][kSrcPX];
+constexpr int kSrcX = 30;         // output columns of a warp: lanes 1 .. 30
+constexpr int kSrcY = 2;          // output rows of a warp
+constexpr int kSrcR = kSrcY + 2;  // rows held, with the halo
+constexpr int kSrcWarps = 4;      // warps of a CTA, along y
+constexpr int kSrcKC = 24;        // planes of a chunk
+
+// Differences of hi/lo pairs, both parts in one packed operation.
+__device__ __forceinline__ float pair_diff(float2 a, float2 b)
+{
+    const float2 d = __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+    return d.x + d.y;
+}
+
+// Fluxes (times h) through two faces, each from its node P to P + e_axis:
+// nu(|g|/a0) * (Phi(Q) - Phi(P)); |g| from the normal difference dn and the
+// means of the two nodes' transverse central differences (ta, tb their sums);
+// a face with g = 0 carries no flux.
+__device__ __forceinline__ float2 face_flux(float2 dn, float2 ta, float2 tb, float inv_h, float four_a0)
+{
+    const float q = 0.25f * inv_h;
+    const float2 gn = __fmul2_rn(dn, make_float2(inv_h, inv_h));
+    const float2 ga = __fmul2_rn(ta, make_float2(q, q)), gb = __fmul2_rn(tb, make_float2(q, q));
+    const float2 g2 = __ffma2_rn(gb, gb, __ffma2_rn(gn, gn, __fmul2_rn(ga, ga)));
+    const float2 y = __ffma2_rn(make_float2(four_a0, four_a0), make_float2(rsqrtf(g2.x), rsqrtf(g2.y)),
+                                make_float2(1.0f, 1.0f));
+    const float2 w = __fadd2_rn(make_float2(sqrtf(y.x), sqrtf(y.y)), make_float2(1.0f, 1.0f));
+    const float2 f = __fmul2_rn(__fmul2_rn(w, make_float2(0.5f, 0.5f)), dn);
+    return make_float2(g2.x > 0.0f ? f.x : 0.0f, g2.y > 0.0f ? f.y : 0.0f);
+}
+
+// One plane's part of the warp's columns: the values and the differences that
+// need no other plane.
+struct SrcPlane {
+    float2 v[kSrcR];
+    float cx[kSrcR];      // Phi(i+1) - Phi(i-1)
+    float2 cy;            // Phi(j+1) - Phi(j-1), rows 1, 2
+    float2 dx;            // Phi(i+1) - Phi(i), rows 1, 2
+    float dy[kSrcY + 1];  // Phi(j+1) - Phi(j), rows 0 .. 2
 };
 
-// Phi(a) - Phi(b) for smem positions (plane, y, x).
-#define SRC_D(pa, ya, xa, pb, yb, xb)                                                                                  \
-    ((S.hi[pa][ya][xa] - S.hi[pb][yb][xb]) + (S.lo[pa][ya][xa] - S.lo[pb][yb][xb]))
-
-// Flux (times h) through the face from node P to node P + e_axis:
-// nu(|g|/a0) * (Phi(Q) - Phi(P)); |g| from the normal difference and the
-// means of the two nodes' transverse central differences.
-__device__ __forceinline__ float face_flux(float dn, float ta, float tb, float inv_h, float four_a0)
+__device__ __forceinline__ void src_plane(const double (&v)[kSrcR], SrcPlane& p)
 {
-    const float gn = dn * inv_h;
-    const float q = 0.25f * inv_h;
-    const float g2 = gn * gn + (ta * q) * (ta * q) + (tb * q) * (tb * q);
-    if (!(g2 > 0.0f)) return 0.0f;
-    const float nu = 0.5f * (1.0f + sqrtf(1.0f + four_a0 * rsqrtf(g2)));
-    return nu * dn;
+    constexpr unsigned kAll = 0xffffffffu;
+    bool fast = true;
+#pragma unroll
+    for (int r = 0; r < kSrcR; ++r) {
+        fast = fast && split_field(v[r]) - (949u << 20) <= (1150u - 949u) << 20;
+        p.v[r] = split_hi_lo(v[r]);
+    }
+    if (!fast) {
+#pragma unroll
+        for (int r = 0; r < kSrcR; ++r)
+            if (split_field(v[r]) - (949u << 20) > (1150u - 949u) << 20) p.v[r] = split_hi_lo_ends(v[r]);
+    }
+    float dx[kSrcR];
+#pragma unroll
+    for (int r = 0; r < kSrcR; ++r) {
+        const float2 right = make_float2(__shfl_down_sync(kAll, p.v[r].x, 1), __shfl_down_sync(kAll, p.v[r].y, 1));
+        const float2 left = make_float2(__shfl_up_sync(kAll, p.v[r].x, 1), __shfl_up_sync(kAll, p.v[r].y, 1));
+        p.cx[r] = pair_diff(right, left);
+        dx[r] = pair_diff(right, p.v[r]);
+    }
+    p.dx = make_float2(dx[1], dx[2]);
+    p.cy = make_float2(pair_diff(p.v[2], p.v[0]), pair_diff(p.v[3], p.v[1]));
+#pragma unroll
+    for (int r = 0; r <= kSrcY; ++r) p.dy[r] = pair_diff(p.v[r + 1], p.v[r]);
 }
 
-// Face fluxes with P at smem position (plane p, y, x).  pm/pp: planes below/above p.
-__device__ __forceinline__ float flux_x(const SrcPlanes& S, int pm, int p, int pp, int y, int x, float ih, float fa)
+// fluxes through the faces between planes p and q = p + e_z of rows 1, 2
+__device__ __forceinline__ float2 src_flux_z(const SrcPlane& p, const SrcPlane& q, float ih, float fa)
 {
-    const float dn = SRC_D(p, y, x + 1, p, y, x);
-    const float ty = SRC_D(p, y + 1, x, p, y - 1, x) + SRC_D(p, y + 1, x + 1, p, y - 1, x + 1);
-    const float tz = SRC_D(pp, y, x, pm, y, x) + SRC_D(pp, y, x + 1, pm, y, x + 1);
-    return face_flux(dn, ty, tz, ih, fa);
-}
-__device__ __forceinline__ float flux_y(const SrcPlanes& S, int pm, int p, int pp, int y, int x, float ih, float fa)
-{
-    const float dn = SRC_D(p, y + 1, x, p, y, x);
-    const float tx = SRC_D(p, y, x + 1, p, y, x - 1) + SRC_D(p, y + 1, x + 1, p, y + 1, x - 1);
-    const float tz = SRC_D(pp, y, x, pm, y, x) + SRC_D(pp, y + 1, x, pm, y + 1, x);
-    return face_flux(dn, tx, tz, ih, fa);
-}
-// face between plane p (P) and plane pp (Q = P + e_z)
-__device__ __forceinline__ float flux_z(const SrcPlanes& S, int p, int pp, int y, int x, float ih, float fa)
-{
-    const float dn = SRC_D(pp, y, x, p, y, x);
-    const float tx = SRC_D(p, y, x + 1, p, y, x - 1) + SRC_D(pp, y, x + 1, pp, y, x - 1);
-    const float ty = SRC_D(p, y + 1, x, p, y - 1, x) + SRC_D(pp, y + 1, x, pp, y - 1, x);
-    return face_flux(dn, tx, ty, ih, fa);
+    const float2 dz = make_float2(pair_diff(q.v[1], p.v[1]), pair_diff(q.v[2], p.v[2]));
+    const float2 tx = __fadd2_rn(make_float2(p.cx[1], p.cx[2]), make_float2(q.cx[1], q.cx[2]));
+    return face_flux(dz, tx, __fadd2_rn(p.cy, q.cy), ih, fa);
 }
 
-__global__ void __launch_bounds__(kSrcTX * kSrcTY)
+__global__ void __launch_bounds__(32 * kSrcWarps)
 source_kernel(const double* __restrict__ phi, double* __restrict__ src, int n, float inv_h, float four_a0,
               float inv_h2, int zper)
 {
-    __shared__ SrcPlanes S;
-    __shared__ float Fx[kSrcTY][kSrcTX + 1];  // Fx[y][x + 1]: face (x, x+1), x = -1 .. 31
-    __shared__ float Fy[kSrcTY + 1][kSrcTX];  // Fy[y + 1][x]: face (y, y+1), y = -1 .. 7
+    constexpr unsigned kAll = 0xffffffffu;
     const int set = (int)gridDim.z == zper ? 0 : blockIdx.z / zper;  // blockIdx.z = zper * set + chunk
     const int kc = blockIdx.z - set * zper;
     phi += set * nat_elems(n);
     src += set * nat_elems(n);
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kSrcTX + tx;
-    const int i0 = blockIdx.x * kSrcTX, j0 = blockIdx.y * kSrcTY;
-    const int k0 = kc * kSrcKC;
-    const int k1 = min(k0 + kSrcKC, n + 1);
-    const long long P = n + 1;
-
-    // plane k of the tile (with halo) into slot `slot`; outside the grid -> 0
-    auto load_plane = [&](int k, int slot) {
-        for (int t = tid; t < kSrcPX * kSrcPY; t += kSrcTX * kSrcTY) {
-            const int lx = t % kSrcPX, ly = t / kSrcPX;
-            const int gi = i0 - 1 + lx, gj = j0 - 1 + ly;
-            float h = 0.0f, l = 0.0f;
-            if (k >= 0 && k <= n && gi >= 0 && gi <= n && gj >= 0 && gj <= n)
-                split_hi_lo(phi[gi + P * (gj + P * (long long)k)], h, l);
-            S.hi[slot][ly][lx] = h;
-            S.lo[slot][ly][lx] = l;
-        }
-    };
-
-    const int x = tx + 1, y = ty + 1;
-    const int i = i0 + tx, j = j0 + ty;
-    load_plane(k0 - 1, 0);
-    load_plane(k0, 1);
-    // the next plane's values are fetched into registers one plane ahead, so their loads are in flight
-    // while the current plane's fluxes are computed
-    constexpr int kEnt = (kSrcPX * kSrcPY + kSrcTX * kSrcTY - 1) / (kSrcTX * kSrcTY);  // 2
-    double pre[kEnt];
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kSrcX - 1 + lane;
+    const int j0 = (blockIdx.y * kSrcWarps + (threadIdx.x >> 5)) * kSrcY;  // output rows j0, j0 + 1
+    if (j0 > n) return;  // the whole warp
+    const int k0 = kc * kSrcKC, k1 = min(k0 + kSrcKC, n + 1);
+    const int P = n + 1;
+    const long long Q = (long long)P * P;
+    // rows j0 - 1 .. j0 + 2 of this lane's column; outside the grid the nearest node (it only feeds boundary
+    // nodes, whose source is 0)
+    int off[kSrcR];
+#pragma unroll
+    for (int r = 0; r < kSrcR; ++r) off[r] = min(max(i, 0), n) + P * min(max(j0 - 1 + r, 0), n);
+    double v[kSrcR];
     auto fetch = [&](int k) {
+        const double* at = phi + Q * min(max(k, 0), n);
 #pragma unroll
-        for (int q = 0; q < kEnt; ++q) {
-            const int t = tid + q * kSrcTX * kSrcTY;
-            const int lx = t % kSrcPX, ly = t / kSrcPX;
-            const int gi = i0 - 1 + lx, gj = j0 - 1 + ly;
-            pre[q] = (t < kSrcPX * kSrcPY && k >= 0 && k <= n && gi >= 0 && gi <= n && gj >= 0 && gj <= n)
-                         ? phi[gi + P * (gj + P * (long long)k)]
-                         : 0.0;
-        }
+        for (int r = 0; r < kSrcR; ++r) v[r] = at[off[r]];
     };
-    auto store = [&](int slot) {  // the fetched plane into a slot, split into hi/lo
+    const bool store = lane >= 1 && lane <= kSrcX && i <= n;
+    const bool inner0 = i > 0 && i < n && j0 > 0 && j0 < n, inner1 = i > 0 && i < n && j0 + 1 < n;
+    const bool store0 = store, store1 = store && j0 + 1 <= n;
+    float2 fzm;  // fluxes through the -z faces of plane k
+    // sources of plane k from planes m = k-1 and p = k; leaves plane k+1 in q and fetches plane k+2
+    auto step = [&](int k, const SrcPlane& m, const SrcPlane& p, SrcPlane& q) {
+        src_plane(v, q);
+        if (k + 1 < k1) fetch(k + 2);  // in flight while this plane's fluxes are computed
+        const float2 fz = src_flux_z(p, q, inv_h, four_a0);
+        float cz[kSrcR];
 #pragma unroll
-        for (int q = 0; q < kEnt; ++q) {
-            const int t = tid + q * kSrcTX * kSrcTY;
-            if (t >= kSrcPX * kSrcPY) continue;
-            const int lx = t % kSrcPX, ly = t / kSrcPX;
-            float h = 0.0f, l = 0.0f;
-            split_hi_lo(pre[q], h, l);  // zero -> (0, 0), as for nodes outside the grid
-            S.hi[slot][ly][lx] = h;
-            S.lo[slot][ly][lx] = l;
-        }
+        for (int r = 0; r < kSrcR; ++r) cz[r] = pair_diff(q.v[r], m.v[r]);
+        const float2 cz12 = make_float2(cz[1], cz[2]);
+        const float2 fy01 = face_flux(make_float2(p.dy[0], p.dy[1]),
+                                      __fadd2_rn(make_float2(p.cx[0], p.cx[1]), make_float2(p.cx[1], p.cx[2])),
+                                      __fadd2_rn(make_float2(cz[0], cz[1]), cz12), inv_h, four_a0);
+        const float2 fx = face_flux(
+            p.dx, __fadd2_rn(p.cy, make_float2(__shfl_down_sync(kAll, p.cy.x, 1), __shfl_down_sync(kAll, p.cy.y, 1))),
+            __fadd2_rn(cz12, make_float2(__shfl_down_sync(kAll, cz[1], 1), __shfl_down_sync(kAll, cz[2], 1))), inv_h,
+            four_a0);
+        const float2 fxm = make_float2(__shfl_up_sync(kAll, fx.x, 1), __shfl_up_sync(kAll, fx.y, 1));
+        const float fy2 = face_flux(make_float2(p.dy[2], 0.0f), make_float2(p.cx[2] + p.cx[3], 0.0f),
+                                    make_float2(cz[2] + cz[3], 0.0f), inv_h, four_a0).x;
+        const bool inner_k = k > 0 && k < n;
+        double* out = src + (Q * k + off[1]);
+        const float s0 = ((fx.x - fxm.x) + (fy01.y - fy01.x) + (fz.x - fzm.x)) * inv_h2;
+        const float s1 = ((fx.y - fxm.y) + (fy2 - fy01.y) + (fz.y - fzm.y)) * inv_h2;
+        if (store0) out[0] = inner0 && inner_k ? f32_to_f64(s0) : 0.0;
+        if (store1) out[P] = inner1 && inner_k ? f32_to_f64(s1) : 0.0;
+        fzm = fz;
     };
+    SrcPlane a, b, c;
+    fetch(k0 - 1);
+    src_plane(v, a);
+    fetch(k0);
+    src_plane(v, b);
+    fzm = src_flux_z(a, b, inv_h, four_a0);
     fetch(k0 + 1);
-    __syncthreads();
-    // flux through the -z face of plane k0 (between k0-1 and k0)
-    float fz_prev = flux_z(S, 0, 1, y, x, inv_h, four_a0);
-    int pm = 0, pc = 1, pp = 2;  // slots of planes k-1, k, k+1
     for (int k = k0; k < k1; ++k) {
-        __syncthreads();  // everyone is done with the slot about to be overwritten
-        store(pp);        // plane k + 1
-        if (k + 1 < k1) fetch(k + 2);
-        __syncthreads();
-        Fx[ty][tx + 1] = flux_x(S, pm, pc, pp, y, x, inv_h, four_a0);
-        if (tx == 0) Fx[ty][0] = flux_x(S, pm, pc, pp, y, x - 1, inv_h, four_a0);
-        Fy[ty + 1][tx] = flux_y(S, pm, pc, pp, y, x, inv_h, four_a0);
-        if (ty == 0) Fy[0][tx] = flux_y(S, pm, pc, pp, y - 1, x, inv_h, four_a0);
-        const float fz = flux_z(S, pc, pp, y, x, inv_h, four_a0);
-        __syncthreads();
-        if (i <= n && j <= n) {
-            const bool inner = i > 0 && i < n && j > 0 && j < n && k > 0 && k < n;
-            const float v = inner ? ((Fx[ty][tx + 1] - Fx[ty][tx]) + (Fy[ty + 1][tx] - Fy[ty][tx]) + (fz - fz_prev)) * inv_h2
-                                  : 0.0f;
-            src[i + P * (j + P * (long long)k)] = f32_to_f64(v);
-        }
-        fz_prev = fz;
-        const int t = pm;
-        pm = pc;
-        pc = pp;
-        pp = t;
+        step(k, a, b, c);
+        a = b;
+        b = c;
     }
 }
-#undef SRC_D
 
 // ---------------------------------------------------------------------------
 // Forces at points: finest box whose containing cell has 8 interior corners.
@@ -619,8 +633,8 @@ void launch_boundary_from_parent(const double* parent, double* u, int n, int rat
 void launch_source(const double* phi, double* src, int n, double h, double a0, cudaStream_t s, int nsets)
 {
     const unsigned zper = cdiv(n + 1, kSrcKC);
-    const dim3 grid(cdiv(n + 1, kSrcTX), cdiv(n + 1, kSrcTY), zper * (unsigned)nsets);
-    source_kernel<<<grid, dim3(kSrcTX, kSrcTY), 0, s>>>(phi, src, n, (float)(1.0 / h), (float)(4.0 * a0),
+    const dim3 grid(cdiv(n + 1, kSrcX), cdiv(n + 1, kSrcY * kSrcWarps), zper * (unsigned)nsets);
+    source_kernel<<<grid, 32 * kSrcWarps, 0, s>>>(phi, src, n, (float)(1.0 / h), (float)(4.0 * a0),
                                                         (float)(1.0 / (h * h)), (int)zper);
 }
 

@@ -65,3 +65,22 @@ def test_deposit_at_cell_edges_and_rounding_ties(q, ora, n, center):
     assert np.array_equal(got, want)
     assert np.array_equal(rho.cpu().numpy(), got * (2.0 ** -shift * (n / L0) ** 3))
     ctx.close()
+
+
+@pytest.mark.parametrize("n,sets", [(2, 1), (4, 3), (8, 1), (16, 2), (32, 1), (64, 2)])
+def test_source_on_partial_tiles(q, ora, n, sets):
+    # every position of the last column, row and plane within the tiles of 30 columns, 8 rows and 24 planes, several sets
+    L0, a0 = 3.0 * n, 3.6
+    rng = np.random.default_rng(n)
+    phi = rng.uniform(-1.0, 1.0, (sets, (n + 1) ** 3))
+    phi[0, :n] = 0.5  # equal neighbours: faces without a flux
+    ctx = q.Context(n=n, nboxes=1, L0=L0, a0=a0, nsets=sets)
+    src = torch.full((sets * (n + 1) ** 3,), 7.0, dtype=torch.float64, device="cuda")
+    ctx.qumond_source(0, to_dev(phi.reshape(-1)), src)
+    got = src.cpu().numpy().reshape(sets, -1)
+    h = L0 / n
+    # six fluxes of at most nu dPhi <= 2 + sqrt(2 a0 h), each with about ten FP32 roundings, over h^2
+    tol = 60 * 2.0 ** -24 * (2.0 + np.sqrt(2.0 * a0 * h)) / h ** 2
+    for s in range(sets):
+        assert np.max(np.abs(got[s] - ora.source(n, h, a0, phi[s]))) <= tol
+    ctx.close()
