@@ -19,6 +19,7 @@ struct Level {
     LevelView v;
     void* e = nullptr;  // iterate / correction, 2 colours
     void* f = nullptr;  // right-hand side, 2 colours
+    float* t = nullptr; // second array of the black colour (FP32 levels that whole sweeps cover)
     RbMaps maps;        // TMA descriptors of e (FP32 levels with n >= 64)
 };
 
@@ -105,6 +106,7 @@ struct qumond_ctx {
     int lc = 0;  // level handed to the coarse-grid kernel
     size_t elt = 4;
     std::vector<Level> lev;  // index l = 0..L; only l >= lc allocated
+    void* pool = nullptr;    // the levels' arrays
     double* partials = nullptr;
     int max_partials = 0;
     double* d_norms = nullptr;
@@ -325,6 +327,27 @@ void rb(qumond_ctx* c, int l, int colour, bool zero, double h, cudaStream_t s)
     });
 }
 
+// Whether level l's V-cycles on a zero-boundary problem run as whole sweeps:
+// the black values alternate between e and t, so both legs of the cycle take
+// an even number of sweeps (other counts go through the half-sweeps).
+inline bool whole_sweeps(const qumond_ctx* c, int l)
+{
+    return c->lev[l].t != nullptr && c->p.npre % 2 == 0 && c->p.npost % 2 == 0;  // each at least 2
+}
+
+// One red-black sweep in one pass; q: which of its leg (the even ones write t).
+void sweep(qumond_ctx* c, int l, SweepStart start, int q, bool red, double h, cudaStream_t s)
+{
+    const int n = c->lev[l].v.n;
+    count_cells(c, (long long)(n - 1) * (n - 1) * (n - 1));
+    const double words = 1.5 + (start == SweepStart::kZero ? 0.0 : 0.5) +
+                         (start == SweepStart::kCorrected ? 0.125 : 0.0) + (red ? 0.5 : 0.0);
+    run(c, l == c->L ? K_RB_FINEST : K_RB_COARSER, words * cube(n) * sizeof(float), s, [&] {
+        launch_sweep(E<float>(c, l), c->lev[l].t, F<float>(c, l), c->lev[l].v, start, q % 2 == 0, red,
+                     E<float>(c, l - 1), c->lev[l - 1].v, h, s, sets_of(c));
+    });
+}
+
 // The first pre-smoothing sweep of a correction that starts from zero, both
 // half-sweeps in one launch, on the FP32 levels whose black half-sweep has no
 // TMA form (the same bits as rb() for colour 0 from zero, then colour 1).
@@ -425,16 +448,24 @@ cudaError_t vsub(qumond_ctx* c, int box, bool zero_top, cudaStream_t s)
     return err;
 }
 
-// One V-cycle at level l on the correction problem held in lev[l] (for l <
-// L the initial guess is zero; at l = L the caller says so).
+// One V-cycle at level l on the problem held in lev[l] (for l < L the initial
+// guess is zero; at l = L the caller says so).  bnd: e may hold boundary values
+// other than zero (FMG).  red: the red values of the result are needed (by a
+// finer level's correction, or the caller), not only the black ones, from which
+// a further V-cycle starts.
 template <typename T>
-cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, cudaStream_t s)
+cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, bool bnd, bool red, cudaStream_t s)
 {
     const qumond_params& p = c->p;
     const double h = level_h(c, box, l);
     if (l <= c->lc) return coarse<T>(c, box, 0, nullptr, s);
     if (l == c->vtop) return vsub<T>(c, box, zero_guess, s);
+    const bool whole = !bnd && whole_sweeps(c, l);
     for (int q = 0; q < p.npre; ++q) {
+        if (whole) {
+            sweep(c, l, zero_guess && q == 0 ? SweepStart::kZero : SweepStart::kBlack, q, q == p.npre - 1, h, s);
+            continue;
+        }
         if (zero_guess && q == 0 && rb_first<T>(c, l, h, s)) continue;
         rb<T>(c, l, 0, zero_guess && q == 0, h, s);
         rb<T>(c, l, 1, false, h, s);
@@ -448,10 +479,14 @@ cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, cudaStream_t 
             launch_restrict_resid_red<T>(E<T>(c, l), F<T>(c, l), c->lev[l].v, F<T>(c, l - 1), c->lev[l - 1].v, h, s,
                                          sets_of(c));
     });
-    cudaError_t err = vcycle<T>(c, box, l - 1, true, s);
+    cudaError_t err = vcycle<T>(c, box, l - 1, true, false, true, s);
     if (err != cudaSuccess) return err;
-    prolong<T>(c, l, true, s);
+    if (!whole) prolong<T>(c, l, true, s);
     for (int q = 0; q < p.npost; ++q) {
+        if (whole) {
+            sweep(c, l, q == 0 ? SweepStart::kCorrected : SweepStart::kBlack, q, red && q == p.npost - 1, h, s);
+            continue;
+        }
         rb<T>(c, l, 0, false, h, s);
         rb<T>(c, l, 1, false, h, s);
     }
@@ -476,12 +511,13 @@ cudaError_t fmg(qumond_ctx* c, int box, const double* u64, cudaStream_t s)
     }
     cudaError_t err = coarse<T>(c, box, 1, u64, s);
     if (err != cudaSuccess) return err;
+    const bool bnd = box > 0 || p.bc_mode != QUMOND_BC_ZERO;
     for (int l = c->lc + 1; l <= c->L; ++l) {
         set_bnd<T>(c, l, u64, s);
         prolong<T>(c, l, false, s);
         set_bnd<T>(c, l - 1, nullptr, s);
         for (int q = 0; q < p.ncycle; ++q) {
-            err = vcycle<T>(c, box, l, false, s);
+            err = vcycle<T>(c, box, l, false, bnd, q == p.ncycle - 1, s);
             if (err != cudaSuccess) return err;
         }
     }
@@ -582,7 +618,7 @@ cudaError_t enqueue_body(qumond_ctx* c, int box, const double* rhs, double coef,
         ~BodyFlag() { c->in_body = false; }
     } body_flag(c);
     for (int q = 0; q < c->p.dc_vcycles; ++q) {  // the first from e = 0, the others continue it
-        cudaError_t err = vcycle<T>(c, box, c->L, q == 0, s);
+        cudaError_t err = vcycle<T>(c, box, c->L, q == 0, false, q == c->p.dc_vcycles - 1, s);
         if (err != cudaSuccess) return err;
     }
     if (fixed_mode(c)) {
@@ -916,19 +952,32 @@ qumond_status qumond_create(const qumond_params* p, qumond_ctx** out)
     while ((2 << lc) < kCoarseN && lc < L) ++lc;
     c->lc = lc;
     c->lev.resize(L + 1);
+    // every level's arrays in one zeroed allocation, each on a 256-byte boundary
     bool ok = true;
-    for (int l = 0; l <= L; ++l) {
-        c->lev[l].v = make_view(2 << l);
-        if (l < lc) continue;
-        const size_t bytes = (size_t)(2 * c->lev[l].v.cs) * c->elt * ns;
-        if (cudaMalloc(&c->lev[l].e, bytes) != cudaSuccess || cudaMalloc(&c->lev[l].f, bytes) != cudaSuccess) {
-            ok = false;
-            break;
+    auto place = [&](unsigned char* base) {
+        size_t used = 0;
+        auto take = [&](size_t bytes) {
+            unsigned char* at = base ? base + used : nullptr;
+            used += (bytes + 255) & ~(size_t)255;
+            return at;
+        };
+        for (int l = lc; l <= L; ++l) {
+            Level& lv = c->lev[l];
+            const size_t bytes = (size_t)(2 * lv.v.cs) * c->elt * ns;
+            lv.e = take(bytes);
+            lv.f = take(bytes);
+            if (c->elt == sizeof(float) && l > lc && sweep_level(lv.v.n))
+                lv.t = reinterpret_cast<float*>(take(bytes / 2));
         }
-        if (cudaMemset(c->lev[l].e, 0, bytes) != cudaSuccess || cudaMemset(c->lev[l].f, 0, bytes) != cudaSuccess) {
-            ok = false;
-            break;
-        }
+        return used;
+    };
+    for (int l = 0; l <= L; ++l) c->lev[l].v = make_view(2 << l);
+    const size_t pool = place(nullptr);
+    ok = cudaMalloc(&c->pool, pool) == cudaSuccess && cudaMemset(c->pool, 0, pool) == cudaSuccess;
+    if (ok) {
+        place(static_cast<unsigned char*>(c->pool));
+        for (int l = lc; l <= L; ++l)
+            if (c->lev[l].t && prepare_sweep_level(c->lev[l].v.n) != cudaSuccess) ok = false;
     }
     if (ok) {
         const int nrows = residual_rows_blocks(p->n > 2 ? p->n : 2);
@@ -1024,10 +1073,7 @@ void qumond_destroy(qumond_ctx* c)
 {
     if (!c) return;
     cudaDeviceSynchronize();
-    for (auto& l : c->lev) {
-        if (l.e) cudaFree(l.e);
-        if (l.f) cudaFree(l.f);
-    }
+    if (c->pool) cudaFree(c->pool);
     if (c->partials) cudaFree(c->partials);
     if (c->d_norms) cudaFree(c->d_norms);
     if (c->h_norms) cudaFreeHost(c->h_norms);

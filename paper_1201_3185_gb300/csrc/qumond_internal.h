@@ -138,6 +138,18 @@ void launch_decide(const double* partials, int nblocks, SolveState* st, double t
                    bool refine, const cudaGraphConditionalHandle* handle, int* fault, cudaStream_t s,
                    const Sets& sets = Sets());
 
+// --- whole sweeps in one pass on FP32 levels with zero boundary values (sweep.cu) ---
+// What a sweep starts from: the black values as they are, zero, or the black values plus the correction
+// interpolated from the next coarser level.
+enum class SweepStart { kBlack = 0, kZero = 1, kCorrected = 2 };
+bool sweep_level(int n);  // levels the kernels cover
+// One red-black sweep of a level: black values from e (to_t) or from t into the other of the two; red (kBlack only):
+// the red values are written to e too.  t holds one colour array per set (v.cs entries), zero off the interior.  Zero
+// boundary values in e, t and ec.  The same bits as launch_prolong_black (add) and two launch_rb_half.
+void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepStart start, bool to_t, bool red,
+                  const float* ec, const LevelView& vc, double h, cudaStream_t s, const Sets& sets = Sets());
+cudaError_t prepare_sweep_level(int n);  // kernel attributes, before any launch or capture
+
 // --- TMA-staged half-sweep for FP32 levels with n >= 64 (rb_tma.cu) ----------
 struct RbMaps {
     CUtensorMap map[2];   // colour c of the iterate as a 3-D tensor (m, j, k), tile + halo boxes

@@ -84,3 +84,43 @@ def test_source_on_partial_tiles(q, ora, n, sets):
     for s in range(sets):
         assert np.max(np.abs(got[s] - ora.source(n, h, a0, phi[s]))) <= tol
     ctx.close()
+
+
+def _mond(q, src, phi0, n, box, **kw):
+    ctx = q.Context(n=n, nboxes=box + 1, L0=64.0, precision=q.QUMOND_PREC_MIXED, **kw)
+    phi = phi0.clone()
+    ctx.qumond_solve_mond(box, src, None, phi)
+    ctx.close()
+    return phi
+
+
+@pytest.mark.parametrize("n,sets,ncycle", [(64, 1, 2), (64, 5, 1), (128, 1, 1), (128, 3, 2), (256, 1, 1), (256, 2, 1),
+                                           (512, 1, 1)])
+def test_whole_sweeps_give_the_bits_of_the_half_sweeps(q, n, sets, ncycle):
+    # full multigrid without a tolerance: with zero boundary values by bc_mode ZERO each level's V-cycles run as whole
+    # sweeps, with zeros given by the caller (GIVEN) as half-sweeps, restriction and prolongation of their own
+    g = torch.Generator(device="cuda").manual_seed(n + sets)
+    src = torch.rand(sets * (n + 1) ** 3, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    phi0 = torch.zeros_like(src)
+    kw = dict(ncycle=ncycle, nsets=sets)
+    a = _mond(q, src, phi0, n, 0, bc_mode=q.QUMOND_BC_ZERO, **kw)
+    b = _mond(q, src, phi0, n, 0, bc_mode=q.QUMOND_BC_GIVEN, **kw)
+    assert torch.equal(a, b)
+    if sets > 1:  # and those of the last set alone
+        k = (sets - 1) * (n + 1) ** 3
+        c = _mond(q, src[k:].clone(), phi0[k:].clone(), n, 0, bc_mode=q.QUMOND_BC_ZERO, ncycle=ncycle)
+        assert torch.equal(a[k:], c)
+
+
+def test_whole_sweeps_give_the_bits_of_the_solve_without_allocation(q):
+    # that solve runs half-sweeps on every level: the corrections that start from zero are among them here
+    n = 64
+    g = torch.Generator(device="cuda").manual_seed(3)
+    src = torch.rand((n + 1) ** 3, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    phi0 = torch.zeros_like(src)
+    kw = dict(ncycle=1, rel_tol=1e-9, max_vcycles=40, dc_vcycles=3)
+    a = _mond(q, src, phi0, n, 0, **kw)
+    b = phi0.clone()
+    q.qumond.qumond_solve_mond_noalloc(
+        q.default_params(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, **kw), 0, src, None, b)
+    assert torch.equal(a, b)
