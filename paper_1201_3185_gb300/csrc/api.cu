@@ -336,15 +336,16 @@ inline bool whole_sweeps(const qumond_ctx* c, int l)
 }
 
 // One red-black sweep in one pass; q: which of its leg (the even ones write t).
-void sweep(qumond_ctx* c, int l, SweepStart start, int q, bool red, double h, cudaStream_t s)
+void sweep(qumond_ctx* c, int l, SweepStart start, int q, SweepAfter after, double h, cudaStream_t s)
 {
     const int n = c->lev[l].v.n;
     count_cells(c, (long long)(n - 1) * (n - 1) * (n - 1));
     const double words = 1.5 + (start == SweepStart::kZero ? 0.0 : 0.5) +
-                         (start == SweepStart::kCorrected ? 0.125 : 0.0) + (red ? 0.5 : 0.0);
+                         (start == SweepStart::kCorrected ? 0.125 : 0.0) +
+                         (after == SweepAfter::kRed ? 0.5 : after == SweepAfter::kRestrict ? 0.125 : 0.0);
     run(c, l == c->L ? K_RB_FINEST : K_RB_COARSER, words * cube(n) * sizeof(float), s, [&] {
-        launch_sweep(E<float>(c, l), c->lev[l].t, F<float>(c, l), c->lev[l].v, start, q % 2 == 0, red,
-                     E<float>(c, l - 1), c->lev[l - 1].v, h, s, sets_of(c));
+        launch_sweep(E<float>(c, l), c->lev[l].t, F<float>(c, l), c->lev[l].v, start, q % 2 == 0, after,
+                     E<float>(c, l - 1), F<float>(c, l - 1), c->lev[l - 1].v, h, s, sets_of(c));
     });
 }
 
@@ -463,7 +464,8 @@ cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, bool bnd, boo
     const bool whole = !bnd && whole_sweeps(c, l);
     for (int q = 0; q < p.npre; ++q) {
         if (whole) {
-            sweep(c, l, zero_guess && q == 0 ? SweepStart::kZero : SweepStart::kBlack, q, q == p.npre - 1, h, s);
+            sweep(c, l, zero_guess && q == 0 ? SweepStart::kZero : SweepStart::kBlack, q,
+                  q == p.npre - 1 ? SweepAfter::kRestrict : SweepAfter::kNothing, h, s);
             continue;
         }
         if (zero_guess && q == 0 && rb_first<T>(c, l, h, s)) continue;
@@ -471,7 +473,7 @@ cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, bool bnd, boo
         rb<T>(c, l, 1, false, h, s);
     }
     const double nodes = cube(c->lev[l].v.n);
-    run(c, K_RESTRICT_RESID, (1.5 + 0.125) * nodes * sizeof(T), s, [&] {
+    if (!whole) run(c, K_RESTRICT_RESID, (1.5 + 0.125) * nodes * sizeof(T), s, [&] {
         if (sizeof(T) == sizeof(float) && c->lev[l].maps.ok)
             launch_restrict_tma(reinterpret_cast<float*>(F<T>(c, l - 1)), c->lev[l].v, c->lev[l - 1].v, c->lev[l].maps,
                                 h, c->fault, s, sets_of(c));
@@ -484,7 +486,8 @@ cudaError_t vcycle(qumond_ctx* c, int box, int l, bool zero_guess, bool bnd, boo
     if (!whole) prolong<T>(c, l, true, s);
     for (int q = 0; q < p.npost; ++q) {
         if (whole) {
-            sweep(c, l, q == 0 ? SweepStart::kCorrected : SweepStart::kBlack, q, red && q == p.npost - 1, h, s);
+            sweep(c, l, q == 0 ? SweepStart::kCorrected : SweepStart::kBlack, q,
+                  red && q == p.npost - 1 ? SweepAfter::kRed : SweepAfter::kNothing, h, s);
             continue;
         }
         rb<T>(c, l, 0, false, h, s);

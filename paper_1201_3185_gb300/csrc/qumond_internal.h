@@ -142,12 +142,15 @@ void launch_decide(const double* partials, int nblocks, SolveState* st, double t
 // What a sweep starts from: the black values as they are, zero, or the black values plus the correction
 // interpolated from the next coarser level.
 enum class SweepStart { kBlack = 0, kZero = 1, kCorrected = 2 };
+// What it leaves beside the black values (other than nothing only from kBlack): the red values in e, or the full
+// weighting of the red residuals in the coarser level's right-hand side fc.
+enum class SweepAfter { kNothing = 0, kRed = 1, kRestrict = 2 };
 bool sweep_level(int n);  // levels the kernels cover
-// One red-black sweep of a level: black values from e (to_t) or from t into the other of the two; red (kBlack only):
-// the red values are written to e too.  t holds one colour array per set (v.cs entries), zero off the interior.  Zero
-// boundary values in e, t and ec.  The same bits as launch_prolong_black (add) and two launch_rb_half.
-void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepStart start, bool to_t, bool red,
-                  const float* ec, const LevelView& vc, double h, cudaStream_t s, const Sets& sets = Sets());
+// One red-black sweep of a level: black values from e (to_t) or from t into the other of the two.  t holds one
+// colour array per set (v.cs entries), zero off the interior.  Zero boundary values in e, t and ec.  The same bits as
+// launch_prolong_black (add), two launch_rb_half and launch_restrict_resid_red.
+void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepStart start, bool to_t, SweepAfter after,
+                  const float* ec, float* fc, const LevelView& vc, double h, cudaStream_t s, const Sets& sets = Sets());
 cudaError_t prepare_sweep_level(int n);  // kernel attributes, before any launch or capture
 
 // --- TMA-staged half-sweep for FP32 levels with n >= 64 (rb_tma.cu) ----------

@@ -9,13 +9,17 @@
 // node (each reads the other colour and f and writes its own); this pass moves
 // 8 (b 2, f 4, b' 2), 6 from a zero start, and costs one launch.  b' goes to
 // another array, since neighbouring blocks still read b around their tiles;
-// the two change roles from sweep to sweep.  The red values are written (2
-// more) only where something reads them: before the restriction of the
-// residual and after the last sweep.  With PROLONG the sweep starts from
-// b + P e_c, the coarse-grid correction applied as the planes are loaded.
+// the two change roles from sweep to sweep.  With kProlong the sweep starts from
+// b + P e_c, the coarse-grid correction applied as the planes arrive; with
+// kRestrict the residual of the red nodes (the black ones' vanishes) is formed
+// from b' and the red values a plane later and weighted into the coarser
+// level's right-hand side (0.5 bytes more, where the restriction on its own
+// reads 6 bytes again and needs the red values in memory); with kRed, the last
+// sweep, the red values are written (2 more).
 //
-// Every node's arithmetic is rb_half4_kernel's (and prolong_black4_kernel's),
-// in the same order, so the values are the same bits.
+// Every node's arithmetic is that of rb_half4_kernel, prolong_black4_kernel and
+// restrict_resid4_kernel, in the same order (in pairs: one instruction rounds
+// two sums as two would), so the values are the same bits.
 //
 // Layout: a thread owns four consecutive entries of two rows (j, j+1) of the
 // colour-split level and walks k.  Up to n = 256 the LPR = n/8 threads of a row
@@ -32,11 +36,17 @@
 // read): with one plane ahead in registers, half the bytes were in flight and
 // a sweep of 257^3 took 36 us.
 //
-// Measured at 257^3 (two launches of the half-sweeps, with the prolongation
-// where there is one, before): plain 25.7 us (36.2), with the red values written
-// 31.7, from zero 16.8 (29.3), corrected 29.2 (52.9).  513^3: 211 (248), 145
-// (213), 247 (354).  Eight sets of 129^3: 27 (41), 18 (32), 31 (56).  The
-// memory system bounds them (8 bytes a node in 25.7 us: 5.3 TB/s).
+// The residual and its restriction follow two and three planes behind, so such
+// a tile loses four rows on each side and holds 24 of them (registers, shared
+// memory).
+//
+// Measured at 257^3 (in brackets the launches replaced): from zero 16.7 us
+// (29.4), plain 25.1 (36.3), with the restriction 39.2 (66.5), corrected 28.6
+// (52.6), with the red values 30.4 (36.3): a V(2,2) leg pair 110 us (185).
+// 513^3: 157 (213), 205 (248), 342 (466), 235 (354), 268 (248).  Eight sets of
+// 129^3: 19 (32), 27 (41), 38 (71), 31 (56), 34 (41).  The plain sweep moves its
+// 8 bytes a node at 5.4 TB/s; the one with the restriction is bound by its
+// instructions, 12 warps an SM.
 #include "qumond_internal.h"
 
 #include <type_traits>
@@ -55,8 +65,9 @@ struct SweepArgs {
     float* red;        // red values after (or null); set s at + s * 2 cs
     const float* f;    // both colours
     const float* ec;   // coarser level, both colours (kProlong)
+    float* fc;         // right-hand side of the coarser level, both colours (kRestrict)
     LevelView v, vc;
-    float h2, sixth;
+    float h2, sixth, ih2;
     int tiles;         // tiles along j
     int chunk;         // planes of a chunk (even)
     const SolveState* act;
@@ -64,46 +75,104 @@ struct SweepArgs {
 
 __device__ __forceinline__ float4 zero4() { return make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
 
-// (sum of the six neighbours - h2 f) / 6 for four entries of a row with parity P of i: v the row itself in the
-// other colour, nb its entry past the end on the side that P needs, y and z pairs of neighbours.
-template <int P>
-__device__ __forceinline__ float4 relax4(const float4& v, float nb, const float4& y0, const float4& y1,
-                                         const float4& z0, const float4& z1, const float4& f, float h2, float sixth)
+__device__ __forceinline__ float2 two(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 lo(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi(const float4& v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 join(float2 l, float2 h) { return make_float4(l.x, l.y, h.x, h.y); }
+// four sums, or four a b + c, in two instructions that round each as the scalar ones do
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b)
 {
-    const float o0 = P ? v.y : nb, o1 = P ? v.z : v.x, o2 = P ? v.w : v.y, o3 = P ? nb : v.z;
-    const float s0 = (v.x + o0) + (y0.x + y1.x) + (z0.x + z1.x);
-    const float s1 = (v.y + o1) + (y0.y + y1.y) + (z0.y + z1.y);
-    const float s2 = (v.z + o2) + (y0.z + y1.z) + (z0.z + z1.z);
-    const float s3 = (v.w + o3) + (y0.w + y1.w) + (z0.w + z1.w);
-    return make_float4((s0 - h2 * f.x) * sixth, (s1 - h2 * f.y) * sixth, (s2 - h2 * f.z) * sixth,
-                       (s3 - h2 * f.w) * sixth);
+    return join(__fadd2_rn(lo(a), lo(b)), __fadd2_rn(hi(a), hi(b)));
+}
+__device__ __forceinline__ float4 fma4(const float4& a, float b, const float4& c)
+{
+    return join(__ffma2_rn(lo(a), two(b), lo(c)), __ffma2_rn(hi(a), two(b), hi(c)));
+}
+__device__ __forceinline__ float4 mul4(const float4& a, float b)
+{
+    return join(__fmul2_rn(lo(a), two(b)), __fmul2_rn(hi(a), two(b)));
 }
 
+// The sum of the six neighbours of four entries of a row with parity P of i: v the row itself in the other colour, nb
+// its entry past the end on the side that P needs, y and z pairs of neighbours.
+template <int P>
+__device__ __forceinline__ float4 sum6(const float4& v, float nb, const float4& y0, const float4& y1, const float4& z0,
+                                       const float4& z1)
+{
+    const float4 x = make_float4(v.x + (P ? v.y : nb), v.y + (P ? v.z : v.x), v.z + (P ? v.w : v.y),
+                                 v.w + (P ? nb : v.z));
+    return add4(add4(x, add4(y0, y1)), add4(z0, z1));
+}
+
+// (sum - h2 f) / 6, and the residual f - (sum - 6 e) / h2
+__device__ __forceinline__ float4 relax4(const float4& sum, const float4& f, float h2, float sixth)
+{
+    return mul4(fma4(f, -h2, sum), sixth);
+}
+__device__ __forceinline__ float4 resid4(const float4& sum, const float4& e, const float4& f, float ih2)
+{
+    return fma4(fma4(e, -6.0f, sum), -ih2, f);
+}
+
+constexpr int kThreads = 512, kThreadsRed = 384, kThreadsRestrict = 384, kThreadsSmall = 128;
 constexpr int kAhead = 2;               // planes in flight
-constexpr int kRingB = kAhead + 2, kRingF = kAhead + 1;
+constexpr int kRingB = kAhead + 2;      // planes of b in shared memory
+// What a sweep leaves beside the black values: nothing, the red values, or the residual's restriction.
+constexpr int kNothing = (int)SweepAfter::kNothing, kRed = (int)SweepAfter::kRed,
+              kRestrict = (int)SweepAfter::kRestrict;
 static_assert((kRingB & (kRingB - 1)) == 0, "a plane's place in the ring of b is a mask of its index");
 constexpr int kWide = 34;               // threads of a row of a tile above n = 256: 32 groups and one on each side
 
-// planes of a tile in shared memory: rings of b and of both colours of f, two planes of red values
-template <int MODE>
-constexpr int smem_planes() { return (MODE == kZero ? 0 : kRingB) + 2 * kRingF + 2; }
+// Planes of red f in shared memory (the residual of plane k-2 needs f again), of black f, and of all that a tile
+// holds there: the rings of b and f, two planes of red values, and for the residual two of the new black values and
+// two of residuals (of the odd rows; of both where rows straddle warps).
+template <int AFTER>
+constexpr int ring_fr() { return kAhead + 1 + (AFTER == kRestrict ? 2 : 0); }
+constexpr int kRingFb = kAhead + 1;
+template <int LPR, int MODE, int AFTER>
+constexpr int smem_planes()
+{
+    return (MODE == kZero ? 0 : kRingB) + ring_fr<AFTER>() + kRingFb + 2 +
+           (AFTER == kRestrict ? 2 + (LPR == kWide ? 2 : 1) : 0);
+}
+// The most threads of a CTA.  The residual takes about 150 registers (12 warps: with 13 an SM's quarter holds four
+// warps of at most 128); sweeps that write both colours, and the tiles along rows,
+// measured faster with fewer warps (257^3 with the red values: 30.4 us, 32.1 with 512 threads; 513^3 plain: 206, 225).
+template <int LPR, int MODE, int AFTER>
+constexpr int most_threads()
+{
+    return AFTER == kRestrict ? kThreadsRestrict
+           : AFTER == kRed || (LPR == kWide && MODE != kProlong) ? kThreadsRed : kThreads;
+}
+constexpr int kSmem = 227 * 1024;  // shared memory of an SM
+// Row pairs of the largest tile.
+template <int LPR, int MODE, int AFTER>
+constexpr int most_pairs()
+{
+    constexpr int fit = kSmem / (smem_planes<LPR, MODE, AFTER>() * 2 * LPR * 16);
+    constexpr int w = most_threads<LPR, MODE, AFTER>() / LPR;
+    return fit < w ? fit : w;
+}
+template <int AFTER>
+constexpr int halo_pairs() { return AFTER == kRestrict ? 2 : 1; }  // row pairs on each side that are no output
 
-__device__ __forceinline__ void copy16(float4* dst, const float* src, bool valid)
+// bytes: 16, or 0: the 16 bytes are filled with zeros, nothing is read
+__device__ __forceinline__ void copy16(float4* dst, const float* src, int bytes)
 {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const int bytes = valid ? 16 : 0;  // 0: the 16 bytes are filled with zeros, nothing is read
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
 }
 
-template <int LPR, int MODE, bool RED>
-__global__ void __launch_bounds__(512)
+template <int LPR, int MODE, int AFTER>
+__global__ void __launch_bounds__(most_threads<LPR, MODE, AFTER>())
 sweep_kernel(const SweepArgs a)
 {
     extern __shared__ __align__(16) float4 sm[];
-    constexpr bool kTiledX = LPR == kWide;
+    constexpr bool kTiledX = LPR == kWide, RED = AFTER == kRed, RES = AFTER == kRestrict;
+    constexpr int kRingFr = ring_fr<AFTER>(), HP = halo_pairs<AFTER>();
     const int set = blockIdx.y;
     if (a.act && !a.act[set].cont) return;  // this set's correction has stopped (the whole CTA)
-    const int n = a.v.n;
+    const int n = kTiledX ? a.v.n : 8 * LPR;
     const int W = (int)blockDim.x / LPR;          // row pairs of the tile
     const int x = (int)threadIdx.x % LPR;
     const int w = (int)threadIdx.x / LPR;
@@ -112,14 +181,16 @@ sweep_kernel(const SweepArgs a)
     const int gx = kTiledX ? 32 * (int)blockIdx.z + x - 1 : x;  // entries 4 gx .. 4 gx + 3
     const bool gin = !kTiledX || (gx >= 0 && gx < (n >> 3));
     const bool gout = !kTiledX || (x >= 1 && x <= 32);
-    const int j0 = 1 + ty * (2 * W - 4);          // first output row (odd)
+    const int j0 = 1 + ty * (2 * W - 4 * HP);     // first output row (odd)
     const int kb = 1 + tz * a.chunk;              // first output plane (odd)
     const int ke = min(kb + a.chunk, n);
-    const int ja = j0 - 2 + 2 * w;                // this thread's rows ja (odd) and ja + 1
+    const int klast = RES ? ke + 3 : ke;          // the last step
+    const int ja = j0 - 2 * HP + 2 * w;           // this thread's rows ja (odd) and ja + 1
     const bool in0 = gin && ja >= 1 && ja < n, in1 = gin && ja + 1 >= 1 && ja + 1 < n;  // interior rows
-    const bool pair_out = w >= 1 && w < W - 1;
+    const bool all_in = !kTiledX && j0 - 2 * HP >= 1 && j0 - 2 * HP + 2 * W <= n;  // every row of the tile
+    const bool pair_out = w >= HP && w < W - HP;
     const bool out0 = gout && pair_out && in0, out1 = gout && pair_out && in1;
-    const int M = a.v.M;
+    const int M = kTiledX ? a.v.M : 4 * LPR + 4;
     const long long Q = (long long)M * (n + 1);
     const long long row0 = (long long)ja * M + 4 * gx;  // first entry in row ja of plane 0 of a colour
     const float* const b = MODE == kZero ? nullptr : a.b + set * a.bset + row0;
@@ -131,30 +202,48 @@ sweep_kernel(const SweepArgs a)
     const int at0 = 2 * w * LPR + x;  // row ja of a plane in shared memory; row ja + 1 is LPR further
     float4* const sB = sm + at0;
     float4* const sFr = sm + (MODE == kZero ? 0 : kRingB) * plane4 + at0;
-    float4* const sFb = sFr + kRingF * plane4;
-    float4* const sR = sFb + kRingF * plane4;
+    float4* const sFb = sFr + kRingFr * plane4;
+    float4* const sR = sFb + kRingFb * plane4;
+    float4* const sN = sR + 2 * plane4;  // the new black values, two planes (RES)
+    // residuals, two planes: of row ja (RES), and row ja + 1 beside it where the shuffles need it
+    constexpr int kResRow = kTiledX ? 2 * LPR : LPR;
+    float4* const sE = sN + 2 * plane4 - at0 + w * kResRow + x;
+    const int res4 = W * kResRow;
     const bool up = w > 0, dn = w < W - 1;
 
-    // the asynchronous copies of step k: b(k+1), red f(k), black f(k-1), of the rows that use them; `fslot`: k's place
-    // in the rings of f
-    auto fetch = [&](int k, int fslot) {
+    // The asynchronous copies of step k: b(k+1), red f(k), black f(k-1), of the rows that use them; rslot, bslot: the
+    // places of f's planes in their rings.  A row outside the level reads nothing (zeros), through a pointer that stays
+    // inside f.  The addresses run along with k where registers are free, and are formed from k where they are not
+    // (kProlong of 257^3: 28.6 us, 33.0 with running ones; kZero 16.6 and 18.3).
+    constexpr bool kRun = MODE == kZero || RES;
+    const int ks = kb - (RES ? 3 : 1);  // the first step (even)
+    const float* pb0 = in0 && MODE != kZero ? b : a.f;
+    const float* pb1 = in1 && MODE != kZero ? b + M : a.f;
+    const float* pr = fr;
+    const float* pk = fb;
+    if (kRun) pb0 += Q * (ks + 1), pb1 += Q * (ks + 1), pr += Q * ks, pk += Q * (ks - 1);
+    const int bytes0 = in0 ? 16 : 0, bytes1 = in1 ? 16 : 0;
+    const bool fr0 = in0 && up, fr1 = in1 && dn;
+    const bool fb0 = RES ? in0 && up && dn : out0, fb1 = RES ? in1 && up && dn : out1;
+    auto fetch = [&](int k, int rslot, int bslot) {
         if (MODE != kZero) {
-            const bool kin = k + 1 >= 1 && k + 1 < n && k + 1 <= ke + 1;
             float4* d = sB + ((k + 1) & (kRingB - 1)) * plane4;
-            const float* at = b + Q * (k + 1);
-            copy16(d, kin && in0 ? at : a.f, kin && in0);
-            copy16(d + LPR, kin && in1 ? at + M : a.f, kin && in1);
+            const bool kin = k + 1 >= 0 && k + 1 <= n && k <= klast;
+            const long long o = kRun ? 0 : Q * (k + 1);
+            copy16(d, kin ? pb0 + o : a.f, kin ? bytes0 : 0);
+            copy16(d + LPR, kin ? pb1 + o : a.f, kin ? bytes1 : 0);
         }
-        if (k >= 1 && k < n && k <= ke) {
-            const float* at = fr + Q * k;
-            if (in0 && up) copy16(sFr + fslot * plane4, at, true);
-            if (in1 && dn) copy16(sFr + fslot * plane4 + LPR, at + M, true);
+        if (k >= 0 && k <= n && k <= klast) {
+            const float* at = pr + (kRun ? 0 : Q * k);
+            if (fr0) copy16(sFr + rslot * plane4, at, 16);
+            if (fr1) copy16(sFr + rslot * plane4 + LPR, at + M, 16);
         }
-        if (k - 1 >= kb && k - 1 < ke) {
-            const float* at = fb + Q * (k - 1);
-            if (out0) copy16(sFb + fslot * plane4, at, true);
-            if (out1) copy16(sFb + fslot * plane4 + LPR, at + M, true);
+        if (k > kb - (RES ? 1 : 0) && k <= n + 1 && k <= klast) {
+            const float* at = pk + (kRun ? 0 : Q * (k - 1));
+            if (fb0) copy16(sFb + bslot * plane4, at, 16);
+            if (fb1) copy16(sFb + bslot * plane4 + LPR, at + M, 16);
         }
+        if (kRun) pb0 += Q, pb1 += Q, pr += Q, pk += Q;
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     // the entry past the end of a row: to the right (P = 1) or to the left (P = 0); past the tile's row it is a
@@ -223,7 +312,20 @@ sweep_kernel(const SweepArgs a)
 
     float4 bm0 = zero4(), bm1 = zero4(), bc0 = zero4(), bc1 = zero4(), bp0, bp1;  // b: planes k-1, k, k+1
     float4 rm0 = zero4(), rm1 = zero4(), rc0 = zero4(), rc1 = zero4(), rp0, rp1;  // red: planes k-2, k-1, k
-    int fs = 0;  // place of k in the rings of f
+    int fs = 0, gs = 0;  // places of red f(k) and black f(k-1) in their rings
+    // RES: the new black values of planes k-2, k-3, the residuals of plane k-3 (rows ja, ja + 1), and of the coarse
+    // plane in the making its centre and edge terms (restrict_node's, in its order)
+    float4 n20 = zero4(), n21 = zero4(), n30 = zero4(), n31 = zero4(), e0 = zero4(), e1 = zero4();
+    float4 um = zero4(), tm = zero4(), edge = zero4(), centre = zero4();
+    const int Jc = (ja + 1) >> 1;  // the coarse row on row ja + 1
+    const int nh = n >> 1;
+    float* const fc = RES ? a.fc + (long long)set * 2 * a.vc.cs : nullptr;
+    auto left = [&](const float4& v, const float4* srow) {  // the entry before a group of four
+        float l = __shfl_up_sync(0xffffffffu, v.w, 1);
+        if (kTiledX && lane == 0 && x != 0) l = srow[-1].w;
+        return l;
+    };
+    auto shifted = [](const float4& v, float l) { return make_float4(l, v.x, v.y, v.z); };
 
     using Even = std::integral_constant<int, 0>;
     using Odd = std::integral_constant<int, 1>;
@@ -233,7 +335,7 @@ sweep_kernel(const SweepArgs a)
         constexpr int KP = decltype(KPc)::value;
         // the copies of step k + kAhead go where nothing is read any more: b's place held plane k-1, which the
         // neighbouring rows read before the last barrier, f's held what this thread read in step k-1
-        fetch(k + kAhead, fs == 0 ? kRingF - 1 : fs - 1);
+        fetch(k + kAhead, (fs + kAhead) % kRingFr, gs == 0 ? kRingFb - 1 : gs - 1);
         asm volatile("cp.async.wait_group %0;" ::"n"(kAhead) : "memory");
         if (MODE != kZero) {  // plane k+1 has arrived
             float4* s = sB + ((k + 1) & (kRingB - 1)) * plane4;
@@ -256,20 +358,18 @@ sweep_kernel(const SweepArgs a)
         using Pb = std::integral_constant<int, P1>;
         const float4 f0 = sFr[fs * plane4], f1 = sFr[fs * plane4 + LPR];
         if (MODE == kZero) {
-            const float z = 0.0f;
-            rp0 = make_float4((z - a.h2 * f0.x) * a.sixth, (z - a.h2 * f0.y) * a.sixth, (z - a.h2 * f0.z) * a.sixth,
-                              (z - a.h2 * f0.w) * a.sixth);
-            rp1 = make_float4((z - a.h2 * f1.x) * a.sixth, (z - a.h2 * f1.y) * a.sixth, (z - a.h2 * f1.z) * a.sixth,
-                              (z - a.h2 * f1.w) * a.sixth);
+            rp0 = relax4(zero4(), f0, a.h2, a.sixth);
+            rp1 = relax4(zero4(), f1, a.h2, a.sixth);
         } else {
             const float4* s = sB + (k & (kRingB - 1)) * plane4;
             const float4 ym = up ? s[-LPR] : zero4(), yp = dn ? s[2 * LPR] : zero4();
-            rp0 = relax4<P0>(bc0, beyond(Pa{}, bc0, s), ym, bc1, bm0, bp0, f0, a.h2, a.sixth);
-            rp1 = relax4<P1>(bc1, beyond(Pb{}, bc1, s + LPR), bc0, yp, bm1, bp1, f1, a.h2, a.sixth);
+            rp0 = relax4(sum6<P0>(bc0, beyond(Pa{}, bc0, s), ym, bc1, bm0, bp0), f0, a.h2, a.sixth);
+            rp1 = relax4(sum6<P1>(bc1, beyond(Pb{}, bc1, s + LPR), bc0, yp, bm1, bp1), f1, a.h2, a.sixth);
         }
-        const bool kin = k >= 1 && k < n;
-        if (!(kin && in0)) rp0 = zero4();
-        if (!(kin && in1)) rp1 = zero4();
+        if (!all_in || k < 1 || k >= n) {
+            if (!in0 || k < 1 || k >= n) rp0 = zero4();
+            if (!in1 || k < 1 || k >= n) rp1 = zero4();
+        }
         if (gx == 0) {  // i = 0 is a boundary node
             if (P0 == 0) rp0.x = 0.0f;
             if (P1 == 0) rp1.x = 0.0f;
@@ -278,33 +378,79 @@ sweep_kernel(const SweepArgs a)
             float4* s = sR + (k & 1) * plane4;
             s[0] = rp0, s[LPR] = rp1;
         }
-        if (k > kb) {  // black values of plane k-1, whose rows have the parities of the red ones of plane k
+        if (RES && k >= kb + 3) {  // the residuals of plane q into the coarse plane
+            const int q = k - 3;
+            const float4* se = sE + ((k - 1) & 1) * res4;
+            const float4 e2 = w + 1 < W ? se[kResRow] : zero4();  // row ja + 2
+            if (KP == 1) {  // q even: the plane of the coarse nodes
+                centre = e1;
+                edge = add4(add4(e2, shifted(e2, left(e2, se + kResRow))), add4(e0, shifted(e0, left(e0, se))));
+            } else {
+                const float4 u = add4(e1, shifted(e1, left(e1, se + LPR))), t = add4(e2, e0);
+                const int K = (q - 1) >> 1;
+                if (q >= kb + 2 && gout && pair_out && Jc >= 1 && Jc < nh && K < nh && gin) {
+                    const float4 s = add4(add4(edge, add4(u, um)), add4(t, tm));
+                    const float c0 = 0.125f * centre.x + 0.03125f * s.x, c1 = 0.125f * centre.y + 0.03125f * s.y;
+                    const float c2 = 0.125f * centre.z + 0.03125f * s.z, c3 = 0.125f * centre.w + 0.03125f * s.w;
+                    const int col = (Jc + K) & 1;  // colour of the nodes with even I
+                    const long long at = ((long long)K * (nh + 1) + Jc) * a.vc.M + 2 * gx;
+                    float* A = fc + (long long)col * a.vc.cs + at;
+                    if (gx == 0) A[1] = c2;  // I = 0 is a boundary node
+                    else *reinterpret_cast<float2*>(A) = make_float2(c0, c2);
+                    *reinterpret_cast<float2*>(fc + (long long)(col ^ 1) * a.vc.cs + at) = make_float2(c1, c3);
+                }
+                um = u, tm = t;
+            }
+        }
+        float4 b0 = zero4(), b1 = zero4();
+        if (k > kb - (RES ? 1 : 0)) {  // black values of plane k-1, whose rows have the parities of the red ones of plane k
             const float4* s = sR + ((k - 1) & 1) * plane4;
             const float4 ym = up ? s[-LPR] : zero4(), yp = dn ? s[2 * LPR] : zero4();
-            const float4 g0 = sFb[fs * plane4], g1 = sFb[fs * plane4 + LPR];
-            float4 b0 = relax4<P0>(rc0, beyond(Pa{}, rc0, s), ym, rc1, rm0, rp0, g0, a.h2, a.sixth);
-            float4 b1 = relax4<P1>(rc1, beyond(Pb{}, rc1, s + LPR), rc0, yp, rm1, rp1, g1, a.h2, a.sixth);
+            const float4 g0 = sFb[gs * plane4], g1 = sFb[gs * plane4 + LPR];
+            b0 = relax4(sum6<P0>(rc0, beyond(Pa{}, rc0, s), ym, rc1, rm0, rp0), g0, a.h2, a.sixth);
+            b1 = relax4(sum6<P1>(rc1, beyond(Pb{}, rc1, s + LPR), rc0, yp, rm1, rp1), g1, a.h2, a.sixth);
             if (gx == 0) {
                 if (P0 == 0) b0.x = 0.0f;
                 if (P1 == 0) b1.x = 0.0f;
             }
             const long long o = Q * (k - 1);
-            if (out0) *reinterpret_cast<float4*>(out + o) = b0;
-            if (out1) *reinterpret_cast<float4*>(out + o + M) = b1;
+            const bool own = !RES || (k - 1 >= kb && k - 1 < ke);
+            if (own && out0) *reinterpret_cast<float4*>(out + o) = b0;
+            if (own && out1) *reinterpret_cast<float4*>(out + o + M) = b1;
+            if (RES) {
+                if (!all_in || k - 1 < 1 || k - 1 >= n) {
+                    if (!in0 || k - 1 < 1 || k - 1 >= n) b0 = zero4();
+                    if (!in1 || k - 1 < 1 || k - 1 >= n) b1 = zero4();
+                }
+                float4* d = sN + ((k - 1) & 1) * plane4;
+                d[0] = b0, d[LPR] = b1;
+            }
             if (RED) {
                 if (out0) *reinterpret_cast<float4*>(red + o) = rc0;
                 if (out1) *reinterpret_cast<float4*>(red + o + M) = rc1;
             }
         }
+        if (RES && k >= kb + 2 && k <= ke + 2) {  // red residuals of plane k-2, rows as those of plane k
+            const float4* s = sN + (k & 1) * plane4;
+            const float4 ym = up ? s[-LPR] : zero4(), yp = dn ? s[2 * LPR] : zero4();
+            const int f2 = (fs + kRingFr - 2) % kRingFr;
+            const float4 g0 = sFr[f2 * plane4], g1 = sFr[f2 * plane4 + LPR];
+            e0 = resid4(sum6<P0>(n20, beyond(Pa{}, n20, s), ym, n21, n30, b0), rm0, g0, a.ih2);
+            e1 = resid4(sum6<P1>(n21, beyond(Pb{}, n21, s + LPR), n20, yp, n31, b1), rm1, g1, a.ih2);
+            float4* d = sE + (k & 1) * res4;
+            d[0] = e0;
+            if (kTiledX) d[LPR] = e1;
+        }
+        if (RES) n30 = n20, n31 = n21, n20 = b0, n21 = b1;
         bm0 = bc0, bm1 = bc1, bc0 = bp0, bc1 = bp1;
         rm0 = rc0, rm1 = rc1, rc0 = rp0, rc1 = rp1;
-        fs = fs == kRingF - 1 ? 0 : fs + 1;
+        fs = fs == kRingFr - 1 ? 0 : fs + 1;
+        gs = gs == kRingFb - 1 ? 0 : gs + 1;
         __syncthreads();
     };
 
-    const int ks = kb - 1;  // the first step (even)
 #pragma unroll
-    for (int q = 0; q < kAhead; ++q) fetch(ks + q, q);
+    for (int q = 0; q < kAhead; ++q) fetch(ks + q, q, q);
     if (MODE != kZero) {  // planes ks - 1 and ks of b
         auto load = [&](int k, float4& q0, float4& q1) {
             if (k >= 1 && k < n) {
@@ -335,9 +481,9 @@ sweep_kernel(const SweepArgs a)
     for (int k = ks;; k += 2) {
         if (MODE == kProlong) finish_coarse(cb);
         step(Even{}, k);
-        if (k + 1 > ke) break;
+        if (k + 1 > klast) break;
         step(Odd{}, k + 1);
-        if (k + 2 > ke) break;
+        if (k + 2 > klast) break;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -346,25 +492,23 @@ sweep_kernel(const SweepArgs a)
 // reads c + 4 of b, so large CTAs (512 threads, one on an SM) load and recompute least; they are taken where the
 // level fills the GPU with them.  Levels that do not are latency-bound and take CTAs of 128 threads: a plain sweep of
 // 129^3 7.2 us instead of 7.5, of 65^3 3.9 instead of 4.9; 257^3 25.7 us with 512 threads, 31.5 with 256.
-constexpr int kThreads = 512, kThreadsSmall = 128;
 constexpr long long kLarge = 1 << 20;   // threads that a plane-by-plane pass of the level has work for
-constexpr size_t kSmem = 227 * 1024;    // shared memory of an SM
 
-// The chunk whose waves of CTAs take the fewest plane steps, each CTA taking its planes and about six more (the halo
-// and the first loads).
-int best_chunk(int rows, long long columns, int slots)
+// The chunk whose waves of CTAs take the fewest plane steps, each CTA taking its planes and `extra` more (the halo and
+// the first loads).
+int best_chunk(int rows, long long columns, int slots, int extra)
 {
     int best = 2;
     long long cost = -1;
     for (int c = 2; c <= 64; c += 2) {
         const long long ctas = columns * ((rows + c - 1) / c);
-        const long long t = (ctas + slots - 1) / slots * (c + 6);
+        const long long t = (ctas + slots - 1) / slots * (c + extra);
         if (cost < 0 || t < cost) cost = t, best = c;
     }
     return best;
 }
 
-template <int LPR, int MODE, bool RED>
+template <int LPR, int MODE, int AFTER>
 void launch(const SweepArgs& in, cudaStream_t s, const Sets& sets)
 {
     static int sms = 0;
@@ -376,44 +520,49 @@ void launch(const SweepArgs& in, cudaStream_t s, const Sets& sets)
     SweepArgs a = in;
     const int rows = a.v.n - 1;
     constexpr int kWarpPairs = LPR >= 32 ? 1 : 32 / LPR;  // row pairs of a warp: W is a multiple
-    const int maxw = ((long long)rows * rows * (a.v.n / 8) * sets.n >= kLarge ? kThreads : kThreadsSmall) / LPR;
+    constexpr int kHalo = 4 * halo_pairs<AFTER>();        // rows of a tile that are no output
+    constexpr int kSmall = AFTER == kRestrict && LPR > 8 ? 2 * kThreadsSmall : kThreadsSmall;
+    const int maxw = (long long)rows * rows * (a.v.n / 8) * sets.n >= kLarge ? most_pairs<LPR, MODE, AFTER>()
+                                                                             : kSmall / LPR;
     const int xt = LPR == kWide ? a.v.n / 256 : 1;         // tiles along a row
-    a.tiles = (rows + 2 * maxw - 5) / (2 * maxw - 4);
-    int W = ((rows + a.tiles - 1) / a.tiles + 5) / 2;      // 2W - 4 >= rows / tiles
+    a.tiles = (rows + 2 * maxw - kHalo - 1) / (2 * maxw - kHalo);
+    int W = ((rows + a.tiles - 1) / a.tiles + kHalo + 1) / 2;  // 2W - kHalo >= rows / tiles
     W = (W + kWarpPairs - 1) / kWarpPairs * kWarpPairs;
     const int threads = W * LPR;
-    const size_t smem = sizeof(float4) * (size_t)smem_planes<MODE>() * 2 * W * LPR;
-    const int per_sm = max(1, min(512 / threads, (int)(kSmem / smem)));
-    a.chunk = best_chunk(rows, (long long)a.tiles * xt * sets.n, sms * per_sm);
+    const size_t smem = sizeof(float4) * (size_t)smem_planes<LPR, MODE, AFTER>() * 2 * W * LPR;
+    const int per_sm = max(1, min(most_threads<LPR, MODE, AFTER>() / threads, (int)(kSmem / smem)));
+    a.chunk = best_chunk(rows, (long long)a.tiles * xt * sets.n, sms * per_sm, AFTER == kRestrict ? 11 : 6);
     const dim3 grid((unsigned)(a.tiles * ((rows + a.chunk - 1) / a.chunk)), (unsigned)sets.n, (unsigned)xt);
-    sweep_kernel<LPR, MODE, RED><<<grid, threads, smem, s>>>(a);
+    sweep_kernel<LPR, MODE, AFTER><<<grid, threads, smem, s>>>(a);
 }
 
-// The forms that a V-cycle uses: a leg of an even number of sweeps writes the red values in its last one, which is
-// a plain one.
+// The forms that a V-cycle uses: each leg has an even number of sweeps, the last of which, a plain one, is followed
+// by the restriction or leaves the red values.
 template <int LPR>
-void launch_mode(const SweepArgs& a, int mode, bool red, cudaStream_t s, const Sets& sets)
+void launch_mode(const SweepArgs& a, int mode, int after, cudaStream_t s, const Sets& sets)
 {
-    if (mode == kZero) launch<LPR, kZero, false>(a, s, sets);
-    else if (mode == kProlong) launch<LPR, kProlong, false>(a, s, sets);
-    else if (red) launch<LPR, kPlain, true>(a, s, sets);
-    else launch<LPR, kPlain, false>(a, s, sets);
+    if (mode == kZero) launch<LPR, kZero, kNothing>(a, s, sets);
+    else if (mode == kProlong) launch<LPR, kProlong, kNothing>(a, s, sets);
+    else if (after == kRestrict) launch<LPR, kPlain, kRestrict>(a, s, sets);
+    else if (after == kRed) launch<LPR, kPlain, kRed>(a, s, sets);
+    else launch<LPR, kPlain, kNothing>(a, s, sets);
 }
 
-template <int LPR, int MODE, bool RED>
+template <int LPR, int MODE, int AFTER>
 cudaError_t prepare()
 {
-    return cudaFuncSetAttribute(sweep_kernel<LPR, MODE, RED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sizeof(float4) * smem_planes<MODE>() * 2 * kThreads));
+    return cudaFuncSetAttribute(sweep_kernel<LPR, MODE, AFTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(float4) * smem_planes<LPR, MODE, AFTER>() * 2 * LPR * most_pairs<LPR, MODE, AFTER>()));
 }
 
 template <int LPR>
 cudaError_t prepare_lpr()
 {
-    cudaError_t e = prepare<LPR, kPlain, false>();
-    if (e == cudaSuccess) e = prepare<LPR, kPlain, true>();
-    if (e == cudaSuccess) e = prepare<LPR, kZero, false>();
-    if (e == cudaSuccess) e = prepare<LPR, kProlong, false>();
+    cudaError_t e = prepare<LPR, kPlain, kNothing>();
+    if (e == cudaSuccess) e = prepare<LPR, kPlain, kRed>();
+    if (e == cudaSuccess) e = prepare<LPR, kPlain, kRestrict>();
+    if (e == cudaSuccess) e = prepare<LPR, kZero, kNothing>();
+    if (e == cudaSuccess) e = prepare<LPR, kProlong, kNothing>();
     return e;
 }
 
@@ -432,8 +581,8 @@ cudaError_t prepare_sweep_level(int n)
     }
 }
 
-void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepStart start, bool to_t, bool red,
-                  const float* ec, const LevelView& vc, double h, cudaStream_t s, const Sets& sets)
+void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepStart start, bool to_t, SweepAfter after,
+                  const float* ec, float* fc, const LevelView& vc, double h, cudaStream_t s, const Sets& sets)
 {
     SweepArgs a{};
     float* eb = e + v.cs;
@@ -441,20 +590,22 @@ void launch_sweep(float* e, float* t, const float* f, const LevelView& v, SweepS
     a.bset = to_t ? 2 * v.cs : v.cs;
     a.out = to_t ? t : eb;
     a.oset = to_t ? v.cs : 2 * v.cs;
-    a.red = red ? e : nullptr;
+    a.red = e;
     a.f = f;
     a.ec = ec;
+    a.fc = fc;
     a.v = v;
     a.vc = vc;
     a.h2 = (float)(h * h);
     a.sixth = 1.0f / 6.0f;
+    a.ih2 = (float)(1.0 / (h * h));
     a.act = sets.act;
     const int mode = (int)start;
     switch (v.n) {
-    case 64: launch_mode<8>(a, mode, red, s, sets); break;
-    case 128: launch_mode<16>(a, mode, red, s, sets); break;
-    case 256: launch_mode<32>(a, mode, red, s, sets); break;
-    default: launch_mode<kWide>(a, mode, red, s, sets); break;
+    case 64: launch_mode<8>(a, mode, (int)after, s, sets); break;
+    case 128: launch_mode<16>(a, mode, (int)after, s, sets); break;
+    case 256: launch_mode<32>(a, mode, (int)after, s, sets); break;
+    default: launch_mode<kWide>(a, mode, (int)after, s, sets); break;
     }
 }
 
