@@ -554,7 +554,28 @@ struct CoarseSmem {
     T* u[kMaxCoarseLevels];
     T* f[kMaxCoarseLevels];
     T* r[kMaxCoarseLevels];
+    T* x[kMaxCoarseLevels];  // row exchange of the levels n >= 8
 };
+
+// Elements of level n in the coarse solver's shared memory: u, f, r and the row exchange.
+__host__ __device__ inline int row_exchange(int n) { return n >= 8 ? (n + 1) * (n + 2) * n : 0; }
+__host__ __device__ inline int cube4(int n) { return (cube(n) + 3) & ~3; }
+__host__ __device__ inline int coarse_elems(int n) { return 3 * cube4(n) + row_exchange(n); }
+
+template <typename T>
+__device__ __forceinline__ void coarse_layout(CoarseSmem<T>& S, T* base, int top)
+{
+#pragma unroll
+    for (int l = 0; l < kMaxCoarseLevels; ++l) {
+        if (l > top) break;
+        const int c = cube4(2 << l);
+        S.x[l] = base;
+        S.u[l] = base + row_exchange(2 << l);
+        S.f[l] = S.u[l] + c;
+        S.r[l] = S.f[l] + c;
+        base += coarse_elems(2 << l);
+    }
+}
 
 // Every level size is a compile-time constant (N = 2 << L), so the index
 // arithmetic below is shifts and multiplications.  Each routine is run either
@@ -578,12 +599,18 @@ __device__ __forceinline__ void sm_sync()
         __syncthreads();
 }
 
+// a b + c rounded once (written out: where a product is the same in every
+// sweep, the compiler would round it on its own and keep it).
+__device__ __forceinline__ float fused(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fused(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // One colour of the interior of an N-level: row (j, k) holds that colour's
 // nodes at i = first, first + 2, ... (first = 1 or 2), N/2 slots per row.
 // The stride is a multiple of N/2, so a thread keeps its slot and steps its
 // row (j, k) without divisions (the residual and the prolongation below do
 // the same with N lanes per row, the last one idle).
-template <typename T, int N, bool W = false>
+// ZERO: every neighbour is known to be zero.
+template <typename T, int N, bool W = false, bool ZERO = false>
 __device__ void sm_relax(T* u, const T* f, T h2, int colour)
 {
     constexpr int M = N - 1, P = N + 1, H = N / 2, ROWS = M * M;
@@ -596,8 +623,9 @@ __device__ void sm_relax(T* u, const T* f, T h2, int colour)
         const int i = 1 + (((1 + j + k) & 1) != colour ? 1 : 0) + 2 * sl;
         if (i <= M) {
             const int o = i + P * (j + P * k);
-            const T sum = (u[o + 1] + u[o - 1]) + (u[o + P] + u[o - P]) + (u[o + P * P] + u[o - P * P]);
-            u[o] = (sum - h2 * f[o]) * (T(1) / T(6));
+            T sum = T(0);
+            if (!ZERO) sum = (u[o + 1] + u[o - 1]) + (u[o + P] + u[o - P]) + (u[o + P * P] + u[o - P * P]);
+            u[o] = fused(-h2, f[o], sum) * (T(1) / T(6));
         }
         j += dj;
         k += dk;
@@ -685,6 +713,30 @@ __device__ void sm_prolong(const T* coarse, T* fine, bool add)
     sm_sync<W>();
 }
 
+// The correction of the black nodes alone (the red half-sweep after it does not
+// read the red ones): as sm_prolong, with the slots of sm_relax.
+template <typename T, int NC>
+__device__ void sm_correct(const T* coarse, T* fine)
+{
+    constexpr int NF = 2 * NC, M = NF - 1, PF = NF + 1, PC = NC + 1, H = NF / 2, ROWS = M * M;
+    const int dr = (int)blockDim.x / H, sl = (int)threadIdx.x % H;
+    for (int row = (int)threadIdx.x / H; row < ROWS; row += dr) {
+        const int j = row % M + 1, k = row / M + 1;
+        const int i = 1 + ((j + k) & 1) + 2 * sl;
+        if (i <= M) {
+            const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1, K0 = k >> 1, K1 = (k + 1) >> 1;
+            T sum = (coarse[I0 + PC * (J0 + PC * K0)] + coarse[I1 + PC * (J0 + PC * K0)])
+                  + (coarse[I0 + PC * (J1 + PC * K0)] + coarse[I1 + PC * (J1 + PC * K0)]);
+            sum += (coarse[I0 + PC * (J0 + PC * K1)] + coarse[I1 + PC * (J0 + PC * K1)])
+                 + (coarse[I0 + PC * (J1 + PC * K1)] + coarse[I1 + PC * (J1 + PC * K1)]);
+            sum *= T(0.125);
+            const int o = i + PF * (j + PF * k);
+            fine[o] = fine[o] + sum;
+        }
+    }
+    __syncthreads();
+}
+
 template <typename T, int N, bool W = false>
 __device__ void sm_fill(T* a, T val)
 {
@@ -704,32 +756,430 @@ __device__ void sm_coarsest(T* u, const T* f, T h)
     sm_sync<W>();
 }
 
+// --- the levels n = 8 and 16 with a row of nodes per thread ---------------------------------------------------------
+// A phase of these levels is bound by latencies (a few shared-memory reads, a
+// short chain of sums, a block barrier), so a thread keeps a whole interior row
+// (j, k) and its right-hand side in registers for the whole V-cycle: nodes of
+// odd i in O, of even i in E (its last entry the boundary node i = n), the
+// x-neighbours are its own, and the rows j +- 1, k +- 1 come from an exchange
+// array in vectors of four nodes.  Rows with j + k even (s = 0) take the first
+// half of the threads and the others the second, so that a warp updates O or
+// E as a whole.  Measured, one V-cycle from the level 17^3 (FP32, its launch
+// included): 10.1 us, 17.3 with a node at a time from the natural layout (a
+// half-sweep 0.8 us).  The nodes' arithmetic is sm_relax's, sm_residual's and
+// sm_prolong's; the correction goes to the black nodes only (the red half-sweep
+// after it does not read the red ones).
+template <typename T>
+struct alignas(16) RowVec {
+    T v[4];
+};
+
+template <typename T, int N>
+struct Row {
+    static constexpr int M = N - 1, P = N + 1, H = N / 2, NV = N / 8;
+    static constexpr int ROWS = 2 * (N + 1) * (H + 1);         // rows (s, k, j >> 1) of the exchange
+    static constexpr int HALF = (M * M / 2 + 1 + 31) / 32 * 32;  // threads of the rows of one s
+    int s, j, k;
+    bool on;
+    T O[H], E[H], eL;  // i = 1, 3, ..; 2, 4, .., N; i = 0
+    T fO[H], fE[H];
+
+    __device__ __forceinline__ Row()
+    {
+        const int t = (int)threadIdx.x;
+        s = t >= HALF ? 1 : 0;
+        const int r = t - s * HALF;
+        // planes in pairs: for s = 0 plane 2q+1 has H rows (odd j) and plane 2q+2 H-1 (even j); for s = 1 the reverse
+        const int q = r / M, m = r - q * M, first = s ? H - 1 : H;
+        k = 2 * q + 1 + (m >= first ? 1 : 0);
+        j = m < first ? 2 * m + (s ? 2 : 1) : 2 * (m - first) + (s ? 1 : 2);
+        on = t < 2 * HALF && k <= M;
+    }
+    static __device__ __forceinline__ int row(int sv, int kv, int jv) { return (sv * P + kv) * (H + 1) + (jv >> 1); }
+    static __device__ __forceinline__ RowVec<T>* vec(T* x, int v, int even, int r)
+    {
+        return reinterpret_cast<RowVec<T>*>(x) + (v * 2 + even) * ROWS + r;
+    }
+    template <bool EVEN>
+    __device__ __forceinline__ void put(T* x) const
+    {
+        const T* a = EVEN ? E : O;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            RowVec<T> w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w.v[e] = a[4 * v + e];
+            *vec(x, v, EVEN, row(s, k, j)) = w;
+        }
+    }
+    // the sums of the six neighbours of the row's nodes of one parity of i; ZERO: known to be zero
+    template <bool EVEN>
+    __device__ __forceinline__ void sums(T* x, T (&sum)[H]) const
+    {
+        const int o = s ^ 1;
+        const int ym = row(o, k, j - 1), yp = row(o, k, j + 1), zm = row(o, k - 1, j), zp = row(o, k + 1, j);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const RowVec<T> a = *vec(x, v, EVEN, ym), b = *vec(x, v, EVEN, yp);
+            const RowVec<T> c = *vec(x, v, EVEN, zm), d = *vec(x, v, EVEN, zp);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int q = 4 * v + e;
+                const T right = EVEN ? (q + 1 < H ? O[q + 1 < H ? q + 1 : 0] : T(0)) : E[q];
+                const T left = EVEN ? O[q] : (q == 0 ? eL : E[q == 0 ? 0 : q - 1]);
+                sum[q] = (right + left) + (b.v[e] + a.v[e]) + (d.v[e] + c.v[e]);
+            }
+        }
+    }
+    template <bool EVEN, bool ZERO>
+    __device__ __forceinline__ void relax_own(T* x, T h2)
+    {
+        T sum[H];
+        if (ZERO) {
+#pragma unroll
+            for (int q = 0; q < H; ++q) sum[q] = T(0);
+        } else {
+            sums<EVEN>(x, sum);
+        }
+#pragma unroll
+        for (int q = 0; q < (EVEN ? H - 1 : H); ++q) {
+            T& u = EVEN ? E[q] : O[q];
+            u = fused(-h2, EVEN ? fE[q] : fO[q], sum[q]) * (T(1) / T(6));
+        }
+        put<EVEN>(x);
+    }
+    template <bool ZERO>
+    __device__ __forceinline__ void relax(T* x, T h2, int colour)
+    {
+        if (on) {
+            if ((s ^ colour) == 0) relax_own<true, ZERO>(x, h2);  // this colour's nodes of the row have even i
+            else relax_own<false, ZERO>(x, h2);
+        }
+        __syncthreads();
+    }
+    // Residual of every interior node of the row into r: rows of N + 4, odd i first and even i from H on, so that the
+    // threads of restrict_rows read neighbouring words.
+    static constexpr int RS = N + 4;
+    __device__ __forceinline__ void residual(T* x, T* r, T ih2) const
+    {
+        if (on) {
+            T* at = r + RS * (j - 1 + M * (k - 1));
+            auto half = [&](const T* f, const T* u, const T (&sum)[H], T* to) {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    RowVec<T> w;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int q = 4 * v + e;
+                        w.v[e] = fused(-fused(T(-6), u[q], sum[q]), ih2, f[q]);
+                    }
+                    reinterpret_cast<RowVec<T>*>(to)[v] = w;
+                }
+            };
+            T sum[H];
+            sums<false>(x, sum);
+            half(fO, O, sum, at);
+            sums<true>(x, sum);
+            half(fE, E, sum, at + H);
+        }
+        __syncthreads();
+    }
+    // sm_restrict from that layout
+    static __device__ __forceinline__ void restrict_rows(const T* r, T* coarse)
+    {
+        constexpr int MC = H - 1, PC = H + 1;
+        for (int t = (int)threadIdx.x; t < MC * MC * MC; t += (int)blockDim.x) {
+            const int I = t % MC + 1, J = (t / MC) % MC + 1, K = t / (MC * MC) + 1;
+            T acc = T(0);
+#pragma unroll
+            for (int c = -1; c <= 1; ++c)
+#pragma unroll
+                for (int b = -1; b <= 1; ++b) {
+                    const T* at = r + RS * (2 * J + b - 1 + M * (2 * K + c - 1)) + I - 1;
+                    const T w = T(0.125) * T(b == 0 ? 2 : 1) * T(c == 0 ? 2 : 1) * T(0.125);
+                    acc += w * at[0];
+                    acc += T(2) * w * at[H];
+                    acc += w * at[1];
+                }
+            coarse[I + PC * (J + PC * K)] = acc;
+        }
+        __syncthreads();
+    }
+    // the correction of the row's black nodes from the natural coarse array c
+    __device__ __forceinline__ void correct(T* x, const T* c)
+    {
+        if (on) {
+            constexpr int PC = H + 1;
+            const T* c00 = c + PC * ((j >> 1) + PC * (k >> 1));
+            const T* c10 = c + PC * (((j + 1) >> 1) + PC * (k >> 1));
+            const T* c01 = c + PC * ((j >> 1) + PC * ((k + 1) >> 1));
+            const T* c11 = c + PC * (((j + 1) >> 1) + PC * ((k + 1) >> 1));
+            if (s == 0) {  // black: odd i = 2q + 1, between I = q and q + 1
+#pragma unroll
+                for (int q = 0; q < H; ++q) {
+                    T sum = (c00[q] + c00[q + 1]) + (c10[q] + c10[q + 1]);
+                    sum += (c01[q] + c01[q + 1]) + (c11[q] + c11[q + 1]);
+                    sum *= T(0.125);
+                    O[q] = O[q] + sum;
+                }
+                put<false>(x);
+            } else {  // even i = 2q + 2, on I = q + 1
+#pragma unroll
+                for (int q = 0; q < H - 1; ++q) {
+                    T sum = (c00[q + 1] + c00[q + 1]) + (c10[q + 1] + c10[q + 1]);
+                    sum += (c01[q + 1] + c01[q + 1]) + (c11[q + 1] + c11[q + 1]);
+                    sum *= T(0.125);
+                    E[q] = E[q] + sum;
+                }
+                put<true>(x);
+            }
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void load_f(const T* f)
+    {
+        const T* at = f + P * (j + P * k);
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            fO[q] = on ? at[2 * q + 1] : T(0);
+            fE[q] = on && q < H - 1 ? at[2 * q + 2] : T(0);
+        }
+    }
+    __device__ __forceinline__ void load_u(const T* u)
+    {
+        const T* at = u + P * (j + P * k);
+        eL = on ? at[0] : T(0);
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            O[q] = on ? at[2 * q + 1] : T(0);
+            E[q] = on ? at[2 * q + 2] : T(0);
+        }
+    }
+    // The same row of a level in global memory (colour-split rows of lv.M entries): the colour with even i holds
+    // i = 2m at m, the other i = 2m + 1.
+    __device__ __forceinline__ void load_f(const T* __restrict__ f, const LevelView& lv)
+    {
+        clear_f();
+        if (!on) return;
+        const long long at = ((long long)k * P + j) * lv.M;
+        const T* ev = f + (s ? lv.cs : 0) + at;  // s = 0: red has even i
+        const T* od = f + (s ? 0 : lv.cs) + at;
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            fO[q] = od[q];
+            if (q < H - 1) fE[q] = ev[q + 1];
+        }
+    }
+    __device__ __forceinline__ void store_u(T* __restrict__ e, const LevelView& lv) const
+    {
+        if (!on) return;
+        const long long at = ((long long)k * P + j) * lv.M;
+        T* ev = e + (s ? lv.cs : 0) + at;
+        T* od = e + (s ? 0 : lv.cs) + at;
+#pragma unroll
+        for (int q = 0; q < H; ++q) {
+            od[q] = O[q];
+            if (q < H - 1) ev[q + 1] = E[q];
+        }
+    }
+    __device__ __forceinline__ void clear_f()
+    {
+#pragma unroll
+        for (int q = 0; q < H; ++q) fO[q] = T(0), fE[q] = T(0);
+    }
+    // zero boundary rows in the exchange
+    static __device__ __forceinline__ void clear_boundary(T* x)
+    {
+        for (int t = (int)threadIdx.x; t < 4 * N; t += (int)blockDim.x) {
+            const int side = t / N, a = t - side * N;
+            const int jv = side == 0 ? 0 : side == 1 ? N : a + (side == 3 ? 1 : 0);
+            const int kv = side == 0 ? a + 1 : side == 1 ? a : side == 2 ? 0 : N;
+            const RowVec<T> z = {{T(0), T(0), T(0), T(0)}};
+#pragma unroll
+            for (int v = 0; v < 2 * NV; ++v) *vec(x, v >> 1, v & 1, row((jv + kv) & 1, kv, jv)) = z;
+        }
+    }
+    __device__ __forceinline__ void clear_u()
+    {
+        eL = T(0);
+#pragma unroll
+        for (int q = 0; q < H; ++q) O[q] = T(0), E[q] = T(0);
+    }
+    __device__ __forceinline__ void store_u(T* u) const
+    {
+        if (on) {
+            T* at = u + P * (j + P * k);
+#pragma unroll
+            for (int q = 0; q < H; ++q) {
+                at[2 * q + 1] = O[q];
+                if (q < H - 1) at[2 * q + 2] = E[q];
+            }
+        }
+        __syncthreads();
+    }
+    // the whole natural array u, boundary rows included, into the exchange
+    static __device__ __forceinline__ void fill_exchange(T* x, const T* u)
+    {
+        for (int t = (int)threadIdx.x; t < P * P; t += (int)blockDim.x) {
+            const int jv = t % P, kv = t / P, sv = (jv + kv) & 1;
+            const T* at = u + P * (jv + P * kv);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                RowVec<T> o, e;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) o.v[q] = at[8 * v + 2 * q + 1], e.v[q] = at[8 * v + 2 * q + 2];
+                *vec(x, v, 0, row(sv, kv, jv)) = o;
+                *vec(x, v, 1, row(sv, kv, jv)) = e;
+            }
+        }
+        __syncthreads();
+    }
+};
+
+// The V-cycle of the levels n = 4 and 2 in the registers of one warp: a lane per
+// node, neighbours by shuffles; u and f are the natural arrays of the level
+// n = 4.  The arithmetic of sm_relax, sm_residual, sm_restrict (the terms in the
+// order of the lanes), sm_coarsest and sm_prolong.
+template <typename T>
+__device__ void warp_vcycle4(T* u, const T* f, T h, int npre, int npost)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int P = 5;
+    const int l = (int)threadIdx.x & 31, n = l < 27 ? l : 26;
+    const int i = n % 3 + 1, j = (n / 3) % 3 + 1, k = n / 9 + 1;
+    const int o = i + P * (j + P * k);
+    T v = u[o];
+    const T fv = f[o];
+    const T bx = i == 2 ? T(0) : u[i == 1 ? o - 1 : o + 1];  // the boundary neighbour along each axis, if there is one
+    const T by = j == 2 ? T(0) : u[j == 1 ? o - P : o + P];
+    const T bz = k == 2 ? T(0) : u[k == 1 ? o - P * P : o + P * P];
+    auto sum6 = [&]() {
+        const T xp = __shfl_down_sync(kAll, v, 1), xm = __shfl_up_sync(kAll, v, 1);
+        const T yp = __shfl_down_sync(kAll, v, 3), ym = __shfl_up_sync(kAll, v, 3);
+        const T zp = __shfl_down_sync(kAll, v, 9), zm = __shfl_up_sync(kAll, v, 9);
+        return ((i == 3 ? bx : xp) + (i == 1 ? bx : xm)) + ((j == 3 ? by : yp) + (j == 1 ? by : ym)) +
+               ((k == 3 ? bz : zp) + (k == 1 ? bz : zm));
+    };
+    const int colour = (i + j + k) & 1;
+    const T h2 = h * h;
+    auto relax = [&](int c) {
+        const T w = fused(-h2, fv, sum6()) * (T(1) / T(6));
+        if (colour == c) v = w;
+    };
+    for (int q = 0; q < npre; ++q) {
+        relax(0);
+        relax(1);
+    }
+    {
+        const T r = fused(-fused(T(-6), v, sum6()), T(1) / h2, fv);
+        const T w = T(0.125) * T(i == 2 ? 2 : 1) * T(j == 2 ? 2 : 1) * T(k == 2 ? 2 : 1) * T(0.125);
+        const T p = w * r;  // exact: w is a power of two
+        T acc = T(0);
+#pragma unroll
+        for (int q = 0; q < 27; ++q) acc += __shfl_sync(kAll, p, q);
+        const T hc = h * T(2);
+        const T c = fused(-(hc * hc), acc, T(0)) * (T(1) / T(6));
+        // the coarse node (1, 1, 1) is the only one that is not zero
+        const T x0 = (i >> 1) == 1 ? c : T(0), x1 = ((i + 1) >> 1) == 1 ? c : T(0);
+        auto at = [&](int J, int K) { return J == 1 && K == 1 ? x0 + x1 : T(0); };
+        const int J0 = j >> 1, J1 = (j + 1) >> 1, K0 = k >> 1, K1 = (k + 1) >> 1;
+        T s = at(J0, K0) + at(J1, K0);
+        s += at(J0, K1) + at(J1, K1);
+        s *= T(0.125);
+        v = v + s;
+    }
+    for (int q = 0; q < npost; ++q) {
+        relax(0);
+        relax(1);
+    }
+    if (l < 27) u[o] = v;
+}
+
+template <typename T, int L, bool ZERO>
+__device__ void sm_vcycle(CoarseSmem<T>& S, T h, int npre, int npost);
+
+// The V-cycle from level L down on a row of nodes per thread: right-hand side
+// (and, unless ZERO, the start) in `row`, which holds the result at the end.
+template <typename T, int L, bool ZERO>
+__device__ __forceinline__ void row_vcycle(CoarseSmem<T>& S, Row<T, (2 << L)>& row, T h, int npre, int npost)
+{
+    constexpr int N = 2 << L;
+    for (int q = 0; q < npre; ++q) {
+        if (ZERO && q == 0) row.template relax<true>(S.x[L], h * h, 0);
+        else row.template relax<false>(S.x[L], h * h, 0);
+        row.template relax<false>(S.x[L], h * h, 1);
+    }
+    row.residual(S.x[L], S.r[L], T(1) / (h * h));
+    Row<T, N>::restrict_rows(S.r[L], S.f[L - 1]);
+    if constexpr (!(ZERO && L - 1 >= 2)) sm_fill<T, N / 2>(S.u[L - 1], T(0));
+    sm_vcycle<T, L - 1, ZERO && L - 1 >= 2>(S, h * T(2), npre, npost);
+    row.correct(S.x[L], S.u[L - 1]);
+    for (int q = 0; q < npost; ++q) {
+        row.template relax<false>(S.x[L], h * h, 0);
+        row.template relax<false>(S.x[L], h * h, 1);
+    }
+}
+
+// Levels whose V-cycle keeps rows in registers.  In FP64 the pipe (2 operations
+// a clock) bounds these levels, and more threads with a node each keep it
+// busier (17^3 V-cycle 71 us either way, 9^3 17 us against 21).
+template <typename T, int L>
+constexpr bool by_rows() { return L >= 2 && sizeof(T) == 4; }
+
 // V(npre, npost) cycle from level L down to the 3^3 grid; the coarser levels
-// start from zero (zero boundary values), level L from what u[L] holds.  The
-// levels n <= 4 are run by warp 0 while the rest of the block waits.
-template <typename T, int L, bool W = false>
+// start from zero (zero boundary values), level L from what u[L] holds, or, with
+// ZERO, from zero with zero boundary values (only these are read of u[L], and
+// the boundary rows of its exchange array are zero).  The levels n <= 4 are run
+// by warp 0 while the rest of the block waits.
+template <typename T, int L, bool ZERO = false>
 __device__ void sm_vcycle(CoarseSmem<T>& S, T h, int npre, int npost)
 {
     constexpr int N = 2 << L;
-    if constexpr (!W && L <= 1) {
-        if (threadIdx.x < 32) sm_vcycle<T, L, true>(S, h, npre, npost);
+    if constexpr (L == 0) {
+        sm_coarsest<T>(S.u[0], S.f[0], h);
+    } else if constexpr (L == 1) {
+        if (threadIdx.x < 32) warp_vcycle4(S.u[1], S.f[1], h, npre, npost);
         __syncthreads();
-    } else if constexpr (L == 0) {
-        sm_coarsest<T, W>(S.u[0], S.f[0], h);
+    } else if constexpr (by_rows<T, L>()) {
+        Row<T, N> row;
+        row.load_f(S.f[L]);
+        if (ZERO) {
+            row.clear_u();
+        } else {
+            Row<T, N>::fill_exchange(S.x[L], S.u[L]);
+            row.load_u(S.u[L]);
+        }
+        row_vcycle<T, L, ZERO>(S, row, h, npre, npost);
+        row.store_u(S.u[L]);
     } else {
         for (int q = 0; q < npre; ++q) {
-            sm_relax<T, N, W>(S.u[L], S.f[L], h * h, 0);
-            sm_relax<T, N, W>(S.u[L], S.f[L], h * h, 1);
+            if (ZERO && q == 0) sm_relax<T, N, false, true>(S.u[L], S.f[L], h * h, 0);
+            else sm_relax<T, N>(S.u[L], S.f[L], h * h, 0);
+            sm_relax<T, N>(S.u[L], S.f[L], h * h, 1);
         }
-        sm_residual<T, N, W>(S.u[L], S.f[L], S.r[L], T(1) / (h * h));
-        sm_restrict<T, N, W>(S.r[L], S.f[L - 1]);
-        sm_fill<T, N / 2, W>(S.u[L - 1], T(0));
-        sm_vcycle<T, L - 1, W>(S, h * T(2), npre, npost);
-        sm_prolong<T, N / 2, W>(S.u[L - 1], S.u[L], true);
+        sm_residual<T, N>(S.u[L], S.f[L], S.r[L], T(1) / (h * h));
+        sm_restrict<T, N>(S.r[L], S.f[L - 1]);
+        sm_fill<T, N / 2>(S.u[L - 1], T(0));
+        sm_vcycle<T, L - 1, (L - 1 >= 2)>(S, h * T(2), npre, npost);
+        sm_correct<T, N / 2>(S.u[L - 1], S.u[L]);
         for (int q = 0; q < npost; ++q) {
-            sm_relax<T, N, W>(S.u[L], S.f[L], h * h, 0);
-            sm_relax<T, N, W>(S.u[L], S.f[L], h * h, 1);
+            sm_relax<T, N>(S.u[L], S.f[L], h * h, 0);
+            sm_relax<T, N>(S.u[L], S.f[L], h * h, 1);
         }
+    }
+}
+
+// Before a V-cycle by rows that starts from zero on level L: zero boundary rows
+// in the exchange arrays, and zero boundary values in u of the levels under it
+// (their interior is written before it is read).
+template <typename T, int L>
+__device__ void clear_rows(CoarseSmem<T>& S)
+{
+    if constexpr (by_rows<T, L>()) {
+        Row<T, (2 << L)>::clear_boundary(S.x[L]);
+        if constexpr (L - 1 >= 2)
+            for (int t = (int)threadIdx.x; t < cube(1 << L); t += (int)blockDim.x) S.u[L - 1][t] = T(0);
+        clear_rows<T, L - 1>(S);
     }
 }
 
@@ -778,17 +1228,21 @@ template <typename T, int TOP>
 __device__ void coarse_run(unsigned char* smem_raw, int fmg, T* __restrict__ e, const T* __restrict__ f, LevelView v,
                            T htop, const double* __restrict__ u64, int nfine, int ncycle, int npre, int npost)
 {
-    T* base = reinterpret_cast<T*>(smem_raw);
     CoarseSmem<T> S;
-#pragma unroll
-    for (int l = 0; l <= TOP; ++l) {
-        const int c = cube(2 << l);
-        S.u[l] = base;
-        S.f[l] = base + c;
-        S.r[l] = base + 2 * c;
-        base += 3 * c;
-    }
+    coarse_layout(S, reinterpret_cast<T*>(smem_raw), TOP);
     constexpr int N = 2 << TOP, P = N + 1, TOT = P * P * P;
+    if constexpr (by_rows<T, TOP>()) {
+        if (!fmg) {  // the top level goes from global memory to the threads' rows and back (its boundary nodes hold zeros)
+            Row<T, N> row;
+            row.load_f(f, v);
+            row.clear_u();
+            clear_rows<T, TOP>(S);
+            __syncthreads();
+            row_vcycle<T, TOP, true>(S, row, htop, npre, npost);
+            row.store_u(e, v);
+            return;
+        }
+    }
     // right-hand side of the top level (interior), zero elsewhere
 #pragma unroll 5
     for (int t = threadIdx.x; t < TOT; t += (int)blockDim.x) {
@@ -805,7 +1259,7 @@ __device__ void coarse_run(unsigned char* smem_raw, int fmg, T* __restrict__ e, 
     } else {
         for (int t = threadIdx.x; t < TOT; t += (int)blockDim.x) S.u[TOP][t] = T(0);
         __syncthreads();
-        sm_vcycle<T, TOP>(S, htop, npre, npost);
+        sm_vcycle<T, TOP, (TOP >= 2)>(S, htop, npre, npost);
     }
 #pragma unroll 5
     for (int t = threadIdx.x; t < TOT; t += (int)blockDim.x) {
@@ -1121,16 +1575,7 @@ __global__ void __launch_bounds__(kSlabThreads) vslab_kernel(SlabArgs a)
     float** pf = pe + 40;
     unsigned char* coarse_raw = reinterpret_cast<unsigned char*>(pf + 40);
     CoarseSmem<float> S;
-    {
-        float* base = reinterpret_cast<float*>(coarse_raw);
-        for (int l = 0; l <= 3; ++l) {
-            const int c = cube(2 << l);
-            S.u[l] = base;
-            S.f[l] = base + c;
-            S.r[l] = base + 2 * c;
-            base += 3 * c;
-        }
-    }
+    coarse_layout(S, reinterpret_cast<float*>(coarse_raw), 3);
     float* const e = a.e + (long long)set * 2 * a.cs;
     const float* const f = a.f + (long long)set * 2 * a.cs;
     constexpr int kC3 = kSlabCoarseP * kSlabCoarseP * kSlabCoarseP;
@@ -1166,11 +1611,13 @@ __global__ void __launch_bounds__(kSlabThreads) vslab_kernel(SlabArgs a)
                 v = reinterpret_cast<const float4*>(e + (long long)c * a.cs + (long long)k * kSlabColour)[x];
             reinterpret_cast<float4*>(se + (size_t)(k - k0 + 1) * kSlabPlane + c * kSlabColour)[x] = v;
         }
-        if (rank == 0)  // coarse_run with a zero start: u = 0, f = 0 off the interior
+        if (rank == 0) {  // coarse_run with a zero start: u = 0, f = 0 off the interior
             for (int t = threadIdx.x; t < kC3; t += kSlabThreads) {
                 S.u[3][t] = 0.0f;
                 S.f[3][t] = 0.0f;
             }
+            clear_rows<float, 3>(S);
+        }
     }
     __syncthreads();
     cluster_sync_all();
@@ -1206,7 +1653,7 @@ __global__ void __launch_bounds__(kSlabThreads) vslab_kernel(SlabArgs a)
         }
     }
     cluster_sync_all();
-    if (rank == 0) sm_vcycle<float, 3>(S, a.hc, a.npre, a.npost);
+    if (rank == 0) sm_vcycle<float, 3, true>(S, a.hc, a.npre, a.npost);
     cluster_sync_all();
     // coarse-grid correction of the black nodes (prolong_node's sums in its order); the coarse planes
     // k0/2 .. k1/2 that this slab interpolates from are first copied from CTA 0 into the same place of
@@ -1539,7 +1986,7 @@ template <typename T>
 size_t coarse_smem_bytes(int n)
 {
     size_t tot = 0;
-    for (int m = 2; m <= n; m *= 2) tot += 3 * (size_t)cube(m);
+    for (int m = 2; m <= n; m *= 2) tot += (size_t)coarse_elems(m);
     return tot * sizeof(T);
 }
 

@@ -124,3 +124,25 @@ def test_whole_sweeps_give_the_bits_of_the_solve_without_allocation(q):
     q.qumond.qumond_solve_mond_noalloc(
         q.default_params(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, **kw), 0, src, None, b)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("npre,npost,ncycle", [(1, 1, 1), (2, 2, 6), (3, 1, 2)])
+@pytest.mark.parametrize("n", [2, 4, 8, 16, 32])
+def test_coarse_levels_match_the_oracle(q, ora, n, npre, npost, ncycle):
+    # the levels that one block solves: rows of nodes in registers (n = 8, 16, FP32), a node per lane (n = 4), one
+    # unknown (n = 2); boundary values given, so that each FMG level starts from values other than zero
+    rng = np.random.default_rng(n + npre)
+    L0 = 4.0 * n
+    f = rng.uniform(-1.0, 1.0, (n + 1) ** 3)
+    u = rng.uniform(-1.0, 1.0, (n + 1) ** 3)
+    want = u.copy()
+    ora.fmg(n, L0 / n, want, f, ncycle, npre, npost)
+    for prec, tol in ((q.QUMOND_PREC_FP64, 1e-11), (q.QUMOND_PREC_MIXED, 1e-4)):
+        # FP64: the same iterates, summed in another order; FP32: about 10 roundings of 2^-24 in each of at most 6
+        # cycles of 4 sweeps on 5 levels, 7e-5 of the largest value if all added up
+        ctx = q.Context(n=n, nboxes=1, L0=L0, precision=prec, bc_mode=q.QUMOND_BC_GIVEN, npre=npre, npost=npost,
+                        ncycle=ncycle)
+        phi = to_dev(u)
+        ctx.qumond_solve_mond(0, to_dev(f), None, phi)
+        assert np.max(np.abs(phi.cpu().numpy() - want)) <= tol * np.max(np.abs(want))
+        ctx.close()
