@@ -1465,34 +1465,48 @@ __global__ void __launch_bounds__(kVsubThreads) vcluster_kernel(VsubArgs<T> a, i
 }
 
 // ---------------------------------------------------------------------------
-// The V-cycle from the 32-interval level down, in shared memory: one
-// thread-block cluster of C CTAs per set.  CTA r keeps the planes
-// k0 .. k1-1 of that level's e and f (both colours, each plane's rows laid
-// out as in global memory); CTA 0 also keeps the boundary plane 0 and CTA
-// C-1 the boundary plane 32.  A node on the first or last plane of a slab
-// reads the plane beyond it from the adjacent CTA's shared memory
-// (distributed shared memory, through a table of per-plane addresses).
-// Phases, separated by the cluster's hardware barrier (release / acquire):
+// The V-cycle from the 32-interval level down on one thread-block cluster of C
+// CTAs per set.  CTA r owns the planes k0 .. k1-1 of that level; two threads
+// hold a row (j, k), 16 nodes each, and its right-hand side in registers for the
+// whole V-cycle, as Row does on the levels under it: odd i in O, even i in E,
+// the neighbour across the middle of the row by a shuffle, rows with j + k even
+// (s = 0) in the first half of the threads and the others in the second.
+// Neighbouring rows come from an exchange array in shared memory, which holds the
+// slab's planes and one more on each side; a thread whose plane borders another
+// CTA's slab also stores its new values into that CTA's copy (distributed shared
+// memory), so that every read is local.  Phases, separated by the cluster's
+// hardware barrier (release / acquire):
 //   npre (red, black) half-sweeps;
-//   full weighting of the red residuals, written straight into CTA 0's
-//   arrays of the 16-interval level;
+//   the red residuals, the first plane's also into the CTA below; then their full
+//   weighting, written straight into CTA 0's arrays of the 16-interval level;
 //   one V-cycle of the levels 16 .. 2 in CTA 0 (sm_vcycle, as coarse_run);
-//   the trilinear correction of the black nodes, read from CTA 0;
+//   the trilinear correction of the black nodes, from a copy of CTA 0's planes;
 //   npost (red, black) half-sweeps;
-// then each CTA writes its interior nodes back.  The arithmetic of every
-// node is that of the per-step kernels (rb_half4_kernel, restrict_node,
-// coarse_run, prolong_node) in the same order, with the same constants, so
-// the result is the same bits; the 32-interval level costs one launch and
-// no global traffic between its phases.
+// then the rows go back to global memory.  The arithmetic of every node is that
+// of the per-step kernels (rb_half4_kernel, restrict_node, coarse_run,
+// prolong_node) in the same order, with the same constants, so the result is the
+// same bits.  Bound by latencies: each phase is a few shared-memory reads, a
+// short chain of sums and the cluster's barrier.  Measured with C = 8:
+// 19.5 us a launch, 24.3 with a node at a time read from shared memory (and from
+// the neighbouring CTA's).
 constexpr int kSlabN = 32;
 constexpr int kSlabP = kSlabN + 1;
 constexpr int kSlabM = ((kSlabN / 2 + 1) + 3) & ~3;  // row length of the colour-split layout (make_view)
-constexpr int kSlabColour = kSlabP * kSlabM;         // floats of one colour of one plane
-constexpr int kSlabPlane = 2 * kSlabColour;          // floats of one plane, both colours
-constexpr int kSlabThreads = 512;
-constexpr int kSlabCoarseP = kSlabN / 2 + 1;  // 17: natural layout of CTA 0's 16-interval arrays
+constexpr int kSlabCoarseP = kSlabN / 2 + 1;         // 17: natural layout of CTA 0's 16-interval arrays
+constexpr int kSlabRow = kSlabP + 1;                 // rows of a plane in the exchange (one of padding)
+constexpr int kSlabRes = 20;                         // floats of a row of red residuals (16 and padding)
 
-__host__ __device__ inline int slab_depth(int csize) { return (kSlabN - 1 + csize - 1) / csize; }
+__host__ __device__ inline int slab_depth(int csize) { return (kSlabN - 1 + csize - 1) / csize; }  // 8, 4, 2: even
+// threads of the rows of one s (31 rows in two planes, two threads a row), and of the block (CTA 0 runs Row<16>)
+__host__ __device__ inline int slab_half(int csize) { return (slab_depth(csize) * (kSlabN - 1) + 31) / 32 * 32; }
+__host__ __device__ inline int slab_threads(int csize)
+{
+    const int t = 2 * slab_half(csize), c = 2 * Row<float, 16>::HALF;
+    return t > c ? t : c;
+}
+// vectors of four nodes of one half of the rows in the exchange: [vector][parity of i][plane][row]; the other half
+// lies four vectors past a multiple of 128 bytes from it, so that the two threads of a row meet different banks
+__host__ __device__ inline int slab_half_vecs(int csize) { return 4 * (slab_depth(csize) + 2) * kSlabRow + 4; }
 
 struct SlabArgs {
     float* e;  // the 32-interval level (set 0; set s at + 2 s cs)
@@ -1504,11 +1518,12 @@ struct SlabArgs {
     const SolveState* act;
 };
 
-__device__ __forceinline__ float* cluster_map(float* p, int rank)
+template <class T>
+__device__ __forceinline__ T* cluster_map(T* p, int rank)
 {
     unsigned long long out;
     asm volatile("mapa.u64 %0, %1, %2;" : "=l"(out) : "l"(reinterpret_cast<unsigned long long>(p)), "r"(rank));
-    return reinterpret_cast<float*>(out);
+    return reinterpret_cast<T*>(out);
 }
 
 __device__ __forceinline__ unsigned cluster_rank()
@@ -1518,203 +1533,292 @@ __device__ __forceinline__ unsigned cluster_rank()
     return r;
 }
 
-// One half-sweep of `colour` over the slab's planes (per-node arithmetic of
-// rb_half4_kernel: (x pair) + (y pair) + (z pair), then (sum - h2 f) / 6).
-template <bool ZERO>
-__device__ __forceinline__ void slab_rb(float* const* pe, const float* const* pf, int k0, int k1, int colour,
-                                        float h2, float sixth)
-{
-    const int tot = (k1 - k0) * (kSlabN - 1) * (kSlabN / 2);
-    for (int t = threadIdx.x; t < tot; t += kSlabThreads) {
-        const int m = t & (kSlabN / 2 - 1);
-        const int r = t >> 4;
-        const int j = r % (kSlabN - 1) + 1, k = k0 + r / (kSlabN - 1);
-        const int p = (colour + j + k) & 1;
-        if (p == 0 && m == 0) continue;  // i = 0 is a boundary node
-        const int row = j * kSlabM;
-        float sum = 0.0f;
-        if (!ZERO) {
-            const int oc = (colour ^ 1) * kSlabColour + row;
-            const float* o = pe[k] + oc;
-            const float lo = o[m - 1 + p], hi = o[m + p];
-            const float y0 = o[m - kSlabM], y1 = o[m + kSlabM];
-            const float z0 = pe[k - 1][oc + m], z1 = pe[k + 1][oc + m];
-            sum = (lo + hi) + (y0 + y1) + (z0 + z1);
+using Vec4 = RowVec<float>;
+
+// Half a row of the 32-interval level: nodes i = 16 half + 1 .. 16 half + 16.
+struct SlabRow {
+    int s, j, k, half;
+    bool on;
+    float O[8], E[8], eL;  // odd i; even i (the last one of the second half is the boundary node 32); i = 0
+    float fO[8], fE[8];
+    Vec4* x;               // the row's first vector in the exchange, and its neighbours' (other rows of the same half)
+    int stride;            // vectors between [vector][parity] parts
+    int yp, ym, zp, zm;
+    Vec4* push;            // the row in the exchange of the CTA that its plane borders, or null
+
+    template <bool EVEN>
+    __device__ __forceinline__ void put(bool remote)
+    {
+        const float* a = EVEN ? E : O;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            Vec4 w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w.v[e] = a[4 * v + e];
+            x[(v * 2 + EVEN) * stride] = w;
+            if (remote && push) push[(v * 2 + EVEN) * stride] = w;
         }
-        const float fv = pf[k][colour * kSlabColour + row + m];
-        pe[k][colour * kSlabColour + row + m] = (sum - h2 * fv) * sixth;
     }
-}
+    // sums of the six neighbours of the nodes of one parity of i (the whole warp takes part)
+    template <bool EVEN>
+    __device__ __forceinline__ void sums(float (&sum)[8]) const
+    {
+        const float across = EVEN ? __shfl_down_sync(0xffffffffu, O[0], 1) : __shfl_up_sync(0xffffffffu, E[7], 1);
+        const float left0 = half ? across : eL;  // of O[0]
+        if (!on) return;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const Vec4* p = x + (v * 2 + EVEN) * stride;
+            const Vec4 a = p[ym], b = p[yp], c = p[zm], d = p[zp];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int q = 4 * v + e;
+                const float lo = EVEN ? O[q] : (q == 0 ? left0 : E[q == 0 ? 0 : q - 1]);
+                const float hi = EVEN ? (q == 7 ? across : O[q == 7 ? 0 : q + 1]) : E[q];
+                sum[q] = (lo + hi) + (a.v[e] + b.v[e]) + (c.v[e] + d.v[e]);
+            }
+        }
+    }
+    template <bool EVEN, bool ZERO>
+    __device__ __forceinline__ void relax_own(float h2, float sixth, bool remote)
+    {
+        float sum[8];
+        if (ZERO) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) sum[q] = 0.0f;
+        } else {
+            sums<EVEN>(sum);
+        }
+        if (!on) return;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float w = fused(-h2, EVEN ? fE[q] : fO[q], sum[q]) * sixth;
+            if (!EVEN) O[q] = w;
+            else if (q < 7 || half == 0) E[q] = w;  // not the boundary node
+        }
+        put<EVEN>(remote);
+    }
+    template <bool ZERO>
+    __device__ __forceinline__ void relax(int colour, float h2, float sixth, bool remote)
+    {
+        if ((s ^ colour) == 0) relax_own<true, ZERO>(h2, sixth, remote);
+        else relax_own<false, ZERO>(h2, sixth, remote);
+    }
+    // red residuals of the half row (s = 0: even i, s = 1: odd i)
+    template <bool EVEN>
+    __device__ __forceinline__ void residual(float ih2, float* to, float* remote) const
+    {
+        float sum[8];
+        sums<EVEN>(sum);
+        if (!on) return;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            Vec4 w;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int q = 4 * v + e;
+                w.v[e] = fused(-fused(-6.0f, EVEN ? E[q] : O[q], sum[q]), ih2, EVEN ? fE[q] : fO[q]);
+            }
+            reinterpret_cast<Vec4*>(to)[v] = w;
+            if (remote) reinterpret_cast<Vec4*>(remote)[v] = w;
+        }
+    }
+    // the correction of the black nodes (prolong_node's sums) from the natural coarse array c
+    __device__ __forceinline__ void correct(const float* c)
+    {
+        if (!on) return;
+        constexpr int PC = kSlabCoarseP;
+        const int J0 = j >> 1, J1 = (j + 1) >> 1, K0 = k >> 1, K1 = (k + 1) >> 1, I = 8 * half;
+        const float* c00 = c + I + PC * (J0 + PC * K0);
+        const float* c10 = c + I + PC * (J1 + PC * K0);
+        const float* c01 = c + I + PC * (J0 + PC * K1);
+        const float* c11 = c + I + PC * (J1 + PC * K1);
+        if (s == 0) {  // odd i, between I + q and I + q + 1
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float t = (c00[q] + c00[q + 1]) + (c10[q] + c10[q + 1]);
+                t += (c01[q] + c01[q + 1]) + (c11[q] + c11[q + 1]);
+                t *= 0.125f;
+                O[q] = O[q] + t;
+            }
+            put<false>(true);
+        } else {  // even i, on I + q + 1
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (q == 7 && half) break;
+                float t = (c00[q + 1] + c00[q + 1]) + (c10[q + 1] + c10[q + 1]);
+                t += (c01[q + 1] + c01[q + 1]) + (c11[q + 1] + c11[q + 1]);
+                t *= 0.125f;
+                E[q] = E[q] + t;
+            }
+            put<true>(true);
+        }
+    }
+};
 
-// red_residual on the slab tables
-__device__ __forceinline__ float slab_red_residual(float* const* pe, const float* const* pf, int i, int j, int k,
-                                                   float ih2)
-{
-    const int p = (j + k) & 1;
-    const int m = i >> 1;
-    const int row = j * kSlabM;
-    const float* eb = pe[k] + kSlabColour + row;
-    const float s = (eb[m - 1 + p] + eb[m + p]) + (eb[m - kSlabM] + eb[m + kSlabM]) +
-                    (pe[k - 1][kSlabColour + row + m] + pe[k + 1][kSlabColour + row + m]);
-    return pf[k][row + m] - (s - 6.0f * pe[k][row + m]) * ih2;
-}
-
-__global__ void __launch_bounds__(kSlabThreads) vslab_kernel(SlabArgs a)
+// THREADS: 512 (clusters of 4) or 256
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) vslab_kernel(SlabArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int C = a.csize;
     const int set = (int)blockIdx.x / C;
     const int rank = (int)cluster_rank();
     if (a.act && !a.act[set].cont) return;  // the whole cluster reads the same flag
-    const int q = slab_depth(C);
-    const int k0 = 1 + rank * q;
-    const int k1 = min(kSlabN, k0 + q);
-    float* se = reinterpret_cast<float*>(smem_raw);  // slot s holds plane k0 - 1 + s
-    float* sf = se + (size_t)(q + 2) * kSlabPlane;   // slot s holds plane k0 + s
-    float** pe = reinterpret_cast<float**>(sf + (size_t)q * kSlabPlane);
-    float** pf = pe + 40;
-    unsigned char* coarse_raw = reinterpret_cast<unsigned char*>(pf + 40);
+    const int q = slab_depth(C), slots = q + 2;  // slot p of the exchange holds plane k0 - 1 + p
+    const int k0 = 1 + rank * q, k1 = min(kSlabN, k0 + q);
+    const int t = (int)threadIdx.x, T = (int)blockDim.x;
+    Vec4* const ex = reinterpret_cast<Vec4*>(smem_raw);
+    const int half_vecs = slab_half_vecs(C);
+    float* const rr = reinterpret_cast<float*>(ex + 2 * half_vecs);  // red residuals of planes k0 .. k1
     CoarseSmem<float> S;
-    coarse_layout(S, reinterpret_cast<float*>(coarse_raw), 3);
+    coarse_layout(S, rr + (q + 1) * kSlabP * kSlabRes, 3);
     float* const e = a.e + (long long)set * 2 * a.cs;
     const float* const f = a.f + (long long)set * 2 * a.cs;
     constexpr int kC3 = kSlabCoarseP * kSlabCoarseP * kSlabCoarseP;
 
-    // plane tables: plane k of e lives in the CTA that owns it (plane 0 in CTA 0, plane 32 in CTA C-1)
-    if (threadIdx.x <= kSlabN) {
-        const int k = threadIdx.x;
-        const int owner = k == 0 ? 0 : (k == kSlabN ? C - 1 : (k - 1) / q);
-        const int slot = k - (1 + owner * q) + 1;
-        float* local = se + (size_t)slot * kSlabPlane;
-        pe[k] = owner == rank ? local : cluster_map(local, owner);
-        if (k >= 1 && k < kSlabN) {
-            float* lf = sf + (size_t)(k - (1 + owner * q)) * kSlabPlane;
-            pf[k] = owner == rank ? lf : cluster_map(lf, owner);
-        }
-    }
-    // own planes of f (and of e unless the correction starts from zero), and the boundary planes held here
+    // where a row lies in the exchange, from the first vector of its half: even j first, then odd j, so that the rows
+    // of a warp (every other j) lie next to each other
+    auto place = [&](int k, int j) { return (k - (k0 - 1)) * kSlabRow + (j >> 1) + (j & 1) * (kSlabN / 2 + 1); };
+    const int stride = slots * kSlabRow;
+
+    SlabRow row;
     {
-        const int kb = (rank == 0) ? 0 : k0;
-        const int ke = (rank == C - 1) ? kSlabN + 1 : k1;
-        const int n4 = kSlabColour / 4;  // float4 per colour-plane
-        for (int t = threadIdx.x; t < (k1 - k0) * 2 * n4; t += kSlabThreads) {
-            const int kk = t / (2 * n4), c = (t / n4) & 1, x = t % n4;
-            const float4* src = reinterpret_cast<const float4*>(f + (long long)c * a.cs +
-                                                                (long long)(k0 + kk) * kSlabColour);
-            reinterpret_cast<float4*>(sf + (size_t)kk * kSlabPlane + c * kSlabColour)[x] = src[x];
-        }
-        for (int t = threadIdx.x; t < (ke - kb) * 2 * n4; t += kSlabThreads) {
-            const int kk = t / (2 * n4), c = (t / n4) & 1, x = t % n4;
-            const int k = kb + kk;
-            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (!a.zero_top)
-                v = reinterpret_cast<const float4*>(e + (long long)c * a.cs + (long long)k * kSlabColour)[x];
-            reinterpret_cast<float4*>(se + (size_t)(k - k0 + 1) * kSlabPlane + c * kSlabColour)[x] = v;
-        }
-        if (rank == 0) {  // coarse_run with a zero start: u = 0, f = 0 off the interior
-            for (int t = threadIdx.x; t < kC3; t += kSlabThreads) {
-                S.u[3][t] = 0.0f;
-                S.f[3][t] = 0.0f;
+        const int halft = slab_half(C);
+        row.s = t >= halft ? 1 : 0;
+        const int g = t - row.s * halft, r = g >> 1;
+        row.half = g & 1;
+        // planes in pairs (k0 is odd): for s = 0 the first has the 16 odd j and the second the 15 even ones; for s = 1
+        // the reverse
+        const int pr = r / (kSlabN - 1), m = r - pr * (kSlabN - 1), first = row.s ? kSlabN / 2 - 1 : kSlabN / 2;
+        row.k = k0 + 2 * pr + (m >= first ? 1 : 0);
+        row.j = m < first ? 2 * m + (row.s ? 2 : 1) : 2 * (m - first) + (row.s ? 1 : 2);
+        row.on = t < 2 * halft && row.k < k1;
+        if (!row.on) row.k = k0, row.j = 1;  // any row: nothing of it is used
+        Vec4* const base = ex + row.half * half_vecs;
+        row.x = base + place(row.k, row.j);
+        row.stride = stride;
+        row.yp = place(row.k, row.j + 1) - place(row.k, row.j);
+        row.ym = place(row.k, row.j - 1) - place(row.k, row.j);
+        row.zp = kSlabRow;
+        row.zm = -kSlabRow;
+        // the plane's place in the neighbouring CTA: slot q + 1 of the one below, slot 0 of the one above
+        row.push = nullptr;
+        const int in_plane = place(k0 - 1, row.j);
+        if (row.on && row.k == k0 && rank > 0) row.push = cluster_map(base + (q + 1) * kSlabRow + in_plane, rank - 1);
+        else if (row.on && row.k == k1 - 1 && rank < C - 1) row.push = cluster_map(base + in_plane, rank + 1);
+        // with one plane a slab (the last of 16) both sides would border: it is the last, and has none above
+    }
+    // the row from global memory: even i = 2m at m of one colour, odd i = 2m + 1 of the other
+    const long long at = ((long long)row.k * kSlabP + row.j) * kSlabM + 8 * row.half;
+    const long long ev = (row.s ? a.cs : 0) + at, od = (row.s ? 0 : a.cs) + at;
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        row.fO[v] = f[od + v];
+        row.fE[v] = f[ev + v + 1];
+        row.O[v] = a.zero_top ? 0.0f : e[od + v];
+        row.E[v] = a.zero_top ? 0.0f : e[ev + v + 1];
+    }
+    row.eL = a.zero_top ? 0.0f : e[ev];
+    // the exchange: zeros, or the planes k0 - 1 .. k1 with their boundary rows
+    if (a.zero_top) {
+        const Vec4 z = {{0.0f, 0.0f, 0.0f, 0.0f}};
+        for (int p = t; p < 2 * half_vecs; p += T) ex[p] = z;
+    } else {
+        for (int p = t; p < (k1 - k0 + 2) * kSlabP * 2; p += T) {
+            const int half = p & 1, jr = (p >> 1) % kSlabP, kr = k0 - 1 + (p >> 1) / kSlabP, sr = (jr + kr) & 1;
+            const long long src = ((long long)kr * kSlabP + jr) * kSlabM + 8 * half;
+            const float* od_r = e + (sr ? 0 : a.cs) + src;
+            const float* ev_r = e + (sr ? a.cs : 0) + src;
+            Vec4* to = ex + half * half_vecs + place(kr, jr);
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                Vec4 o, w;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) o.v[c] = od_r[4 * v + c], w.v[c] = ev_r[4 * v + c + 1];
+                to[(v * 2) * stride] = o;
+                to[(v * 2 + 1) * stride] = w;
             }
-            clear_rows<float, 3>(S);
         }
     }
-    __syncthreads();
+    if (rank == 0) {  // as coarse_run with a zero start: zeros off the interior
+        for (int p = t; p < kC3; p += T) S.u[3][p] = 0.0f;
+        clear_rows<float, 3>(S);
+    }
     cluster_sync_all();
 
     // pre-smoothing
-    for (int qq = 0; qq < a.npre; ++qq) {
-        if (qq == 0 && a.zero_top)
-            slab_rb<true>(pe, pf, k0, k1, 0, a.h2, a.sixth);
-        else
-            slab_rb<false>(pe, pf, k0, k1, 0, a.h2, a.sixth);
+    for (int v = 0; v < a.npre; ++v) {
+        if (v == 0 && a.zero_top) row.relax<true>(0, a.h2, a.sixth, true);
+        else row.relax<false>(0, a.h2, a.sixth, true);
         cluster_sync_all();
-        slab_rb<false>(pe, pf, k0, k1, 1, a.h2, a.sixth);
+        row.relax<false>(1, a.h2, a.sixth, true);
         cluster_sync_all();
     }
-    // restriction of the red residuals onto the coarse planes K with 2K in this slab
+    // the red residuals; plane k0's are needed by the CTA below too, as its plane k1
+    {
+        float* to = rr + ((row.k - k0) * kSlabP + row.j) * kSlabRes + 8 * row.half;
+        float* remote = row.on && row.k == k0 && rank > 0
+                            ? cluster_map(rr + (q * kSlabP + row.j) * kSlabRes + 8 * row.half, rank - 1)
+                            : nullptr;
+        if (row.s == 0) row.residual<true>(a.ih2, to, remote);
+        else row.residual<false>(a.ih2, to, remote);
+    }
+    cluster_sync_all();
+    // their full weighting onto the coarse planes K with 2K in this slab (restrict_node's sums)
     {
         float* fc = rank == 0 ? S.f[3] : cluster_map(S.f[3], 0);
         const int K0 = (k0 + 1) >> 1, K1 = (k1 + 1) >> 1;  // 2K in [k0, k1)
         constexpr int MC = kSlabN / 2 - 1;
-        const int tot = (K1 - K0) * MC * MC;
-        for (int t = threadIdx.x; t < tot; t += kSlabThreads) {
-            const int I = t % MC + 1, J = (t / MC) % MC + 1, K = K0 + t / (MC * MC);
-            const int i = 2 * I, j = 2 * J, k = 2 * K;
-            const float ih2 = a.ih2;
-            float edge = (slab_red_residual(pe, pf, i + 1, j + 1, k, ih2) + slab_red_residual(pe, pf, i - 1, j + 1, k, ih2))
-                       + (slab_red_residual(pe, pf, i + 1, j - 1, k, ih2) + slab_red_residual(pe, pf, i - 1, j - 1, k, ih2));
-            edge += (slab_red_residual(pe, pf, i + 1, j, k + 1, ih2) + slab_red_residual(pe, pf, i - 1, j, k + 1, ih2))
-                  + (slab_red_residual(pe, pf, i + 1, j, k - 1, ih2) + slab_red_residual(pe, pf, i - 1, j, k - 1, ih2));
-            edge += (slab_red_residual(pe, pf, i, j + 1, k + 1, ih2) + slab_red_residual(pe, pf, i, j - 1, k + 1, ih2))
-                  + (slab_red_residual(pe, pf, i, j + 1, k - 1, ih2) + slab_red_residual(pe, pf, i, j - 1, k - 1, ih2));
-            const float centre = slab_red_residual(pe, pf, i, j, k, ih2);
+        for (int p = t; p < (K1 - K0) * MC * MC; p += T) {
+            const int I = p % MC + 1, J = (p / MC) % MC + 1, K = K0 + p / (MC * MC);
+            // rows j - 1, j, j + 1 of planes k - 1, k, k + 1 at node i = 2I: odd i = 2I -+ 1 at I - 1 and I, even at I - 1
+            const float* r0 = rr + ((2 * K - k0) * kSlabP + 2 * J) * kSlabRes + I - 1;
+            const float* rm = r0 - kSlabP * kSlabRes;
+            const float* rp = r0 + kSlabP * kSlabRes;
+            float edge = (r0[kSlabRes + 1] + r0[kSlabRes]) + (r0[-kSlabRes + 1] + r0[-kSlabRes]);
+            edge += (rp[1] + rp[0]) + (rm[1] + rm[0]);
+            edge += (rp[kSlabRes] + rp[-kSlabRes]) + (rm[kSlabRes] + rm[-kSlabRes]);
+            const float centre = r0[0];
             fc[I + kSlabCoarseP * (J + kSlabCoarseP * K)] = 0.125f * centre + 0.03125f * edge;
         }
     }
     cluster_sync_all();
     if (rank == 0) sm_vcycle<float, 3, true>(S, a.hc, a.npre, a.npost);
     cluster_sync_all();
-    // coarse-grid correction of the black nodes (prolong_node's sums in its order); the coarse planes
-    // k0/2 .. k1/2 that this slab interpolates from are first copied from CTA 0 into the same place of
-    // this CTA's (otherwise unused) coarse arrays, so that CTA 0's shared memory is read once per value
-    {
-        if (rank != 0) {
-            const float* src = cluster_map(S.u[3], 0);
-            const int lo = (k0 >> 1) * kSlabCoarseP * kSlabCoarseP;
-            const int hi = ((k1 >> 1) + 1) * kSlabCoarseP * kSlabCoarseP;
-            for (int t = lo + threadIdx.x; t < hi; t += 4 * kSlabThreads) {
-                float v[4];
+    // coarse-grid correction; the coarse planes k0/2 .. k1/2 that this slab interpolates from are first copied from
+    // CTA 0 into the same place of this CTA's (otherwise unused) coarse arrays, so that CTA 0's shared memory is read
+    // once per value
+    if (rank != 0) {
+        const float* src = cluster_map(S.u[3], 0);
+        const int lo = (k0 >> 1) * kSlabCoarseP * kSlabCoarseP;
+        const int hi = ((k1 >> 1) + 1) * kSlabCoarseP * kSlabCoarseP;
+        for (int p = lo + t; p < hi; p += 4 * T) {
+            float v[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (t + u * kSlabThreads < hi) v[u] = src[t + u * kSlabThreads];
+            for (int u = 0; u < 4; ++u)
+                if (p + u * T < hi) v[u] = src[p + u * T];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (t + u * kSlabThreads < hi) S.u[3][t + u * kSlabThreads] = v[u];
-            }
-            __syncthreads();
+            for (int u = 0; u < 4; ++u)
+                if (p + u * T < hi) S.u[3][p + u * T] = v[u];
         }
-        const float* ec = S.u[3];
-        const int tot = (k1 - k0) * (kSlabN - 1) * (kSlabN / 2);
-        for (int t = threadIdx.x; t < tot; t += kSlabThreads) {
-            const int m = t & (kSlabN / 2 - 1);
-            const int r = t >> 4;
-            const int j = r % (kSlabN - 1) + 1, k = k0 + r / (kSlabN - 1);
-            const int p = (1 + j + k) & 1;
-            const int i = 2 * m + p;
-            if (i < 1) continue;
-            const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1, K0 = k >> 1, K1 = (k + 1) >> 1;
-            constexpr int PC = kSlabCoarseP;
-            float s = (ec[I0 + PC * (J0 + PC * K0)] + ec[I1 + PC * (J0 + PC * K0)])
-                    + (ec[I0 + PC * (J1 + PC * K0)] + ec[I1 + PC * (J1 + PC * K0)]);
-            s += (ec[I0 + PC * (J0 + PC * K1)] + ec[I1 + PC * (J0 + PC * K1)])
-               + (ec[I0 + PC * (J1 + PC * K1)] + ec[I1 + PC * (J1 + PC * K1)]);
-            s *= 0.125f;
-            float* o = pe[k] + kSlabColour + j * kSlabM + m;
-            *o = *o + s;
-        }
+        __syncthreads();
     }
+    row.correct(S.u[3]);
     cluster_sync_all();
-    // post-smoothing
-    for (int qq = 0; qq < a.npost; ++qq) {
-        slab_rb<false>(pe, pf, k0, k1, 0, a.h2, a.sixth);
+    // post-smoothing; no CTA reads the last black values from the exchange, nor another CTA's after the last barrier
+    for (int v = 0; v < a.npost; ++v) {
+        row.relax<false>(0, a.h2, a.sixth, true);
         cluster_sync_all();
-        slab_rb<false>(pe, pf, k0, k1, 1, a.h2, a.sixth);
-        cluster_sync_all();  // also: no CTA leaves while a neighbour still reads its planes
+        const bool last = v == a.npost - 1;
+        row.relax<false>(1, a.h2, a.sixth, !last);
+        if (!last) cluster_sync_all();
     }
-    // the interior nodes of this slab back to global memory
-    {
-        const int tot = (k1 - k0) * 2 * (kSlabN - 1) * (kSlabN / 2);
-        for (int t = threadIdx.x; t < tot; t += kSlabThreads) {
-            const int m = t & (kSlabN / 2 - 1);
-            const int r = t >> 4;
-            const int j = r % (kSlabN - 1) + 1;
-            const int r2 = r / (kSlabN - 1);
-            const int c = r2 & 1, k = k0 + (r2 >> 1);
-            const int p = (c + j + k) & 1;
-            if (p == 0 && m == 0) continue;
-            const int o = c * kSlabColour + j * kSlabM + m;
-            e[(long long)c * a.cs + (long long)k * kSlabColour + j * kSlabM + m] = se[(size_t)(k - k0 + 1) * kSlabPlane + o];
+    if (row.on) {
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            e[od + v] = row.O[v];
+            if (v < 7 || row.half == 0) e[ev + v + 1] = row.E[v];
         }
     }
 }
@@ -1990,13 +2094,11 @@ size_t coarse_smem_bytes(int n)
     return tot * sizeof(T);
 }
 
-// shared memory of the slab V-cycle kernel: e planes (slab + 2), f planes
-// (slab), the two plane tables, and CTA 0's arrays of the levels 16 .. 2
+// shared memory of the slab V-cycle kernel: the exchange, the red residuals, and CTA 0's arrays of the levels 16 .. 2
 inline size_t slab_smem_bytes(int csize)
 {
-    const int q = slab_depth(csize);
-    return sizeof(float) * (size_t)kSlabPlane * (size_t)(2 * q + 2) + 2 * 40 * sizeof(float*) +
-           coarse_smem_bytes<float>(kSlabN / 2);
+    return sizeof(Vec4) * 2 * (size_t)slab_half_vecs(csize) +
+           sizeof(float) * (size_t)((slab_depth(csize) + 1) * kSlabP * kSlabRes) + coarse_smem_bytes<float>(kSlabN / 2);
 }
 
 }  // namespace
@@ -2248,7 +2350,7 @@ cudaError_t launch_vslab(float* e, const float* f, const LevelView& v, double h,
     a.act = sets.act;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(csize * sets.n));
-    cfg.blockDim = dim3(kSlabThreads);
+    cfg.blockDim = dim3((unsigned)slab_threads(csize));
     cfg.dynamicSmemBytes = slab_smem_bytes(csize);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -2258,7 +2360,8 @@ cudaError_t launch_vslab(float* e, const float* f, const LevelView& v, double h,
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, vslab_kernel, a);
+    return slab_threads(csize) > 256 ? cudaLaunchKernelEx(&cfg, vslab_kernel<512>, a)
+                                     : cudaLaunchKernelEx(&cfg, vslab_kernel<256>, a);
 }
 
 int vslab_size(int want)
@@ -2267,7 +2370,7 @@ int vslab_size(int want)
     if (!(want == 4 || want == 8 || want == 16)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)want);
-    cfg.blockDim = dim3(kSlabThreads);
+    cfg.blockDim = dim3((unsigned)slab_threads(want));
     cfg.dynamicSmemBytes = slab_smem_bytes(want);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2277,7 +2380,9 @@ int vslab_size(int want)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, vslab_kernel, &cfg) == cudaSuccess && n >= 1) return want;
+    const cudaError_t err = slab_threads(want) > 256 ? cudaOccupancyMaxActiveClusters(&n, vslab_kernel<512>, &cfg)
+                                                     : cudaOccupancyMaxActiveClusters(&n, vslab_kernel<256>, &cfg);
+    if (err == cudaSuccess && n >= 1) return want;
     (void)cudaGetLastError();
     return 0;
 }
@@ -2370,9 +2475,11 @@ cudaError_t prepare_kernels()
         cudaFuncSetAttribute(vcluster_kernel<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
             cudaSuccess)
         return cudaGetLastError();
-    if (cudaFuncSetAttribute(vslab_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)slab_smem_bytes(4)) !=
+    if (cudaFuncSetAttribute(vslab_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)slab_smem_bytes(4)) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(vslab_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaFuncSetAttribute(vslab_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)slab_smem_bytes(8)) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(vslab_kernel<256>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return cudaGetLastError();
     cudaError_t e = cudaFuncSetAttribute(coarse_kernel<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)coarse_smem_bytes<float>(kCoarseN));
