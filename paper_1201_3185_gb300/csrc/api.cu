@@ -549,7 +549,7 @@ void check(qumond_ctx* c, int box, const double* rhs, double coef, const double*
         });
     } else {
         run(c, K_RESIDUAL_OUTER, cube(p.n) * (16.0 + sizeof(T)), s, [&] {
-            launch_residual_rows<T>(u, rhs, coef, p.n, box_h(c, box), F<T>(c, c->L), c->lev[c->L].v, c->partials, s,
+            launch_residual_rows<T>(u, rhs, coef, p.n, box_h(c, box), first, F<T>(c, c->L), c->lev[c->L].v, c->partials, s,
                                     sets_of(c));
         });
     }

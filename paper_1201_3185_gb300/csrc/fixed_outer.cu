@@ -60,9 +60,8 @@ __device__ __forceinline__ long long f32_to_i64(float v)
     return (bits >> 31) ? -m : m;
 }
 
-// 2^e as FP32 / FP64 from an integer exponent.
+// 2^e as FP32 from an integer exponent.
 __device__ __forceinline__ float pow2f(int e) { return ldexpf(1.0f, e); }
-__device__ __forceinline__ double pow2d(int e) { return ldexp(1.0, e); }
 
 constexpr int kThreads = 128;
 constexpr int kMaxBlocks = 152 * 16;
@@ -169,14 +168,13 @@ fixed_init_pairs_kernel(const float* __restrict__ e, LevelView v, const double* 
         U += fs, U2 += fs, F += fs;
     }
     const int pairs = n / 2 + 1;
-    const long long idx = blockIdx.x * 256LL + threadIdx.x;
-    if (idx >= (long long)pairs * (n + 1) * (n + 1)) return;
-    const int row = (int)(idx / pairs), a = (int)(idx - (long long)row * pairs);
-    const int j = row % (n + 1), k = row / (n + 1);
+    const unsigned idx = blockIdx.x * 256u + threadIdx.x;  // below 2^30 for n <= 1024
+    const unsigned row = idx / (unsigned)pairs;
+    const int a = (int)(idx - row * (unsigned)pairs);
+    const int k = (int)(row / (unsigned)(n + 1)), j = (int)(row - (unsigned)k * (unsigned)(n + 1));
+    if (k > n) return;
     const int S = st->scale_exp;
-    const double sc = pow2d(S);
     const float scf = pow2f(S);
-    const double kf = coef_h2 * sc;
     const bool brow = j == 0 || j == n || k == 0 || k == n;
     const int i0 = 2 * a;
     const bool has1 = i0 + 1 <= n;
@@ -184,15 +182,17 @@ fixed_init_pairs_kernel(const float* __restrict__ e, LevelView v, const double* 
     const long long o = nat(n, i0, j, k), of = fix(n, i0, j, k);
     const int c0 = (i0 + j + k) & 1;
     const long long er = ((long long)k * (n + 1) + j) * v.M + a;  // entry of both nodes in their colour rows
-    // FP64 -> int64 on the integer pipe (round to nearest even, as the FP64 conversion instruction)
-    const long long v0 = (b0 || from_u64) ? f64_to_i64_rn(u64[o] * sc) : f32_to_i64(e[(long long)c0 * v.cs + er] * scf);
-    long long v1 = 0, f1 = 0;
-    if (has1) {
-        v1 = (b1 || from_u64) ? f64_to_i64_rn(u64[o + 1] * sc) : f32_to_i64(e[(long long)(c0 ^ 1) * v.cs + er] * scf);
-        f1 = b1 ? 0LL : f64_to_i64_rn(rhs[o + 1] * kf);
-    }
-    const long long f0 = b0 ? 0LL : f64_to_i64_rn(rhs[o] * kf);
-    if ((!b0 && f64_nonfinite(rhs[o])) || (has1 && !b1 && f64_nonfinite(rhs[o + 1]))) st->nonfinite = 1;
+    // FP64 -> int64 on the integer pipe (round to nearest even, as the FP64 conversion instruction); the FP64 pipe does
+    // one product a node
+    const double r0 = b0 ? 0.0 : rhs[o], r1 = has1 && !b1 ? rhs[o + 1] : 0.0;
+    const long long v0 =
+        (b0 || from_u64) ? f64_to_i64_rn_scaled(u64[o], S) : f32_to_i64(e[(long long)c0 * v.cs + er] * scf);
+    long long v1 = 0;
+    if (has1)
+        v1 = (b1 || from_u64) ? f64_to_i64_rn_scaled(u64[o + 1], S)
+                              : f32_to_i64(e[(long long)(c0 ^ 1) * v.cs + er] * scf);
+    const long long f0 = f64_to_i64_rn_scaled(r0 * coef_h2, S), f1 = f64_to_i64_rn_scaled(r1 * coef_h2, S);
+    if (f64_nonfinite(r0) || f64_nonfinite(r1)) st->nonfinite = 1;
     *reinterpret_cast<longlong2*>(U + of) = make_longlong2(v0, v1);
     *reinterpret_cast<longlong2*>(F + of) = make_longlong2(f0, f1);
     // the second buffer's interior is written before it is read
@@ -225,15 +225,14 @@ fixed_residual_kernel(const long long* __restrict__ U, const long long* __restri
     }
     const long long P = n + 2, Q = P * (n + 1);
     const float k = pow2f(-st->scale_exp) * ih2;
-    const int half = n / 2;
-    const long long items = (long long)(n - 1) * (n - 1) * half;  // (row, pair)
+    const unsigned half = (unsigned)n / 2, lh = 31u - (unsigned)__clz((int)half);  // a power of two
+    const unsigned items = (unsigned)(n - 1) * (unsigned)(n - 1) * half;           // (row, pair), below 2^30
     float rr = 0.0f, ff = 0.0f;
     constexpr float kDown = 9.313225746154785e-10f;  // 2^-30
-    for (long long it = blockIdx.x * (long long)kThreads + threadIdx.x; it < items;
-         it += (long long)gridDim.x * kThreads) {
-        const int m = (int)(it % half);
-        const long long row = it / half;
-        const int j = (int)(row % (n - 1)) + 1, kk = (int)(row / (n - 1)) + 1;
+    for (unsigned it = blockIdx.x * (unsigned)kThreads + threadIdx.x; it < items; it += gridDim.x * (unsigned)kThreads) {
+        const int m = (int)(it & (half - 1));
+        const unsigned row = it >> lh, plane = row / (unsigned)(n - 1);
+        const int j = (int)(row - plane * (unsigned)(n - 1)) + 1, kk = (int)plane + 1;
         const int i = 2 * m;  // nodes i (i = 0 is a boundary node) and i + 1 (<= n - 1)
         const long long o = fix(n, i, j, kk);
         const longlong2 c = *reinterpret_cast<const longlong2*>(U + o);
@@ -421,7 +420,8 @@ fixed_update_residual_kernel(long long* Ua, long long* Ub, const long long* __re
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+// A pair of nodes (i = 2a, 2a + 1) per thread over a flat grid: one 16-byte load.
+__global__ void __launch_bounds__(256)
 fixed_output_kernel(const long long* Ua, const long long* Ub, double* __restrict__ u, int n,
                     const SolveState* __restrict__ st)
 {
@@ -434,12 +434,16 @@ fixed_output_kernel(const long long* Ua, const long long* Ub, double* __restrict
     }
     const long long* __restrict__ U = (st->it & 1) ? Ub : Ua;
     const int S = st->scale_exp;
-    const int rows = (n - 1) * (n - 1);
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int j = row % (n - 1) + 1, k = row / (n - 1) + 1;
-        // U 2^-S: int64 -> FP64 on the integer pipe (round to nearest even, then an exact power-of-two scale)
-        for (int i = threadIdx.x + 1; i < n; i += kThreads) u[nat(n, i, j, k)] = i64_to_f64_rn_scaled(U[fix(n, i, j, k)], -S);
-    }
+    const unsigned half = (unsigned)n / 2, lh = 31u - (unsigned)__clz((int)half);  // a power of two
+    const unsigned idx = blockIdx.x * 256u + threadIdx.x;
+    const unsigned row = idx >> lh, plane = row / (unsigned)(n - 1);
+    const int k = (int)plane + 1, j = (int)(row - plane * (unsigned)(n - 1)) + 1, i = 2 * (int)(idx & (half - 1));
+    if (k >= n) return;
+    // U 2^-S: int64 -> FP64 on the integer pipe (round to nearest even, then an exact power-of-two scale)
+    const longlong2 w = *reinterpret_cast<const longlong2*>(U + fix(n, i, j, k));
+    double* at = u + nat(n, i, j, k);
+    if (i > 0) at[0] = i64_to_f64_rn_scaled(w.x, -S);  // node 0 is a boundary node
+    at[1] = i64_to_f64_rn_scaled(w.y, -S);
 }
 
 inline int blocks_for_rows(long long rows) { return (int)(rows < kMaxBlocks ? rows : kMaxBlocks); }
@@ -501,7 +505,8 @@ int launch_fixed_residual(const int64_t* U, const int64_t* F, int n, double h, c
 void launch_fixed_output(const int64_t* U, const int64_t* U2, double* u, int n, const SolveState* st, cudaStream_t s,
                          const Sets& sets)
 {
-    fixed_output_kernel<<<dim3(fixed_residual_blocks(n), sets.n), kThreads, 0, s>>>(
+    const long long pairs = (long long)(n - 1) * (n - 1) * (n / 2);
+    fixed_output_kernel<<<dim3((unsigned)((pairs + 255) / 256), sets.n), 256, 0, s>>>(
         reinterpret_cast<const long long*>(U), reinterpret_cast<const long long*>(U2), u, n, st);
 }
 

@@ -159,36 +159,27 @@ __global__ void boundary_zero_kernel(double* __restrict__ u, int n)
     u[set * nat_elems(n) + nat(n, i, j, k)] = 0.0;
 }
 
-// Trilinear interpolation of a natural-layout grid at index coordinates t.
-__device__ __forceinline__ double trilinear_idx(const double* __restrict__ a, int n, double tx, double ty, double tz)
+// Exact FP32 -> FP64 with integer ops (subnormals flushed to zero).
+__device__ __forceinline__ double f32_to_f64(float f)
 {
-    const double t[3] = {tx, ty, tz};
-    int i0[3];
-    double d[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        int ii = (int)floor(t[q]);
-        ii = ii < 0 ? 0 : (ii > n - 1 ? n - 1 : ii);
-        i0[q] = ii;
-        d[q] = t[q] - (double)ii;
-    }
-    double v = 0.0;
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int a3 = 0; a3 < 2; ++a3) {
-                const double w = (a3 ? d[0] : 1.0 - d[0]) * (b ? d[1] : 1.0 - d[1]) * (c ? d[2] : 1.0 - d[2]);
-                v += w * a[nat(n, i0[0] + a3, i0[1] + b, i0[2] + c)];
-            }
-    return v;
+    const unsigned u = __float_as_uint(f);
+    const unsigned sign = u & 0x80000000u, e = u & 0x7f800000u;
+    unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20), lo = u << 29;
+    if (e == 0u) hi = 0u, lo = 0u;
+    if (e == 0x7f800000u) hi += 896u << 20;  // exponent 255 to 2047
+    return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
 // Boundary of a box from its parent (box_ratio times the side, same centre,
 // same n): child node i sits at parent index n (r-1)/(2r) + i/r along each
 // axis (Section 2: the parent solution is interpolated onto the child's
 // boundary).
+//
+// The ratio is a power of two, so the cell and the offsets 0, 1/r, .. (r-1)/r are
+// exact integers, and so are the weights, products of three of them over r^3:
+// they are formed on the integer and FP32 pipes, and the FP64 pipe, which bounds
+// the kernel, does the eight fused products.  6 faces of 257^2: about 13 us, 60
+// with the weights in FP64.
 __global__ void boundary_from_parent_kernel(const double* __restrict__ parent, double* __restrict__ u, int n, int ratio)
 {
     const int set = blockIdx.z / 6, face = blockIdx.z - 6 * set;  // blockIdx.z = 6 * set + face
@@ -198,9 +189,23 @@ __global__ void boundary_from_parent_kernel(const double* __restrict__ parent, d
     if (a > n) return;
     int i, j, k;
     face_node(face, a, b, n, i, j, k);
-    const double inv_r = 1.0 / (double)ratio;
-    const double q = 0.5 * (double)n * (1.0 - inv_r);
-    u[nat(n, i, j, k)] = trilinear_idx(parent, n, q + inv_r * i, q + inv_r * j, q + inv_r * k);
+    const int lr = 31 - __clz(ratio), q = (n >> 1) * (ratio - 1);  // child node 0 lies at q / r
+    const int t[3] = {q + i, q + j, q + k};
+    int i0[3], d[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) i0[x] = t[x] >> lr, d[x] = t[x] & (ratio - 1);
+    const float unit = __int_as_float((127 - 3 * lr) << 23);  // r^-3
+    double v = 0.0;
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const int w = (x ? d[0] : ratio - d[0]) * (y ? d[1] : ratio - d[1]) * (z ? d[2] : ratio - d[2]);
+                v = fma(f32_to_f64((float)w * unit), parent[nat(n, i0[0] + x, i0[1] + y, i0[2] + z)], v);
+            }
+    u[nat(n, i, j, k)] = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -252,17 +257,6 @@ __device__ __forceinline__ float2 split_hi_lo(double x)
     const float hi = __uint_as_float(sign | ((__funnelshift_l(l, h, 3) - (896u << 23)) & 0x7fffffffu));
     const float r = __uint2float_rn(l & 0x1FFFFFFFu);
     return make_float2(hi, r * __uint_as_float(sign | (((ex << 3) - (948u << 23)) & 0x7fffffffu)));
-}
-
-// Exact FP32 -> FP64 with integer ops (subnormals flushed to zero).
-__device__ __forceinline__ double f32_to_f64(float f)
-{
-    const unsigned u = __float_as_uint(f);
-    const unsigned sign = u & 0x80000000u, e = u & 0x7f800000u;
-    unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20), lo = u << 29;
-    if (e == 0u) hi = 0u, lo = 0u;
-    if (e == 0x7f800000u) hi += 896u << 20;  // exponent 255 to 2047
-    return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
 constexpr int kSrcX = 30;         // output columns of a warp: lanes 1 .. 30

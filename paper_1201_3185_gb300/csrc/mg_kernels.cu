@@ -13,6 +13,7 @@
 //  * right after a black half-sweep the black residuals are zero, so the
 //    residual to restrict is nonzero only at red nodes.
 #include "qumond_internal.h"
+#include "fixed_conv.h"
 
 #include <cstdio>
 
@@ -1831,6 +1832,12 @@ __device__ __forceinline__ long long nat(int n, int i, int j, int k)
     return (long long)i + P * ((long long)j + P * (long long)k);
 }
 
+// FP64 to the smoothing precision, on the integer pipe where it is FP32 (the
+// conversion instruction runs on the FP64 pipe, at 2 a clock on each SM).
+template <typename T> __device__ __forceinline__ T narrow(double x);
+template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <> __device__ __forceinline__ float narrow<float>(double x) { return f64_to_f32_rn(x); }
+
 // f = coef rhs on interior nodes, a pair of consecutive nodes (2m, 2m+1) per
 // thread: one red and one black entry with the same index m, so the stores of
 // a warp are contiguous in each colour array.
@@ -1845,8 +1852,10 @@ __global__ void convert_rhs_kernel(const double* __restrict__ rhs, double coef, 
     const double* src = rhs + set * nat_elems(n) + nat(n, 2 * m, j, k);
     T* row = f + set * 2 * v.cs + ((long long)k * (v.n + 1) + j) * v.M + m;
     const int c = (2 * m + j + k) & 1;  // colour of node 2m; node 2m+1 has the other one
-    if (m > 0) row[(long long)c * v.cs] = (T)(coef * src[0]);  // node 0 is a boundary node
-    row[(long long)(c ^ 1) * v.cs] = (T)(coef * src[1]);
+    double a = src[0], b = src[1];
+    if (coef != 1.0) a *= coef, b *= coef;
+    if (m > 0) row[(long long)c * v.cs] = narrow<T>(a);  // node 0 is a boundary node
+    row[(long long)(c ^ 1) * v.cs] = narrow<T>(b);
 }
 
 template <typename T, bool ADD>
@@ -1916,7 +1925,10 @@ constexpr int kResidBlocksPerSM = 16;
 constexpr int kResidMaxBlocks = 152 * kResidBlocksPerSM;
 constexpr int kRowThreads = 128;
 
-template <typename T>
+// WANT_F: the norm of coef*rhs too (the first residual of a solve; otherwise
+// its partial sums are zero).  The FP64 pipe bounds it, so what is not a sum of
+// the result is left out or done on the integer pipe.
+template <typename T, bool WANT_F>
 __global__ void __launch_bounds__(kRowThreads)
 residual_rows_kernel(const double* __restrict__ u, const double* __restrict__ rhs, double coef, int n, double ih2,
                      T* __restrict__ r, LevelView v, double* __restrict__ partials, long long pstride,
@@ -1936,11 +1948,12 @@ residual_rows_kernel(const double* __restrict__ u, const double* __restrict__ rh
         for (int i = threadIdx.x + 1; i < n; i += kRowThreads) {
             const long long o = nat(n, i, j, k);
             const double s = (u[o + 1] + u[o - 1]) + (u[o + P] + u[o - P]) + (u[o + Q] + u[o - Q]);
-            const double fv = coef * rhs[o];
+            double fv = rhs[o];
+            if (coef != 1.0) fv *= coef;
             const double res = fv - (s - 6.0 * u[o]) * ih2;
-            r[node_off(v, i, j, k)] = (T)res;
+            r[node_off(v, i, j, k)] = narrow<T>(res);
             rr = fma(res, res, rr);
-            ff = fma(fv, fv, ff);
+            if (WANT_F) ff = fma(fv, fv, ff);
         }
     }
     for (int off = 16; off > 0; off >>= 1) {
@@ -2431,12 +2444,18 @@ int residual_rows_blocks(int n)
 }
 
 template <typename T>
-int launch_residual_rows(const double* u, const double* rhs, double coef, int n, double h, T* r, const LevelView& v,
-                         double* partials, cudaStream_t s, const Sets& sets)
+int launch_residual_rows(const double* u, const double* rhs, double coef, int n, double h, bool want_f, T* r,
+                         const LevelView& v, double* partials, cudaStream_t s, const Sets& sets)
 {
     const int nb = residual_rows_blocks(n);
-    residual_rows_kernel<T><<<dim3(nb, sets.n), kRowThreads, 0, s>>>(u, rhs, coef, n, 1.0 / (h * h), r, v, partials,
-                                                                     sets.pstride, sets.act);
+    const dim3 g(nb, sets.n);
+    const double ih2 = 1.0 / (h * h);
+    if (want_f)
+        residual_rows_kernel<T, true><<<g, kRowThreads, 0, s>>>(u, rhs, coef, n, ih2, r, v, partials, sets.pstride,
+                                                                sets.act);
+    else
+        residual_rows_kernel<T, false><<<g, kRowThreads, 0, s>>>(u, rhs, coef, n, ih2, r, v, partials, sets.pstride,
+                                                                 sets.act);
     return nb;
 }
 
@@ -2512,8 +2531,8 @@ void launch_reduce_norms(const double* partials, int nblocks, double* out, cudaS
     template void launch_assign_outer<T>(double*, int, const T*, const LevelView&, bool, cudaStream_t, const Sets&);  \
     template int launch_residual_outer<T>(const double*, const double*, double, int, double, T*, const LevelView&,    \
                                           double*, cudaStream_t);                                                      \
-    template int launch_residual_rows<T>(const double*, const double*, double, int, double, T*, const LevelView&,     \
-                                         double*, cudaStream_t, const Sets&);
+    template int launch_residual_rows<T>(const double*, const double*, double, int, double, bool, T*,                  \
+                                         const LevelView&, double*, cudaStream_t, const Sets&);
 
 QUMOND_INSTANTIATE(float)
 QUMOND_INSTANTIATE(double)

@@ -124,8 +124,8 @@ void launch_reduce_norms(const double* partials, int nblocks, double* out, cudaS
 int residual_outer_blocks(int n);
 
 // Residual with a fixed number of blocks (residual_rows_blocks(n) partial sums).
-template <typename T> int launch_residual_rows(const double* u, const double* rhs, double coef, int n, double h, T* r,
-                                               const LevelView& v, double* partials, cudaStream_t s,
+template <typename T> int launch_residual_rows(const double* u, const double* rhs, double coef, int n, double h,
+                                               bool want_f, T* r, const LevelView& v, double* partials, cudaStream_t s,
                                                const Sets& sets = Sets());
 int residual_rows_blocks(int n);
 

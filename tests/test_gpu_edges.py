@@ -146,3 +146,23 @@ def test_coarse_levels_match_the_oracle(q, ora, n, npre, npost, ncycle):
         ctx.qumond_solve_mond(0, to_dev(f), None, phi)
         assert np.max(np.abs(phi.cpu().numpy() - want)) <= tol * np.max(np.abs(want))
         ctx.close()
+
+
+@pytest.mark.parametrize("n,ratio,sets", [(4, 2, 1), (8, 4, 2), (16, 8, 1), (64, 2, 3), (128, 4, 1)])
+def test_boundary_from_the_parent(q, ora, n, ratio, sets):
+    # no V-cycles to speak of: only the boundary nodes are compared; every offset of each ratio occurs
+    rng = np.random.default_rng(n)
+    L0 = 64.0
+    par = rng.uniform(-1.0, 1.0, (sets, (n + 1) ** 3))
+    ctx = q.Context(n=n, nboxes=2, L0=L0, box_ratio=ratio, nsets=sets, ncycle=1)
+    phi = torch.zeros(sets * (n + 1) ** 3, dtype=torch.float64, device="cuda")
+    ctx.qumond_solve_mond(1, torch.zeros_like(phi), to_dev(par.reshape(-1)), phi)
+    got = phi.cpu().numpy().reshape(sets, n + 1, n + 1, n + 1)
+    m = np.ones((n + 1,) * 3, dtype=bool)
+    m[1:-1, 1:-1, 1:-1] = False
+    for s in range(sets):
+        want = np.zeros((n + 1) ** 3)
+        ora.boundary_fill(n, L0, (0.0, 0.0, 0.0), par[s], L0 / ratio, (0.0, 0.0, 0.0), want)
+        # exact weights, eight products of values <= 1 summed in one order: a few roundings on each side
+        assert np.max(np.abs(got[s][m] - want.reshape(m.shape)[m])) <= 16 * 2.0 ** -53
+    ctx.close()
