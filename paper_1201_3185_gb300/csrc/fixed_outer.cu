@@ -117,11 +117,15 @@ __global__ void __launch_bounds__(256) scan_max_level_kernel(const float4* __res
         const unsigned m = m1 > m2 ? m1 : m2;
         local = m > local ? m : local;
     }
-    for (int off = 16; off > 0; off >>= 1) {
-        const unsigned o = __shfl_down_sync(0xffffffffu, local, off);
-        local = o > local ? o : local;
-    }
-    if ((threadIdx.x & 31) == 0) atomicMax(out, local);
+    // one atomic a block, and only where it raises the maximum (one a warp, 2e4 on one address, cost as much as the
+    // pass itself)
+    local = __reduce_max_sync(0xffffffffu, local);
+    __shared__ unsigned most;
+    if (threadIdx.x == 0) most = 0u;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicMax(&most, local);
+    __syncthreads();
+    if (threadIdx.x == 0 && most > *(volatile unsigned*)out) atomicMax(out, most);
 }
 
 // S = 56 - ceil(log2(max|u|)), kept in [-60, 100] so that 2^S and 2^-S stay
@@ -458,8 +462,8 @@ void launch_fixed_scale(const float* e, const LevelView& v, const double* u64, i
         scan_max_kernel<<<dim3(blocks_for_rows((long long)(n + 1) * (n + 1)), ns), kThreads, 0, s>>>(e, v, u64, n, 1,
                                                                                                   maxbits);
     else
-        scan_max_level_kernel<<<dim3(kMaxBlocks, ns), 256, 0, s>>>(reinterpret_cast<const float4*>(e), 2 * v.cs / 4,
-                                                                   maxbits);
+        scan_max_level_kernel<<<dim3((kMaxBlocks / 2 + ns - 1) / ns, ns), 256, 0, s>>>(
+            reinterpret_cast<const float4*>(e), 2 * v.cs / 4, maxbits);
     choose_scale_kernel<<<ns, 1, 0, s>>>(maxbits, st);
 }
 

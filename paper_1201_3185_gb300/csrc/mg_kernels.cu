@@ -452,12 +452,23 @@ restrict_full_kernel(const T* __restrict__ ff, LevelView vf, T* __restrict__ fc,
     const int J = blockIdx.y * kBY + threadIdx.y + 1;
     const int K = kz + 1;
     if (I >= vc.n || J >= vc.n) return;
-    const T w[3] = {T(0.25), T(0.5), T(0.25)};
+    // node i = 2I of a row lies at entry I of one colour, i = 2I -+ 1 at I - 1 and I of the other
+    const int P = vf.M;
+    const long long Q = (long long)P * (vf.n + 1);
+    const T* at = ff + ((2 * K) * Q + (long long)(2 * J) * P + I);
     T acc = T(0);
+#pragma unroll
     for (int c = -1; c <= 1; ++c)
-        for (int b = -1; b <= 1; ++b)
-            for (int a = -1; a <= 1; ++a)
-                acc += (w[a + 1] * w[b + 1] * w[c + 1]) * ff[node_off(vf, 2 * I + a, 2 * J + b, 2 * K + c)];
+#pragma unroll
+        for (int b = -1; b <= 1; ++b) {
+            const bool odd = ((b + c) & 1) != 0;  // j + k odd: the even nodes are black
+            const T* even = at + (c * Q + b * P) + (odd ? vf.cs : 0);
+            const T* other = at + (c * Q + b * P) + (odd ? 0 : vf.cs);
+            const T w = T(b == 0 ? 0.5 : 0.25) * T(c == 0 ? 0.5 : 0.25);
+            acc += (T(0.25) * w) * other[-1];
+            acc += (T(0.5) * w) * even[0];
+            acc += (T(0.25) * w) * other[0];
+        }
     fc[node_off(vc, I, J, K)] = acc;
 }
 
@@ -1838,17 +1849,21 @@ template <typename T> __device__ __forceinline__ T narrow(double x);
 template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
 template <> __device__ __forceinline__ float narrow<float>(double x) { return f64_to_f32_rn(x); }
 
+constexpr int kConvertThreads = 256;
+
 // f = coef rhs on interior nodes, a pair of consecutive nodes (2m, 2m+1) per
-// thread: one red and one black entry with the same index m, so the stores of
+// thread of a flat grid: one red and one black entry with the same index m, so the stores of
 // a warp are contiguous in each colour array.
 template <typename T>
 __global__ void convert_rhs_kernel(const double* __restrict__ rhs, double coef, int n, T* __restrict__ f, LevelView v)
 {
-    int kz;
-    const int set = set_of(n - 1, kz);
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y + 1, k = kz + 1;
-    if (m >= n / 2) return;
+    const int set = blockIdx.y;
+    const unsigned half = (unsigned)n / 2, lh = 31u - (unsigned)__clz((int)half);  // a power of two
+    const unsigned idx = blockIdx.x * (unsigned)kConvertThreads + threadIdx.x;     // (plane, row, pair), below 2^30
+    const unsigned row2 = idx >> lh, plane = row2 / (unsigned)(n - 1);
+    const int m = (int)(idx & (half - 1));
+    const int j = (int)(row2 - plane * (unsigned)(n - 1)) + 1, k = (int)plane + 1;
+    if (k >= n) return;
     const double* src = rhs + set * nat_elems(n) + nat(n, 2 * m, j, k);
     T* row = f + set * 2 * v.cs + ((long long)k * (v.n + 1) + j) * v.M + m;
     const int c = (2 * m + j + k) & 1;  // colour of node 2m; node 2m+1 has the other one
@@ -2410,8 +2425,8 @@ template <typename T>
 void launch_convert_rhs(const double* rhs, double coef, int n, T* f, const LevelView& v, cudaStream_t s,
                         const Sets& sets)
 {
-    const dim3 g(cdiv(n / 2, kOuterThreads), (unsigned)(n - 1), (unsigned)(n - 1));
-    convert_rhs_kernel<T><<<per_sets(g, sets), kOuterThreads, 0, s>>>(rhs, coef, n, f, v);
+    const dim3 g(cdiv((long long)(n - 1) * (n - 1) * (n / 2), kConvertThreads), (unsigned)sets.n);
+    convert_rhs_kernel<T><<<g, kConvertThreads, 0, s>>>(rhs, coef, n, f, v);
 }
 
 template <typename T>
