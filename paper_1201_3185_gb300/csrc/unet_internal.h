@@ -44,7 +44,7 @@ struct WgradArgs {
 
 Brick brick_for(int S);
 size_t conv3_smem_bytes(int cout_tile);
-int conv3_tile(int cout);
+int conv3_tile(int cout, int bricks);  // output channels of a block
 void prepare_conv3();
 void launch_conv3(ConvArgs a, cudaStream_t s);
 

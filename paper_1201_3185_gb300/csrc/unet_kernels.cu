@@ -14,6 +14,8 @@
 // (both operands staged transposed), reduced over CTAs in a fixed order.
 #include "unet_internal.h"
 
+#include <cstring>
+
 #include <cuda_bf16.h>
 
 namespace qumond {
@@ -184,11 +186,16 @@ size_t conv3_smem_bytes(int cout_tile)
     return (size_t)kHaloMax * kHaloStride * 2 + (size_t)cout_tile * kWRow * 2;
 }
 
-int conv3_tile(int cout)
+// The widest tile of output channels that still gives every multiprocessor a
+// block, down to 16: the levels of 16^3 and 8^3 voxels have 32 and 4 bricks, and
+// at 64 channels a tile 32 and 8 blocks ran on 152 multiprocessors (192 -> 64
+// channels at 16^3: 101 us, 82 us with 16; 128 -> 128 at 8^3: 73 us, 43 us).  An
+// output channel's sums do not depend on the tile.
+int conv3_tile(int cout, int bricks)
 {
-    if (cout % 64 == 0) return 64;
-    if (cout % 48 == 0) return 48;
-    if (cout % 32 == 0) return 32;
+    const int tiles[3] = {64, 48, 32};
+    for (int t : tiles)
+        if (cout % t == 0 && (long long)bricks * (cout / t) >= 152) return t;
     return 16;
 }
 
@@ -219,7 +226,7 @@ void launch_conv3(ConvArgs a, cudaStream_t s)
     }
     a.brick = brick_for(a.S);
     const int bricks = (a.S / a.brick.bx) * (a.S / a.brick.by) * (a.S / a.brick.bz);
-    switch (conv3_tile(a.cout)) {
+    switch (conv3_tile(a.cout, bricks)) {
     case 64: launch_conv3_t<8>(a, bricks, s); break;
     case 48: launch_conv3_t<6>(a, bricks, s); break;
     case 32: launch_conv3_t<4>(a, bricks, s); break;
@@ -231,9 +238,24 @@ void launch_conv3(ConvArgs a, cudaStream_t s)
 // Weight gradient: part[blk][co][tap][ci] = sum over the CTA's voxels of
 // g[v, co0+co] x[v + off(tap), ci0+ci], for a tile of 16 MT output channels
 // and 16 input channels; grid = (vblocks, cout/(16 MT), cin/16).  Warp w takes
-// taps w, w+8, w+16, w+24.  The k-dimension (voxels) must be contiguous in
-// pairs for the MMA fragments, so both operands are staged transposed: g as
-// [co][voxel], x as three copies [dx][ci][halo row][x] each shifted by its dx.
+// taps w, w+8, w+16, w+24.  The k-dimension is the voxels, while memory holds
+// channels contiguous: both operands are staged as they lie in memory, one row
+// of 16 MT (or 16) channels per voxel, and ldmatrix transposes 8 x 8 tiles on
+// the way to the registers; it takes an address per row, so a tap is an offset
+// of the rows in the halo.  (Staged transposed, with three shifted copies of
+// the halo in two-byte stores, a brick took 10 us: 273 us for 48 -> 16 channels
+// at 64^3, 155 us now.)
+constexpr int kXRow = 24;  // bf16 of a halo voxel: 16 channels and 8 of padding (8 rows meet all 32 banks)
+
+__device__ __forceinline__ void ldmatrix4_trans(unsigned (&r)[4], const __nv_bfloat16* row)
+{
+    const unsigned at = (unsigned)__cvta_generic_to_shared(row);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(at)
+                 : "memory");
+}
+
 template <int MT>
 __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
 {
@@ -241,11 +263,9 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     const Brick b = a.brick;
     const int S = a.S;
     const int nvox = b.bx * b.by * b.bz;
-    const int gstride = 128 + 8;                           // bf16 per channel row of gT
-    const int hrows = (b.by + 2) * (b.bz + 2);
-    const int xstride = hrows * b.bx + 8;                  // bf16 per channel row of xT
-    __nv_bfloat16* gT = reinterpret_cast<__nv_bfloat16*>(smem_raw);
-    __nv_bfloat16* xT = gT + 16 * MT * gstride;            // [3][16][xstride]
+    constexpr int kGRow = 16 * MT + 8;                     // bf16 of a voxel's gradients, with padding
+    __nv_bfloat16* gs = reinterpret_cast<__nv_bfloat16*>(smem_raw);
+    __nv_bfloat16* xs = gs + 128 * kGRow;                  // the brick's halo
 
     const int nbx = S / b.bx, nby = S / b.by;
     const int nbricks = nbx * nby * (S / b.bz);
@@ -253,6 +273,18 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
     const int ntap = warp < 3 ? 4 : 3;  // taps warp, warp+8, warp+16 (, warp+24)
+    const int hx = b.bx + 2, hy = b.by + 2, hz = b.bz + 2;
+    // the row that this lane addresses in each 16-voxel step: of the gradients, tiles (voxels 0-7, 8-15) x (channels
+    // 0-7, 8-15) in the order of the A fragment; of the halo in that of two B fragments
+    const int rv = lane & 7, mat = lane >> 3;
+    const __nv_bfloat16* const grow = gs + (rv + (mat >> 1) * 8) * kGRow + (mat & 1) * 8;
+    const int xv = rv + (mat & 1) * 8, xc = (mat >> 1) * 8;
+    int toff[4];  // the taps' offsets in the halo
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int t = warp + 8 * q;
+        toff[q] = (((t / 9 - 1) * hy + ((t / 3) % 3 - 1)) * hx + (t % 3 - 1)) * kXRow;
+    }
 
     float acc[4][MT][2][4];
 #pragma unroll
@@ -264,9 +296,9 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
 
     for (int brick = blockIdx.x; brick < nbricks; brick += gridDim.x) {
         const int x0 = (brick % nbx) * b.bx, y0 = ((brick / nbx) % nby) * b.by, z0 = (brick / (nbx * nby)) * b.bz;
-        // g^T: 16 MT channels x nvox voxels (voxels past nvox are zero)
+        // 16 MT channels of nvox voxels (voxels past nvox are zero)
         for (int q = threadIdx.x; q < 128 * 2 * MT; q += blockDim.x) {
-            const int l = q % 128, part = q / 128;  // part: 8 channels
+            const int l = q / (2 * MT), part = q % (2 * MT);  // part: 8 channels
             uint4 val = make_uint4(0u, 0u, 0u, 0u);
             if (l < nvox) {
                 int lz, ly, lx;
@@ -274,70 +306,37 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
                 const long long v = ((long long)(z0 + lz) * S + (y0 + ly)) * S + (x0 + lx);
                 val = *reinterpret_cast<const uint4*>(a.g + v * a.ld_g + a.g_off + co0 + part * 8);
             }
-            const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&val);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) gT[(part * 8 + c) * gstride + l] = e[c];
+            *reinterpret_cast<uint4*>(gs + l * kGRow + part * 8) = val;
         }
-        // x^T: halo rows of the brick, three copies shifted by dx
-        const int hx = b.bx + 2;
-        for (int q = threadIdx.x; q < hrows * hx * 2; q += blockDim.x) {
+        for (int q = threadIdx.x; q < hx * hy * hz * 2; q += blockDim.x) {
             const int part = q & 1, hv = q >> 1;
-            const int ix = hv % hx, row = hv / hx;
-            const int iy = row % (b.by + 2), iz = row / (b.by + 2);
+            const int ix = hv % hx, iy = (hv / hx) % hy, iz = hv / (hx * hy);
             const int gx = x0 + ix - 1, gy = y0 + iy - 1, gz = z0 + iz - 1;
             uint4 val = make_uint4(0u, 0u, 0u, 0u);
             if (gx >= 0 && gx < S && gy >= 0 && gy < S && gz >= 0 && gz < S) {
                 const long long v = ((long long)gz * S + gy) * S + gx;
                 val = *reinterpret_cast<const uint4*>(a.x + v * a.ld_x + a.x_off + ci0 + part * 8);
             }
-            const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&val);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {  // copy d holds dx = d - 1: xT[d][ci][row][lx] = x(lx + dx)
-                const int lx = ix - d;     // ix = lx + dx + 1
-                if (lx >= 0 && lx < b.bx) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) xT[(d * 16 + part * 8 + c) * xstride + row * b.bx + lx] = e[c];
-                }
-            }
+            *reinterpret_cast<uint4*>(xs + hv * kXRow + part * 8) = val;
         }
         __syncthreads();
         for (int s = 0; s * 16 < nvox; ++s) {
-            // A fragments (co x voxel), shared by the warp's taps
-            unsigned af[MT][4];
+            unsigned af[MT][4];  // co x voxel, shared by the warp's taps
 #pragma unroll
-            for (int m = 0; m < MT; ++m) {
-                const __nv_bfloat16* p0 = gT + (m * 16 + g) * gstride + s * 16 + tig * 2;
-                const __nv_bfloat16* p1 = p0 + 8 * gstride;
-                af[m][0] = lds32(p0);
-                af[m][1] = lds32(p1);
-                af[m][2] = lds32(p0 + 8);
-                af[m][3] = lds32(p1 + 8);
-            }
-            // this thread's two k-pairs: voxels s*16 + tig*2 (+1) and + 8
-            int rowk[2], lxk[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int l = s * 16 + tig * 2 + h * 8;
-                int lz, ly, lx;
-                brick_coords(b, l < nvox ? l : 0, lz, ly, lx);
-                rowk[h] = (lz + 1) * (b.by + 2) + (ly + 1);
-                lxk[h] = lx;
-            }
+            for (int m = 0; m < MT; ++m) ldmatrix4_trans(af[m], grow + s * 16 * kGRow + m * 16);
+            const int l = s * 16 + xv;
+            int lz, ly, lx;
+            brick_coords(b, l < nvox ? l : 0, lz, ly, lx);  // past nvox any voxel: its gradients are zero
+            const __nv_bfloat16* xrow = xs + (((lz + 1) * hy + (ly + 1)) * hx + (lx + 1)) * kXRow + xc;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (q < ntap) {
-                    const int t = warp + 8 * q;
-                    const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-                    const int roff = dz * (b.by + 2) + dy;
-                    const __nv_bfloat16* base = xT + ((dx + 1) * 16) * xstride;
+                    unsigned bf[4];  // voxel x ci: input channels 0-7 and 8-15
+                    ldmatrix4_trans(bf, xrow + toff[q]);
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const __nv_bfloat16* cb = base + (j * 8 + g) * xstride;
-                        const unsigned b0 = lds32(cb + (rowk[0] + roff) * b.bx + lxk[0]);
-                        const unsigned b1 = lds32(cb + (rowk[1] + roff) * b.bx + lxk[1]);
+                    for (int j = 0; j < 2; ++j)
 #pragma unroll
-                        for (int m = 0; m < MT; ++m) mma16816(acc[q][m][j], af[m], b0, b1);
-                    }
+                        for (int m = 0; m < MT; ++m) mma16816(acc[q][m][j], af[m], bf[2 * j], bf[2 * j + 1]);
                 }
             }
         }
@@ -363,23 +362,35 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     }
 }
 
-// dW[co][tap][ci] (+)= sum over the vblocks, in order, of the partials
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int vblocks, int mt, int cout, int cin,
-                                    float* __restrict__ dw, int accumulate)
+// dW[co][tap][ci] (+)= sum over the vblocks of the partials: 8 threads an
+// element take every 8th block each, and their sums are added in order (one
+// thread an element, with up to 304 dependent reads, took 24 us on 27 blocks).
+constexpr int kSlices = 8;
+
+__global__ void __launch_bounds__(32 * kSlices)
+wgrad_reduce_kernel(const float* __restrict__ part, int vblocks, int mt, int cout, int cin, float* __restrict__ dw,
+                    int accumulate)
 {
-    const long long total = (long long)cout * 27 * cin;
+    __shared__ float sum[kSlices][32];
+    const int total = cout * 27 * cin;
     const int tile_co = 16 * mt;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int ci = (int)(e % cin);
-        const int t = (int)((e / cin) % 27);
-        const int co = (int)(e / (27LL * cin));
-        const int cot = co / tile_co, cil = ci / 16;
-        const long long blk0 = ((long long)cil * (cout / tile_co) + cot) * vblocks;
-        const long long inner = ((long long)(co % tile_co) * 27 + t) * 16 + (ci % 16);
-        float s = 0.0f;
-        for (int vb = 0; vb < vblocks; ++vb) s += part[(blk0 + vb) * (tile_co * 27 * 16) + inner];
-        dw[e] = accumulate ? dw[e] + s : s;
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
+    float s = 0.0f;
+    if (e < total) {
+        const int ci = e % cin, t = (e / cin) % 27, co = e / (27 * cin);
+        const long long blk0 = ((long long)(ci / 16) * (cout / tile_co) + co / tile_co) * vblocks;
+        const float* at = part + blk0 * (tile_co * 27 * 16) + ((long long)(co % tile_co) * 27 + t) * 16 + (ci % 16);
+#pragma unroll 4
+        for (int vb = slice; vb < vblocks; vb += kSlices) s += at[(long long)vb * (tile_co * 27 * 16)];
+    }
+    sum[slice][lane] = s;
+    __syncthreads();
+    if (slice == 0 && e < total) {
+        float v = sum[0][lane];
+#pragma unroll
+        for (int q = 1; q < kSlices; ++q) v += sum[q][lane];
+        dw[e] = accumulate ? dw[e] + v : v;
     }
 }
 
@@ -387,8 +398,7 @@ int wgrad_mt(int cout) { return cout % 32 == 0 ? 2 : 1; }
 
 size_t wgrad_smem_bytes(int mt, const Brick& b)
 {
-    const int hrows = (b.by + 2) * (b.bz + 2);
-    return (size_t)2 * (16 * mt * (128 + 8) + 3 * 16 * (hrows * b.bx + 8));
+    return sizeof(__nv_bfloat16) * (size_t)(128 * (16 * mt + 8) + (b.bx + 2) * (b.by + 2) * (b.bz + 2) * kXRow);
 }
 
 int wgrad_vblocks(int S, int cout, int cin, int sms)
@@ -418,70 +428,105 @@ void launch_wgrad(WgradArgs a, int vblocks, float* dw, int accumulate, cudaStrea
         wgrad_kernel<2><<<grid, 256, smem, s>>>(a);
     else
         wgrad_kernel<1><<<grid, 256, smem, s>>>(a);
-    const long long total = (long long)a.cout * 27 * a.cin;
-    const int blocks = (int)((total + 255) / 256 < 2048 ? (total + 255) / 256 : 2048);
-    wgrad_reduce_kernel<<<blocks, 256, 0, s>>>(a.part, vblocks, mt, a.cout, a.cin, dw, accumulate);
+    const int total = a.cout * 27 * a.cin;
+    wgrad_reduce_kernel<<<(total + 31) / 32, 32 * kSlices, 0, s>>>(a.part, vblocks, mt, a.cout, a.cin, dw, accumulate);
 }
 
 // ---------------------------------------------------------------------------
-// Bias gradient: db[c] (+)= sum_v g[v, c], per-block partial sums in voxel
-// order, then the blocks in order.
-__global__ void colsum_kernel(const __nv_bfloat16* __restrict__ g, int ld, int off, int C, long long nvox,
-                              float* __restrict__ part)
+// Eight consecutive channels of a voxel as one 16-byte value.
+struct Bf8 {
+    __nv_bfloat16 v[8];
+};
+__device__ __forceinline__ Bf8 load8(const __nv_bfloat16* p)
 {
-    // block: 256 threads = C columns x (256 / C) row lanes (C divides 256)
-    const int c = threadIdx.x % C, lane = threadIdx.x / C, lanes = blockDim.x / C;
+    const uint4 w = *reinterpret_cast<const uint4*>(p);
+    Bf8 r;
+    memcpy(&r, &w, sizeof r);
+    return r;
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const Bf8& r)
+{
+    uint4 w;
+    memcpy(&w, &r, sizeof w);
+    *reinterpret_cast<uint4*>(p) = w;
+}
+
+// ---------------------------------------------------------------------------
+// Bias gradient: db[c] (+)= sum_v g[v, c]: partial sums per block (fixed order),
+// then a warp a channel adds the blocks' (lane l takes blocks l, l + 32, ..).
+__global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16* __restrict__ g, int ld, int off, int C,
+                                                     long long nvox, float* __restrict__ part)
+{
+    // block: C / 8 groups of channels x (2048 / C) row lanes (C divides 2048)
+    const int groups = C / 8;
+    const int c = threadIdx.x % groups, lane = threadIdx.x / groups, lanes = 256 / groups;
     const long long chunk = (nvox + gridDim.x - 1) / gridDim.x;
     const long long v0 = blockIdx.x * chunk, v1 = v0 + chunk < nvox ? v0 + chunk : nvox;
-    float s = 0.0f;
-    for (long long v = v0 + lane; v < v1; v += lanes) s += __bfloat162float(g[v * ld + off + c]);
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
+    float s[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] = 0.0f;
+    for (long long v = v0 + lane; v < v1; v += lanes) {
+        const Bf8 w = load8(g + v * ld + off + 8 * c);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s[q] += __bfloat162float(w.v[q]);
+    }
+    __shared__ float red[8][256];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = s[q];
     __syncthreads();
-    if (lane == 0) {
+    if ((int)threadIdx.x < C) {
+        const int q = threadIdx.x % 8, cc = threadIdx.x / 8;
         float t = 0.0f;
-        for (int r = 0; r < lanes; ++r) t += red[r * C + c];
-        part[(long long)blockIdx.x * C + c] = t;
+        for (int r = 0; r < lanes; ++r) t += red[q][r * groups + cc];
+        part[(long long)blockIdx.x * C + threadIdx.x] = t;
     }
 }
 
 __global__ void colsum_reduce_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out,
                                      int accumulate)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= C) return;
     float s = 0.0f;
-    for (int b = 0; b < nb; ++b) s += part[(long long)b * C + c];
-    out[c] = accumulate ? out[c] + s : s;
+    for (int b = lane; b < nb; b += 32) s += part[(long long)b * C + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[c] = accumulate ? out[c] + s : s;
 }
 
 void launch_bias_grad(const __nv_bfloat16* g, int ld, int off, int C, long long nvox, float* part, int nb, float* db,
                       int accumulate, cudaStream_t s)
 {
-    // C <= 256 and a power of two times 16 or 48 ... the layer widths are 16, 32, 64, 128
+    // the layer widths are 16, 32, 64 and 128
     colsum_kernel<<<nb, 256, 0, s>>>(g, ld, off, C, nvox, part);
-    colsum_reduce_kernel<<<(C + 127) / 128, 128, 0, s>>>(part, nb, C, db, accumulate);
+    colsum_reduce_kernel<<<(C + 3) / 4, 128, 0, s>>>(part, nb, C, db, accumulate);
 }
 
 // ---------------------------------------------------------------------------
 // 2x2x2 average pooling (S -> S/2) and its adjoint with the skip gradient and the ReLU mask
+// (eight channels a thread: the channel counts, row strides and offsets are
+// multiples of 8)
 __global__ void pool_kernel(const __nv_bfloat16* __restrict__ x, int ld_x, int off_x, int C, int S,
                             __nv_bfloat16* __restrict__ y)
 {
-    const int Sh = S / 2;
-    const long long total = (long long)Sh * Sh * Sh * C;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long p = e / C;
-        const int px = (int)(p % Sh), py = (int)((p / Sh) % Sh), pz = (int)(p / ((long long)Sh * Sh));
-        float s = 0.0f;
+    const int Sh = S / 2, groups = C / 8;
+    const int total = Sh * Sh * Sh * groups;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = 8 * (e % groups), p = e / groups;
+        const int px = p % Sh, py = (p / Sh) % Sh, pz = p / (Sh * Sh);
+        float s[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.0f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const long long v = ((long long)(2 * pz + (q >> 2)) * S + (2 * py + ((q >> 1) & 1))) * S + 2 * px + (q & 1);
-            s += __bfloat162float(x[v * ld_x + off_x + c]);
+            const Bf8 w = load8(x + v * ld_x + off_x + c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[k] += __bfloat162float(w.v[k]);
         }
-        y[e] = __float2bfloat16_rn(0.125f * s);
+        Bf8 r;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) r.v[k] = __float2bfloat16_rn(0.125f * s[k]);
+        store8(y + (long long)p * C + c, r);
     }
 }
 
@@ -490,32 +535,42 @@ __global__ void pool_back_kernel(const __nv_bfloat16* __restrict__ gp, const __n
                                  int ld_s, int off_s, const __nv_bfloat16* __restrict__ mask, int ld_m, int off_m,
                                  int C, int S, __nv_bfloat16* __restrict__ gx)
 {
-    const int Sh = S / 2;
-    const long long total = (long long)S * S * S * C;
+    const int Sh = S / 2, groups = C / 8;
+    const long long total = (long long)S * S * S * groups;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long v = e / C;
-        const int x = (int)(v % S), y = (int)((v / S) % S), z = (int)(v / ((long long)S * S));
+        const unsigned u = (unsigned)e;  // below 2^31 for S <= 512, C <= 128
+        const int c = 8 * (int)(u % (unsigned)groups);
+        const unsigned v = u / (unsigned)groups;
+        const int x = (int)(v % (unsigned)S), y = (int)((v / (unsigned)S) % (unsigned)S), z = (int)(v / ((unsigned)S * S));
         const long long p = ((long long)(z / 2) * Sh + y / 2) * Sh + x / 2;
-        float r = 0.125f * __bfloat162float(gp[p * C + c]);
-        if (gskip) r += __bfloat162float(gskip[v * ld_s + off_s + c]);
-        if (!(__bfloat162float(mask[v * ld_m + off_m + c]) > 0.0f)) r = 0.0f;
-        gx[e] = __float2bfloat16_rn(r);
+        const Bf8 a = load8(gp + p * C + c), m = load8(mask + (long long)v * ld_m + off_m + c);
+        Bf8 k = a, r;
+        if (gskip) k = load8(gskip + (long long)v * ld_s + off_s + c);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            float w = 0.125f * __bfloat162float(a.v[q]);
+            if (gskip) w += __bfloat162float(k.v[q]);
+            if (!(__bfloat162float(m.v[q]) > 0.0f)) w = 0.0f;
+            r.v[q] = __float2bfloat16_rn(w);
+        }
+        store8(gx + (long long)v * C + c, r);
     }
 }
 
 // nearest-neighbour upsampling S/2 -> S into channels [0, C) of a concatenation (row stride ld_y)
 __global__ void up_kernel(const __nv_bfloat16* __restrict__ x, int C, int S, __nv_bfloat16* __restrict__ y, int ld_y)
 {
-    const int Sh = S / 2;
-    const long long total = (long long)S * S * S * C;
+    const int Sh = S / 2, groups = C / 8;
+    const long long total = (long long)S * S * S * groups;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long v = e / C;
-        const int px = (int)(v % S) / 2, py = (int)((v / S) % S) / 2, pz = (int)(v / ((long long)S * S)) / 2;
-        y[v * ld_y + c] = x[(((long long)pz * Sh + py) * Sh + px) * C + c];
+        const unsigned u = (unsigned)e;
+        const int c = 8 * (int)(u % (unsigned)groups);
+        const unsigned v = u / (unsigned)groups;
+        const int px = (int)(v % (unsigned)S) / 2, py = (int)((v / (unsigned)S) % (unsigned)S) / 2;
+        const int pz = (int)(v / ((unsigned)S * S)) / 2;
+        store8(y + (long long)v * ld_y + c, load8(x + (((long long)pz * Sh + py) * Sh + px) * C + c));
     }
 }
 
@@ -523,21 +578,26 @@ __global__ void up_kernel(const __nv_bfloat16* __restrict__ x, int C, int S, __n
 __global__ void up_back_kernel(const __nv_bfloat16* __restrict__ gy, int ld_y, const __nv_bfloat16* __restrict__ mask,
                                int C, int S, __nv_bfloat16* __restrict__ gx)
 {
-    const int Sh = S / 2;
-    const long long total = (long long)Sh * Sh * Sh * C;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(e % C);
-        const long long p = e / C;
-        const int px = (int)(p % Sh), py = (int)((p / Sh) % Sh), pz = (int)(p / ((long long)Sh * Sh));
-        float s = 0.0f;
+    const int Sh = S / 2, groups = C / 8;
+    const int total = Sh * Sh * Sh * groups;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const int c = 8 * (e % groups), p = e / groups;
+        const int px = p % Sh, py = (p / Sh) % Sh, pz = p / (Sh * Sh);
+        float s[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.0f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const long long v = ((long long)(2 * pz + (q >> 2)) * S + (2 * py + ((q >> 1) & 1))) * S + 2 * px + (q & 1);
-            s += __bfloat162float(gy[v * ld_y + c]);
+            const Bf8 w = load8(gy + v * ld_y + c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[k] += __bfloat162float(w.v[k]);
         }
-        if (!(__bfloat162float(mask[p * C + c]) > 0.0f)) s = 0.0f;
-        gx[e] = __float2bfloat16_rn(s);
+        const Bf8 m = load8(mask + (long long)p * C + c);
+        Bf8 r;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) r.v[k] = __float2bfloat16_rn(__bfloat162float(m.v[k]) > 0.0f ? s[k] : 0.0f);
+        store8(gx + (long long)p * C + c, r);
     }
 }
 
@@ -549,25 +609,25 @@ static int ew_blocks(long long total)
 
 void launch_pool(const __nv_bfloat16* x, int ld_x, int off_x, int C, int S, __nv_bfloat16* y, cudaStream_t s)
 {
-    pool_kernel<<<ew_blocks((long long)(S / 2) * (S / 2) * (S / 2) * C), 256, 0, s>>>(x, ld_x, off_x, C, S, y);
+    pool_kernel<<<ew_blocks((long long)(S / 2) * (S / 2) * (S / 2) * C / 8), 256, 0, s>>>(x, ld_x, off_x, C, S, y);
 }
 
 void launch_pool_back(const __nv_bfloat16* gp, const __nv_bfloat16* gskip, int ld_s, int off_s,
                       const __nv_bfloat16* mask, int ld_m, int off_m, int C, int S, __nv_bfloat16* gx, cudaStream_t s)
 {
-    pool_back_kernel<<<ew_blocks((long long)S * S * S * C), 256, 0, s>>>(gp, gskip, ld_s, off_s, mask, ld_m, off_m, C,
+    pool_back_kernel<<<ew_blocks((long long)S * S * S * C / 8), 256, 0, s>>>(gp, gskip, ld_s, off_s, mask, ld_m, off_m, C,
                                                                          S, gx);
 }
 
 void launch_up(const __nv_bfloat16* x, int C, int S, __nv_bfloat16* y, int ld_y, cudaStream_t s)
 {
-    up_kernel<<<ew_blocks((long long)S * S * S * C), 256, 0, s>>>(x, C, S, y, ld_y);
+    up_kernel<<<ew_blocks((long long)S * S * S * C / 8), 256, 0, s>>>(x, C, S, y, ld_y);
 }
 
 void launch_up_back(const __nv_bfloat16* gy, int ld_y, const __nv_bfloat16* mask, int C, int S, __nv_bfloat16* gx,
                     cudaStream_t s)
 {
-    up_back_kernel<<<ew_blocks((long long)(S / 2) * (S / 2) * (S / 2) * C), 256, 0, s>>>(gy, ld_y, mask, C, S, gx);
+    up_back_kernel<<<ew_blocks((long long)(S / 2) * (S / 2) * (S / 2) * C / 8), 256, 0, s>>>(gy, ld_y, mask, C, S, gx);
 }
 
 // ---------------------------------------------------------------------------
@@ -714,10 +774,11 @@ __global__ void head_train_kernel(const __nv_bfloat16* __restrict__ a, const flo
 __global__ void head_reduce_kernel(const float* __restrict__ part, int nb, float* __restrict__ dwb, int accumulate,
                                    float* __restrict__ loss, float loss_scale)
 {
-    const int c = threadIdx.x;
-    if (c >= 18) return;
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;  // a warp a column
     float s = 0.0f;
-    for (int b = 0; b < nb; ++b) s += part[(long long)b * 18 + c];
+    for (int b = lane; b < nb; b += 32) s += part[(long long)b * 18 + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane != 0) return;
     if (c < 17)
         dwb[c] = accumulate ? dwb[c] + s : s;
     else if (loss)
@@ -734,7 +795,7 @@ void launch_head_train(const __nv_bfloat16* a, const float* wb, const __nv_bfloa
                        float loss_scale, cudaStream_t s)
 {
     head_train_kernel<<<nb, 256, 0, s>>>(a, wb, target, nvox, k, ga, part);
-    head_reduce_kernel<<<1, 32, 0, s>>>(part, nb, dwb, accumulate, loss, loss_scale);
+    head_reduce_kernel<<<1, 18 * 32, 0, s>>>(part, nb, dwb, accumulate, loss, loss_scale);
 }
 
 // phi[node] = phiN[node] + phi_scale * yhat[v] on the interior nodes 1..S-1 of each axis

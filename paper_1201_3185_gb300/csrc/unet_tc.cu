@@ -320,8 +320,9 @@ void prepare_conv3_tc()
 
 void launch_conv3_tc(const ConvArgs& a, cudaStream_t s)
 {
-    const int nt = conv3_tile(a.cout);
-    const dim3 grid((unsigned)((a.S / 8) * (a.S / 16) * a.S), (unsigned)(a.cout / nt));
+    const int bricks = (a.S / 8) * (a.S / 16) * a.S;
+    const int nt = conv3_tile(a.cout, bricks);
+    const dim3 grid((unsigned)bricks, (unsigned)(a.cout / nt));
     const size_t smem = conv3_tc_smem_bytes(nt);
     switch (nt) {
     case 64: conv3_tc_kernel<64><<<grid, 128, smem, s>>>(a); break;

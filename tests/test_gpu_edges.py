@@ -166,3 +166,27 @@ def test_boundary_from_the_parent(q, ora, n, ratio, sets):
         # exact weights, eight products of values <= 1 summed in one order: a few roundings on each side
         assert np.max(np.abs(got[s][m] - want.reshape(m.shape)[m])) <= 16 * 2.0 ** -53
     ctx.close()
+
+
+@pytest.mark.parametrize("S,tensor_path", [(64, 1), (64, 0), (32, 0)])
+def test_guess_gradients_on_all_tile_widths(q, S, tensor_path):
+    """Levels of 64^3 to 4^3 voxels: every width of the channel tile, and weight gradients over 2048 bricks to one.
+    The bounds are those of the gradient test of the smaller networks (14 layers of BF16 rounding: 3 % of the whole
+    vector, 15 % of a block whose terms cancel); a wrong tap, channel or voxel moves a block by tens of percent."""
+    from oracle import unet as U
+    from tests.test_gpu_guess import he, random_sample, rel_l2
+    rng = np.random.default_rng(S)
+    params = he(S)
+    smp = random_sample(rng, S)
+    g = q.Guess(S, 1e5)
+    g.qumond_guess_set_params(to_dev(params, torch.float32))
+    g.qumond_guess_tensor_path(tensor_path)
+    grads = torch.empty(q.Guess.num_params(), dtype=torch.float32, device="cuda")
+    g.qumond_guess_gradients([smp.cuda()], [1.0], grads)
+    g.qumond_guess_status()
+    got = grads.cpu().numpy().astype(np.float64)
+    _, want = U.loss_and_gradients(params, [smp.float().numpy()], [1.0])
+    assert rel_l2(got, want) < 3e-2
+    for name, sl in U.layer_slices():
+        assert rel_l2(got[sl], want[sl]) < 0.15, name
+    g.close()
