@@ -58,7 +58,7 @@ struct qumond_guess {
     float* wpart = nullptr;
     float* cpart = nullptr;
     float* hpart = nullptr;
-    int cblocks = 0, hblocks = 0;
+    int hblocks = 0;
     int tc_ok = 0;        // the device runs tcgen05 (compute capability 10.3, the architecture this library is built for)
     int use_tc = 0;       // 1: tcgen05 convolutions where they apply, 0: mma.sync everywhere
     int* fault = nullptr; // bounded waits of the tcgen05 path
@@ -211,10 +211,10 @@ void backward(qumond_guess* g, const __nv_bfloat16* target, float k, float loss_
         wa.g = g->G[l], wa.ld_g = cout, wa.g_off = 0, wa.cout = cout;
         wa.part = g->wpart;
         wa.S = S;
-        launch_wgrad(wa, wgrad_vblocks(S, cout, cin, g->sms), g->grads + g->woff[l], accumulate, s);
-        g->launches += 4;  // weight gradient + reduction, bias gradient + reduction
-        launch_bias_grad(g->G[l], cout, 0, cout, vox(g, lev), g->cpart, g->cblocks, g->grads + g->boff[l], accumulate,
-                         s);
+        wa.bias_part = g->cpart;
+        launch_wgrad(wa, wgrad_vblocks(S, cout, cin, g->sms), g->grads + g->woff[l], g->grads + g->boff[l], accumulate,
+                     s);
+        g->launches += 2;  // the gradients' partial sums, their reduction
         if (l == 0) break;
         // data gradient: d(input) = conv(G[l], Wd[l]); masked when the input is a ReLU output
         ConvArgs a{};
@@ -329,17 +329,18 @@ qumond_status qumond_guess_create(int S, double phi_scale, qumond_guess** out)
         ok = ok && alloc(g, &g->G[l], nv);
     }
     // weight-gradient partials: the largest layer
-    long long wp = 0;
+    long long wp = 0, cp = 0;
     for (int l = 0; l < kNumLayers; ++l) {
         const int S_l = S >> kLayers[l].level;
         const int mt = wgrad_mt(kLayers[l].cout);
         const long long tiles = (kLayers[l].cout / (16 * mt)) * (kLayers[l].cin / 16);
         const long long need = tiles * wgrad_vblocks(S_l, kLayers[l].cout, kLayers[l].cin, g->sms) * (16LL * mt * 27 * 16);
         if (need > wp) wp = need;
+        const long long bias = (long long)kLayers[l].cout * wgrad_vblocks(S_l, kLayers[l].cout, kLayers[l].cin, g->sms);
+        if (bias > cp) cp = bias;
     }
-    g->cblocks = 2 * g->sms;
     g->hblocks = 2 * g->sms;
-    ok = ok && alloc(g, &g->wpart, wp) && alloc(g, &g->cpart, (size_t)g->cblocks * 128) &&
+    ok = ok && alloc(g, &g->wpart, wp) && alloc(g, &g->cpart, cp) &&
          alloc(g, &g->hpart, (size_t)g->hblocks * 18) && alloc(g, &g->fault, 1) &&
          cudaMemset(g->fault, 0, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMemset(g->params, 0, g->nparams * sizeof(float)) == cudaSuccess &&

@@ -27,24 +27,52 @@ struct ConvArgs {
     int relu;
     int S;
     Brick brick;  // set by the launcher
+    int stages;   // set by the launcher: chunks of input channels in flight
     int use_tc;   // 1: the convolution may run on the tcgen05 path (where conv3_tc_applies); 0: mma.sync
     int* fault;   // set to 3 when a bounded wait of the tcgen05 path gave up
 };
 
-// Weight gradient of a 3^3 convolution: dW[co][tap][ci] = sum_v g[v, co] x[v + off(tap), ci].
+// Weight gradient of a 3^3 convolution: dW[co][tap][ci] = sum_v g[v, co] x[v + off(tap), ci], and the bias gradient
+// sum_v g[v, co].
 struct WgradArgs {
     const __nv_bfloat16* x;  // layer input, row stride ld_x, channels [x_off, x_off + cin)
     int ld_x, x_off, cin;
     const __nv_bfloat16* g;  // gradient at the layer output (after the ReLU mask), row stride ld_g
     int ld_g, g_off, cout;
     float* part;             // partial sums, (cout/16MT) x (cin/16) x vblocks x (16MT x 27 x 16) floats
+    float* bias_part;        // partial sums, vblocks x cout floats
     int S;
     Brick brick;
 };
 
+// 16 bytes of global memory to shared memory, or 16 zero bytes where !in (the address is not read then); through
+// the L1, since the blocks of a multiprocessor read the same weights and overlapping halos
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool in)
+{
+    const unsigned at = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(at), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest `pending` (0 to 2) of this thread's groups are complete
+__device__ __forceinline__ void cp_async_wait(int pending)
+{
+    if (pending == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    else if (pending == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 2;" ::: "memory");
+}
+
 Brick brick_for(int S);
 size_t conv3_smem_bytes(int cout_tile);
 int conv3_tile(int cout, int bricks);  // output channels of a block
+constexpr size_t kConvSmem = 226 * 1024;  // of a multiprocessor, for the chunk rings of its blocks
+constexpr int kConvStages = 4;
+int conv3_stages(size_t stage_bytes, int blocks, int chunks);
+// the most that conv3_stages gives a block
+inline size_t conv3_smem_max(size_t stage_bytes)
+{
+    const size_t n = kConvSmem / (stage_bytes + 2048);
+    return stage_bytes * (n < kConvStages ? n : kConvStages);
+}
 void prepare_conv3();
 void launch_conv3(ConvArgs a, cudaStream_t s);
 
@@ -53,16 +81,14 @@ int tc_selftest();
 bool conv3_tc_applies(const ConvArgs& a);
 size_t conv3_tc_smem_bytes(int nt);
 void prepare_conv3_tc();
-void launch_conv3_tc(const ConvArgs& a, cudaStream_t s);
+void launch_conv3_tc(ConvArgs a, cudaStream_t s);
 
 int wgrad_mt(int cout);
 size_t wgrad_smem_bytes(int mt, const Brick& b);
 int wgrad_vblocks(int S, int cout, int cin, int sms);
 void prepare_wgrad();
-void launch_wgrad(WgradArgs a, int vblocks, float* dw, int accumulate, cudaStream_t s);
+void launch_wgrad(WgradArgs a, int vblocks, float* dw, float* db, int accumulate, cudaStream_t s);
 
-void launch_bias_grad(const __nv_bfloat16* g, int ld, int off, int C, long long nvox, float* part, int nb, float* db,
-                      int accumulate, cudaStream_t s);
 void launch_pool(const __nv_bfloat16* x, int ld_x, int off_x, int C, int S, __nv_bfloat16* y, cudaStream_t s);
 void launch_pool_back(const __nv_bfloat16* gp, const __nv_bfloat16* gskip, int ld_s, int off_s,
                       const __nv_bfloat16* mask, int ld_m, int off_m, int C, int S, __nv_bfloat16* gx, cudaStream_t s);

@@ -57,13 +57,15 @@ __device__ __forceinline__ void brick_coords(const Brick& b, int l, int& lz, int
 // y[v, co] = act( bias[co] + sum_{tap, ci} x[v + off(tap), ci] W[co][tap][ci] ) * (mask[v, co] > 0)
 // with zero padding outside the S^3 level; tap = (dz+1)*9 + (dy+1)*3 + (dx+1).
 // NTILES = output channels per CTA / 8.  grid = (bricks, Cout / (8 NTILES)).
+// The chunks of 16 input channels come by cp.async into a ring of a.stages
+// buffers (a load at a time by each thread, a chunk's staging was a chain of
+// nine global latencies, 6 us; 128 -> 128 channels at 8^3: 43 -> 23 us).
 template <int NTILES>
 __global__ void __launch_bounds__(256) conv3_kernel(ConvArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __nv_bfloat16* halo = reinterpret_cast<__nv_bfloat16*>(smem_raw);
-    __nv_bfloat16* wsm = halo + kHaloMax * kHaloStride;
     constexpr int NT = NTILES * 8;
+    constexpr int kStage = kHaloMax * kHaloStride + NT * kWRow;  // bf16 of a buffer: halo, weights
 
     const Brick b = a.brick;
     const int S = a.S;
@@ -94,32 +96,46 @@ __global__ void __launch_bounds__(256) conv3_kernel(ConvArgs a)
 #pragma unroll
     for (int j = 0; j < NTILES; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
 
-    for (int ci0 = 0; ci0 < a.cin; ci0 += 16) {
-        // stage the input brick + halo, 16 channels (two 16-byte pieces per voxel)
-        for (int q = threadIdx.x; q < hv_count * 2; q += blockDim.x) {
-            const int hv = q >> 1, part = q & 1;
-            const int ix = hv % hx, iy = (hv / hx) % hy, iz = hv / (hx * hy);
-            const int gx = x0 + ix - 1, gy = y0 + iy - 1, gz = z0 + iz - 1;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (gx >= 0 && gx < S && gy >= 0 && gy < S && gz >= 0 && gz < S) {
-                const long long v = ((long long)gz * S + gy) * S + gx;
-                val = *reinterpret_cast<const uint4*>(a.in + v * a.ld_in + a.in_off + ci0 + part * 8);
+    const int nchunks = a.cin / 16;
+    auto stage = [&](int chunk) {
+        if (chunk < nchunks) {
+            const int ci0 = chunk * 16;
+            __nv_bfloat16* halo = reinterpret_cast<__nv_bfloat16*>(smem_raw) + (chunk % a.stages) * kStage;
+            __nv_bfloat16* wsm = halo + kHaloMax * kHaloStride;
+            // the input brick + halo, 16 channels (two 16-byte pieces per voxel)
+            for (int q = threadIdx.x; q < hv_count * 2; q += blockDim.x) {
+                const int hv = q >> 1, part = q & 1;
+                const int ix = hv % hx, iy = (hv / hx) % hy, iz = hv / (hx * hy);
+                const int gx = x0 + ix - 1, gy = y0 + iy - 1, gz = z0 + iz - 1;
+                const bool in = gx >= 0 && gx < S && gy >= 0 && gy < S && gz >= 0 && gz < S;
+                const long long v = in ? ((long long)gz * S + gy) * S + gx : 0;
+                cp_async16(halo + hv * kHaloStride + part * 8, a.in + v * a.ld_in + a.in_off + ci0 + part * 8, in);
             }
-            *reinterpret_cast<uint4*>(halo + hv * kHaloStride + part * 8) = val;
+            // the weight chunk: W[co0 + n][tap][ci0 .. ci0+15]
+            for (int q = threadIdx.x; q < NT * 27 * 2; q += blockDim.x) {
+                const int part = q & 1, t = (q >> 1) % 27, n = (q >> 1) / 27;
+                cp_async16(wsm + n * kWRow + t * 16 + part * 8,
+                           a.w + ((long long)(co0 + n) * 27 + t) * a.cin + ci0 + part * 8, true);
+            }
         }
-        // stage the weight chunk: W[co0 + n][tap][ci0 .. ci0+15]
-        for (int q = threadIdx.x; q < NT * 27 * 2; q += blockDim.x) {
-            const int part = q & 1, t = (q >> 1) % 27, n = (q >> 1) / 27;
-            const uint4 val =
-                *reinterpret_cast<const uint4*>(a.w + ((long long)(co0 + n) * 27 + t) * a.cin + ci0 + part * 8);
-            *reinterpret_cast<uint4*>(wsm + n * kWRow + t * 16 + part * 8) = val;
-        }
+        cp_async_commit();  // a group a chunk, empty past the last
+    };
+    const int ahead = a.stages - 1;
+    for (int c = 0; c < ahead; ++c) stage(c);
+    for (int c = 0; c < nchunks; ++c) {
+        if (ahead == 0) stage(c);
+        cp_async_wait(ahead > 1 ? ahead - 1 : 0);  // chunk c has landed
         __syncthreads();
+        if (ahead > 0) stage(c + ahead);  // over chunk c - 1, which every warp has left
+        const __nv_bfloat16* halo = reinterpret_cast<const __nv_bfloat16*>(smem_raw) + (c % a.stages) * kStage;
+        const __nv_bfloat16* wsm = halo + kHaloMax * kHaloStride;
         if (warp_on) {
 #pragma unroll 1
-            for (int t = 0; t < 27; ++t) {
-                const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-                const int off = (dz * hy + dy) * hx + dx;
+            for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+                const int t = (dz + 1) * 9 + r;
+                const int off = (dz * hy + r / 3 - 1) * hx + r % 3 - 1;
                 const __nv_bfloat16* r0 = halo + (hc0 + off) * kHaloStride + tig * 2;
                 const __nv_bfloat16* r1 = halo + (hc1 + off) * kHaloStride + tig * 2;
                 unsigned af[4];
@@ -134,7 +150,7 @@ __global__ void __launch_bounds__(256) conv3_kernel(ConvArgs a)
                 }
             }
         }
-        __syncthreads();
+        if (ahead == 0) __syncthreads();
     }
     if (!warp_on) return;
     // epilogue: bias, ReLU, mask, BF16 store
@@ -189,7 +205,8 @@ size_t conv3_smem_bytes(int cout_tile)
 // The widest tile of output channels that still gives every multiprocessor a
 // block, down to 16: the levels of 16^3 and 8^3 voxels have 32 and 4 bricks, and
 // at 64 channels a tile 32 and 8 blocks ran on 152 multiprocessors (192 -> 64
-// channels at 16^3: 101 us, 82 us with 16; 128 -> 128 at 8^3: 73 us, 43 us).  An
+// channels at 16^3: 101 us, 82 us with 16; 128 -> 128 at 8^3: 73 us, 43 us; before
+// the ring of chunks).  An
 // output channel's sums do not depend on the tile.
 int conv3_tile(int cout, int bricks)
 {
@@ -199,18 +216,32 @@ int conv3_tile(int cout, int bricks)
     return 16;
 }
 
-template <int NTILES>
-static void launch_conv3_t(const ConvArgs& a, int bricks, cudaStream_t s)
+// Buffers of a chunk ring: the shared memory of a multiprocessor divided among
+// the blocks it gets, at least one buffer each (many blocks hide one another's
+// loads; a single block needs its next chunks in flight), at most four.
+int conv3_stages(size_t stage_bytes, int blocks, int chunks)
 {
-    const size_t smem = conv3_smem_bytes(NTILES * 8);
-    conv3_kernel<NTILES><<<dim3(bricks, a.cout / (NTILES * 8)), 256, smem, s>>>(a);
+    const int per_sm = (blocks + 151) / 152;
+    int stages = (int)(kConvSmem / (per_sm * (stage_bytes + 2048)));  // 1 KB a block is the system's; static arrays
+    if (stages > chunks) stages = chunks;
+    if (stages > kConvStages) stages = kConvStages;
+    return stages < 1 ? 1 : stages;
+}
+
+template <int NTILES>
+static void launch_conv3_t(ConvArgs a, int bricks, cudaStream_t s)
+{
+    const int nt = NTILES * 8;
+    const int blocks = bricks * (a.cout / nt);
+    a.stages = conv3_stages(conv3_smem_bytes(nt), blocks, a.cin / 16);
+    conv3_kernel<NTILES><<<dim3(bricks, a.cout / nt), 256, a.stages * conv3_smem_bytes(nt), s>>>(a);
 }
 
 void prepare_conv3()
 {
     const int tiles[4] = {16, 32, 48, 64};
     for (int t : tiles) {
-        const int smem = (int)conv3_smem_bytes(t);
+        const int smem = (int)conv3_smem_max(conv3_smem_bytes(t));
         if (t == 16) cudaFuncSetAttribute(conv3_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (t == 32) cudaFuncSetAttribute(conv3_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (t == 48) cudaFuncSetAttribute(conv3_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -244,7 +275,9 @@ void launch_conv3(ConvArgs a, cudaStream_t s)
 // the way to the registers; it takes an address per row, so a tap is an offset
 // of the rows in the halo.  (Staged transposed, with three shifted copies of
 // the halo in two-byte stores, a brick took 10 us: 273 us for 48 -> 16 channels
-// at 64^3, 155 us now.)
+// at 64^3, 53 us now, 155 without bricks in flight and with
+// the voxels' offsets worked out anew in every brick.)
+constexpr int kWgradStages = 3;  // 2 blocks of 3 x 31 KB on a multiprocessor
 constexpr int kXRow = 24;  // bf16 of a halo voxel: 16 channels and 8 of padding (8 rows meet all 32 banks)
 
 __device__ __forceinline__ void ldmatrix4_trans(unsigned (&r)[4], const __nv_bfloat16* row)
@@ -264,8 +297,9 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     const int S = a.S;
     const int nvox = b.bx * b.by * b.bz;
     constexpr int kGRow = 16 * MT + 8;                     // bf16 of a voxel's gradients, with padding
-    __nv_bfloat16* gs = reinterpret_cast<__nv_bfloat16*>(smem_raw);
-    __nv_bfloat16* xs = gs + 128 * kGRow;                  // the brick's halo
+    const int hx = b.bx + 2, hy = b.by + 2, hz = b.bz + 2;
+    const int ring = 128 * kGRow + hx * hy * hz * kXRow;   // bf16 of a buffer: the gradients, the brick's halo
+    __nv_bfloat16* const smem = reinterpret_cast<__nv_bfloat16*>(smem_raw);
 
     const int nbx = S / b.bx, nby = S / b.by;
     const int nbricks = nbx * nby * (S / b.bz);
@@ -273,11 +307,10 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
     const int ntap = warp < 3 ? 4 : 3;  // taps warp, warp+8, warp+16 (, warp+24)
-    const int hx = b.bx + 2, hy = b.by + 2, hz = b.bz + 2;
     // the row that this lane addresses in each 16-voxel step: of the gradients, tiles (voxels 0-7, 8-15) x (channels
     // 0-7, 8-15) in the order of the A fragment; of the halo in that of two B fragments
     const int rv = lane & 7, mat = lane >> 3;
-    const __nv_bfloat16* const grow = gs + (rv + (mat >> 1) * 8) * kGRow + (mat & 1) * 8;
+    const int grow0 = (rv + (mat >> 1) * 8) * kGRow + (mat & 1) * 8;
     const int xv = rv + (mat & 1) * 8, xc = (mat >> 1) * 8;
     int toff[4];  // the taps' offsets in the halo
 #pragma unroll
@@ -294,40 +327,79 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
 #pragma unroll
             for (int j = 0; j < 2; ++j) acc[q][m][j][0] = acc[q][m][j][1] = acc[q][m][j][2] = acc[q][m][j][3] = 0.0f;
 
+    // this thread's pieces (8 channels of a voxel) of the gradients and of the halo, and its voxel of each 16-voxel
+    // step, by their offsets in a brick: the divisions once, not in every brick
+    constexpr int kPieces = (2 * kHaloMax + 255) / 256;
+    int gvox[MT], hvox[kPieces], xstep[8];  // gvox: offset in the level; hvox: x | y << 8 | z << 16 (-1: no piece)
+#pragma unroll
+    for (int i = 0; i < MT; ++i) {
+        const int l = (threadIdx.x + 256 * i) / (2 * MT);
+        int lz, ly, lx;
+        brick_coords(b, l < nvox ? l : 0, lz, ly, lx);
+        gvox[i] = l < nvox ? (lz * S + ly) * S + lx : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < kPieces; ++i) {
+        const int hv = (threadIdx.x + 256 * i) >> 1;
+        hvox[i] = hv < hx * hy * hz ? (hv % hx) | ((hv / hx) % hy) << 8 | hv / (hx * hy) << 16 : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int l = i * 16 + xv;
+        int lz, ly, lx;
+        brick_coords(b, l < nvox ? l : 0, lz, ly, lx);  // past nvox any voxel: its gradients are zero
+        xstep[i] = (((lz + 1) * hy + (ly + 1)) * hx + (lx + 1)) * kXRow + xc;
+    }
+    // a brick's operands by cp.async, two bricks ahead
+    auto stage = [&](int brick, int slot) {
+        if (brick < nbricks) {
+            __nv_bfloat16* const gs = smem + slot * ring;
+            __nv_bfloat16* const xs = gs + 128 * kGRow;
+            const int x0 = (brick % nbx) * b.bx, y0 = ((brick / nbx) % nby) * b.by, z0 = (brick / (nbx * nby)) * b.bz;
+            const long long v0 = ((long long)z0 * S + y0) * S + x0;
+            // 16 MT channels of nvox voxels (voxels past nvox are zero)
+#pragma unroll
+            for (int i = 0; i < MT; ++i) {
+                const int piece = threadIdx.x + 256 * i, l = piece / (2 * MT), part = piece % (2 * MT);
+                const bool in = gvox[i] >= 0;
+                cp_async16(gs + l * kGRow + part * 8, a.g + (v0 + (in ? gvox[i] : 0)) * a.ld_g + a.g_off + co0 + part * 8,
+                           in);
+            }
+#pragma unroll
+            for (int i = 0; i < kPieces; ++i) {
+                if (hvox[i] < 0) continue;
+                const int piece = threadIdx.x + 256 * i, part = piece & 1;
+                const int gx = x0 + (hvox[i] & 255) - 1, gy = y0 + (hvox[i] >> 8 & 255) - 1, gz = z0 + (hvox[i] >> 16) - 1;
+                const bool in = gx >= 0 && gx < S && gy >= 0 && gy < S && gz >= 0 && gz < S;
+                const long long v = in ? (gz * S + gy) * S + gx : 0;  // S <= 512: below 2^27
+                cp_async16(xs + (piece >> 1) * kXRow + part * 8, a.x + v * a.ld_x + a.x_off + ci0 + part * 8, in);
+            }
+        }
+        cp_async_commit();
+    };
+    constexpr int kRows = 256 / (16 * MT);
+    float bias = 0.0f;
+    for (int k = 0; k < kWgradStages - 1; ++k) stage(blockIdx.x + k * gridDim.x, k);
+    int slot = 0;
     for (int brick = blockIdx.x; brick < nbricks; brick += gridDim.x) {
-        const int x0 = (brick % nbx) * b.bx, y0 = ((brick / nbx) % nby) * b.by, z0 = (brick / (nbx * nby)) * b.bz;
-        // 16 MT channels of nvox voxels (voxels past nvox are zero)
-        for (int q = threadIdx.x; q < 128 * 2 * MT; q += blockDim.x) {
-            const int l = q / (2 * MT), part = q % (2 * MT);  // part: 8 channels
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (l < nvox) {
-                int lz, ly, lx;
-                brick_coords(b, l, lz, ly, lx);
-                const long long v = ((long long)(z0 + lz) * S + (y0 + ly)) * S + (x0 + lx);
-                val = *reinterpret_cast<const uint4*>(a.g + v * a.ld_g + a.g_off + co0 + part * 8);
-            }
-            *reinterpret_cast<uint4*>(gs + l * kGRow + part * 8) = val;
-        }
-        for (int q = threadIdx.x; q < hx * hy * hz * 2; q += blockDim.x) {
-            const int part = q & 1, hv = q >> 1;
-            const int ix = hv % hx, iy = (hv / hx) % hy, iz = hv / (hx * hy);
-            const int gx = x0 + ix - 1, gy = y0 + iy - 1, gz = z0 + iz - 1;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (gx >= 0 && gx < S && gy >= 0 && gy < S && gz >= 0 && gz < S) {
-                const long long v = ((long long)gz * S + gy) * S + gx;
-                val = *reinterpret_cast<const uint4*>(a.x + v * a.ld_x + a.x_off + ci0 + part * 8);
-            }
-            *reinterpret_cast<uint4*>(xs + hv * kXRow + part * 8) = val;
-        }
+        cp_async_wait(kWgradStages - 2);
         __syncthreads();
-        for (int s = 0; s * 16 < nvox; ++s) {
+        // over the brick before, which every warp has left
+        stage(brick + (kWgradStages - 1) * gridDim.x, slot > 0 ? slot - 1 : kWgradStages - 1);
+        if (blockIdx.z == 0) {  // bias gradient: channel threadIdx.x % (16 MT), every kRows-th voxel
+            const __nv_bfloat16* const col = smem + slot * ring + (threadIdx.x / (16 * MT)) * kGRow + threadIdx.x % (16 * MT);
+#pragma unroll
+            for (int l = 0; l < 128; l += kRows) bias += __bfloat162float(col[l * kGRow]);
+        }
+        const __nv_bfloat16* const grow = smem + slot * ring + grow0;
+        const __nv_bfloat16* const xs = smem + slot * ring + 128 * kGRow;
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            if (s * 16 >= nvox) break;
             unsigned af[MT][4];  // co x voxel, shared by the warp's taps
 #pragma unroll
             for (int m = 0; m < MT; ++m) ldmatrix4_trans(af[m], grow + s * 16 * kGRow + m * 16);
-            const int l = s * 16 + xv;
-            int lz, ly, lx;
-            brick_coords(b, l < nvox ? l : 0, lz, ly, lx);  // past nvox any voxel: its gradients are zero
-            const __nv_bfloat16* xrow = xs + (((lz + 1) * hy + (ly + 1)) * hx + (lx + 1)) * kXRow + xc;
+            const __nv_bfloat16* const xrow = xs + xstep[s];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if (q < ntap) {
@@ -340,7 +412,16 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
                 }
             }
         }
+        slot = slot + 1 < kWgradStages ? slot + 1 : 0;
+    }
+    if (blockIdx.z == 0) {
+        __shared__ float red[256];
+        red[threadIdx.x] = bias;
         __syncthreads();
+        if (threadIdx.x < 16 * MT) {
+            for (int r = 1; r < kRows; ++r) bias += red[r * 16 * MT + threadIdx.x];
+            a.bias_part[(long long)blockIdx.x * a.cout + co0 + threadIdx.x] = bias;
+        }
     }
     // partials: part[blk][co (16 MT)][27][16]
     const long long blk = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -362,35 +443,55 @@ __global__ void __launch_bounds__(256) wgrad_kernel(WgradArgs a)
     }
 }
 
-// dW[co][tap][ci] (+)= sum over the vblocks of the partials: 8 threads an
-// element take every 8th block each, and their sums are added in order (one
-// thread an element, with up to 304 dependent reads, took 24 us on 27 blocks).
-constexpr int kSlices = 8;
-
-__global__ void __launch_bounds__(32 * kSlices)
-wgrad_reduce_kernel(const float* __restrict__ part, int vblocks, int mt, int cout, int cin, float* __restrict__ dw,
-                    int accumulate)
+// dW[co][tap][ci] (+)= sum over the vblocks of the partials: SLICES threads an
+// element take every SLICES-th block each, and their sums are added in order
+// (one thread an element, with up to 304 dependent reads on 27 blocks, took
+// 24 us, 32 threads 7; with 4 blocks one thread an element reads them at once).
+// Four input channels a thread.  The blocks past the weights' add the bias
+// gradient's partials, a warp a channel (lane l takes the vblocks l, l + 32, ..).
+template <int SLICES>
+__global__ void __launch_bounds__(256)
+wgrad_reduce_kernel(const float* __restrict__ part, const float* __restrict__ bias_part, int vblocks, int mt, int cout,
+                    int cin, float* __restrict__ dw, float* __restrict__ db, int accumulate)
 {
-    __shared__ float sum[kSlices][32];
+    constexpr int kElems = 256 / SLICES;
+    __shared__ float4 sum[SLICES][kElems];
     const int total = cout * 27 * cin;
+    const int wblocks = (total / 4 + kElems - 1) / kElems;
+    if (blockIdx.x >= wblocks) {
+        const int c = (blockIdx.x - wblocks) * 8 + (threadIdx.x >> 5);  // cout is a multiple of 8
+        float s = 0.0f;
+        for (int vb = threadIdx.x & 31; vb < vblocks; vb += 32) s += bias_part[(long long)vb * cout + c];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) db[c] = accumulate ? db[c] + s : s;
+        return;
+    }
     const int tile_co = 16 * mt;
-    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
-    const int e = blockIdx.x * 32 + lane;
-    float s = 0.0f;
+    const int lane = threadIdx.x % kElems, slice = threadIdx.x / kElems;
+    const int e = 4 * (blockIdx.x * kElems + lane);
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (e < total) {
         const int ci = e % cin, t = (e / cin) % 27, co = e / (27 * cin);
         const long long blk0 = ((long long)(ci / 16) * (cout / tile_co) + co / tile_co) * vblocks;
         const float* at = part + blk0 * (tile_co * 27 * 16) + ((long long)(co % tile_co) * 27 + t) * 16 + (ci % 16);
-#pragma unroll 4
-        for (int vb = slice; vb < vblocks; vb += kSlices) s += at[(long long)vb * (tile_co * 27 * 16)];
+#pragma unroll 5
+        for (int vb = slice; vb < vblocks; vb += SLICES) {
+            const float4 w = *reinterpret_cast<const float4*>(at + (long long)vb * (tile_co * 27 * 16));
+            s.x += w.x, s.y += w.y, s.z += w.z, s.w += w.w;
+        }
     }
-    sum[slice][lane] = s;
-    __syncthreads();
-    if (slice == 0 && e < total) {
-        float v = sum[0][lane];
-#pragma unroll
-        for (int q = 1; q < kSlices; ++q) v += sum[q][lane];
-        dw[e] = accumulate ? dw[e] + v : v;
+    if (SLICES > 1) {
+        sum[slice][lane] = s;
+        __syncthreads();
+        if (slice == 0)
+            for (int q = 1; q < SLICES; ++q) {
+                const float4 w = sum[q][lane];
+                s.x += w.x, s.y += w.y, s.z += w.z, s.w += w.w;
+            }
+    }
+    if (slice == 0 && e < total) {  // (a layer's offset in the gradients need not be a multiple of 16 bytes)
+        const float v[4] = {s.x, s.y, s.z, s.w};
+        for (int k = 0; k < 4; ++k) dw[e + k] = accumulate ? dw[e + k] + v[k] : v[k];
     }
 }
 
@@ -398,7 +499,7 @@ int wgrad_mt(int cout) { return cout % 32 == 0 ? 2 : 1; }
 
 size_t wgrad_smem_bytes(int mt, const Brick& b)
 {
-    return sizeof(__nv_bfloat16) * (size_t)(128 * (16 * mt + 8) + (b.bx + 2) * (b.by + 2) * (b.bz + 2) * kXRow);
+    return kWgradStages * sizeof(__nv_bfloat16) * (size_t)(128 * (16 * mt + 8) + (b.bx + 2) * (b.by + 2) * (b.bz + 2) * kXRow);
 }
 
 int wgrad_vblocks(int S, int cout, int cin, int sms)
@@ -406,7 +507,7 @@ int wgrad_vblocks(int S, int cout, int cin, int sms)
     const Brick b = brick_for(S);
     const int nbricks = (S / b.bx) * (S / b.by) * (S / b.bz);
     const int tiles = (cout / (16 * wgrad_mt(cout))) * (cin / 16);
-    int vb = (2 * sms + tiles - 1) / tiles;
+    int vb = 2 * sms / tiles;  // one wave: two blocks a multiprocessor
     if (vb > nbricks) vb = nbricks;
     return vb < 1 ? 1 : vb;
 }
@@ -418,7 +519,7 @@ void prepare_wgrad()
     cudaFuncSetAttribute(wgrad_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem_bytes(2, b));
 }
 
-void launch_wgrad(WgradArgs a, int vblocks, float* dw, int accumulate, cudaStream_t s)
+void launch_wgrad(WgradArgs a, int vblocks, float* dw, float* db, int accumulate, cudaStream_t s)
 {
     a.brick = brick_for(a.S);
     const int mt = wgrad_mt(a.cout);
@@ -428,8 +529,17 @@ void launch_wgrad(WgradArgs a, int vblocks, float* dw, int accumulate, cudaStrea
         wgrad_kernel<2><<<grid, 256, smem, s>>>(a);
     else
         wgrad_kernel<1><<<grid, 256, smem, s>>>(a);
-    const int total = a.cout * 27 * a.cin;
-    wgrad_reduce_kernel<<<(total + 31) / 32, 32 * kSlices, 0, s>>>(a.part, vblocks, mt, a.cout, a.cin, dw, accumulate);
+    const int total4 = a.cout * 27 * a.cin / 4, bb = a.cout / 8;
+    const float *wp = a.part, *bp = a.bias_part;
+    if (vblocks <= 4)
+        wgrad_reduce_kernel<1><<<(total4 + 255) / 256 + bb, 256, 0, s>>>(wp, bp, vblocks, mt, a.cout, a.cin, dw, db,
+                                                                         accumulate);
+    else if (vblocks <= 64)
+        wgrad_reduce_kernel<8><<<(total4 + 31) / 32 + bb, 256, 0, s>>>(wp, bp, vblocks, mt, a.cout, a.cin, dw, db,
+                                                                       accumulate);
+    else
+        wgrad_reduce_kernel<32><<<(total4 + 7) / 8 + bb, 256, 0, s>>>(wp, bp, vblocks, mt, a.cout, a.cin, dw, db,
+                                                                      accumulate);
 }
 
 // ---------------------------------------------------------------------------
@@ -449,56 +559,6 @@ __device__ __forceinline__ void store8(__nv_bfloat16* p, const Bf8& r)
     uint4 w;
     memcpy(&w, &r, sizeof w);
     *reinterpret_cast<uint4*>(p) = w;
-}
-
-// ---------------------------------------------------------------------------
-// Bias gradient: db[c] (+)= sum_v g[v, c]: partial sums per block (fixed order),
-// then a warp a channel adds the blocks' (lane l takes blocks l, l + 32, ..).
-__global__ void __launch_bounds__(256) colsum_kernel(const __nv_bfloat16* __restrict__ g, int ld, int off, int C,
-                                                     long long nvox, float* __restrict__ part)
-{
-    // block: C / 8 groups of channels x (2048 / C) row lanes (C divides 2048)
-    const int groups = C / 8;
-    const int c = threadIdx.x % groups, lane = threadIdx.x / groups, lanes = 256 / groups;
-    const long long chunk = (nvox + gridDim.x - 1) / gridDim.x;
-    const long long v0 = blockIdx.x * chunk, v1 = v0 + chunk < nvox ? v0 + chunk : nvox;
-    float s[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[q] = 0.0f;
-    for (long long v = v0 + lane; v < v1; v += lanes) {
-        const Bf8 w = load8(g + v * ld + off + 8 * c);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) s[q] += __bfloat162float(w.v[q]);
-    }
-    __shared__ float red[8][256];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = s[q];
-    __syncthreads();
-    if ((int)threadIdx.x < C) {
-        const int q = threadIdx.x % 8, cc = threadIdx.x / 8;
-        float t = 0.0f;
-        for (int r = 0; r < lanes; ++r) t += red[q][r * groups + cc];
-        part[(long long)blockIdx.x * C + threadIdx.x] = t;
-    }
-}
-
-__global__ void colsum_reduce_kernel(const float* __restrict__ part, int nb, int C, float* __restrict__ out,
-                                     int accumulate)
-{
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (c >= C) return;
-    float s = 0.0f;
-    for (int b = lane; b < nb; b += 32) s += part[(long long)b * C + c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) out[c] = accumulate ? out[c] + s : s;
-}
-
-void launch_bias_grad(const __nv_bfloat16* g, int ld, int off, int C, long long nvox, float* part, int nb, float* db,
-                      int accumulate, cudaStream_t s)
-{
-    // the layer widths are 16, 32, 64 and 128
-    colsum_kernel<<<nb, 256, 0, s>>>(g, ld, off, C, nvox, part);
-    colsum_reduce_kernel<<<(C + 3) / 4, 128, 0, s>>>(part, nb, C, db, accumulate);
 }
 
 // ---------------------------------------------------------------------------
