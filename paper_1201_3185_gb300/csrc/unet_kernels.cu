@@ -187,12 +187,22 @@ Brick brick_for(int S)
 {
     // 128 voxels where the level allows (two planes of 4 rows of 16), else the whole level
     Brick b;
-    if (S >= 16) {
+    if (S % 16 == 0) {
         b.bz = 2, b.by = 4, b.bx = 16;
     } else if (S == 8) {
         b.bz = 2, b.by = 8, b.bx = 8;
-    } else {
+    } else if (S <= 4) {
         b.bz = S, b.by = S, b.bx = S;  // S = 4: 64 voxels; S = 2: 8
+    } else {
+        // the coarse levels of a size that is no power of two (24, 12 and 6 of 48): the most voxels, up to 128, of a
+        // brick that divides the level and whose halo fits its buffer
+        b.bz = b.by = b.bx = 1;
+        for (int z = 1; z <= S; ++z)
+            for (int y = 1; y <= S && z * y <= 128; ++y)
+                for (int x = 1; x <= S && z * y * x <= 128; ++x)
+                    if (S % z == 0 && S % y == 0 && S % x == 0 && (z + 2) * (y + 2) * (x + 2) <= kHaloMax &&
+                        z * y * x > b.bz * b.by * b.bx)
+                        b.bz = z, b.by = y, b.bx = x;
     }
     return b;
 }

@@ -168,9 +168,10 @@ def test_boundary_from_the_parent(q, ora, n, ratio, sets):
     ctx.close()
 
 
-@pytest.mark.parametrize("S,tensor_path", [(64, 1), (64, 0), (32, 0)])
+@pytest.mark.parametrize("S,tensor_path", [(64, 1), (64, 0), (32, 0), (48, 1), (80, 0)])
 def test_guess_gradients_on_all_tile_widths(q, S, tensor_path):
-    """Levels of 64^3 to 4^3 voxels: every width of the channel tile, and weight gradients over 2048 bricks to one.
+    """Levels of 64^3 to 4^3 voxels: every width of the channel tile, and weight gradients over 2048 bricks to one;
+    48 and 80: levels of 24, 12, 6 and of 40, 20, 10 voxels, which no power of two divides into bricks.
     The bounds are those of the gradient test of the smaller networks (14 layers of BF16 rounding: 3 % of the whole
     vector, 15 % of a block whose terms cancel); a wrong tap, channel or voxel moves a block by tens of percent."""
     from oracle import unet as U
