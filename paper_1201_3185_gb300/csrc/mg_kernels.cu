@@ -1545,6 +1545,193 @@ __device__ __forceinline__ unsigned cluster_rank()
     return r;
 }
 
+// ---------------------------------------------------------------------------
+// The coarse solver from the 16-interval level in FP64, on one cluster of eight
+// CTAs per set: coarse_run<double, 3>, a V-cycle from zero or the full multigrid
+// with its ncycle V-cycles.  On one multiprocessor a V-cycle is bound by the two
+// FP64 lanes a clock: the 3375 nodes take eight operations in each of four sweeps
+// and twelve in the residual, 71 of 90 us.  (A 129^3 solve with six V-cycles a level,
+// 18 V-cycles and the full multigrid here: 1704 -> 834 us, launches included; the
+// levels 2 .. 8, in CTA 0, are half of the rest.)  CTA r owns the planes 2r + 1 and 2r + 2, a
+// thread one node of each colour; a node's new value also goes to the CTA whose
+// slab its plane borders (distributed shared memory), so that every read is
+// local.  The arithmetic is that of sm_relax, sm_residual, sm_restrict,
+// sm_prolong and sm_correct.
+constexpr int kDeep = 8;             // CTAs: two of the 15 interior planes each
+constexpr int kDeepThreads = 256;    // 2 planes x 15 rows x 8 nodes of a colour
+constexpr int kDeepPlane = 17 * 17;
+
+size_t deep_smem_bytes()
+{
+    int elems = 7 * kDeepPlane + 1;  // u: four planes, residuals: three; kept even
+    for (int l = 0; l < 3; ++l) elems += coarse_elems(2 << l);
+    return sizeof(double) * elems;
+}
+
+__global__ void __cluster_dims__(kDeep, 1, 1) __launch_bounds__(kDeepThreads)
+coarse_deep_kernel(int fmg, double* __restrict__ e, const double* __restrict__ f, LevelView v, double h,
+                   const double* __restrict__ u64, int nfine, int ncycle, int npre, int npost,
+                   const SolveState* __restrict__ act)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int P = 17, PP = kDeepPlane;
+    const int set = (int)blockIdx.x / kDeep, rank = (int)cluster_rank(), t = (int)threadIdx.x;
+    if (act && !act[set].cont) return;  // the whole cluster reads the same flag
+    e += (long long)set * 2 * v.cs;
+    f += (long long)set * 2 * v.cs;
+    if (u64) u64 += set * nat_elems(nfine);
+    double* const u = reinterpret_cast<double*>(smem_raw);  // slot p: plane k0 - 1 + p
+    double* const res = u + 4 * PP;                         // planes k0, k0 + 1, k0 + 2
+    CoarseSmem<double> S;
+    coarse_layout(S, res + 3 * PP + 1, 2);
+    const int k0 = 2 * rank + 1;
+    const double h2 = h * h, ih2 = 1.0 / (h * h);
+
+    // this thread's node of each colour (sm_relax's slots), at o in u
+    const int kk = t / 120, j = t % 120 / 8 + 1, m = t % 8, k = k0 + kk;
+    const bool row_on = kk < 2 && k < 16;
+    int o[2];
+    bool on[2];
+    double fv[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int i = 1 + (((1 + j + k) & 1) != c ? 1 : 0) + 2 * m;
+        on[c] = row_on && i < 16;
+        o[c] = on[c] ? i + P * j + PP * (kk + 1) : P + 1 + PP;
+        fv[c] = on[c] ? f[node_off(v, i, j, k)] : 0.0;
+    }
+    // plane k0 is slot 3 of the CTA below, plane k0 + 1 slot 0 of the one above
+    double* push = nullptr;
+    if (row_on && kk == 0 && rank > 0) push = cluster_map(u, rank - 1) + 2 * PP;
+    if (row_on && kk == 1 && rank < kDeep - 1) push = cluster_map(u, rank + 1) - 2 * PP;
+    double* const below = row_on && kk == 0 && rank > 0 ? cluster_map(res, rank - 1) + 2 * PP : nullptr;
+
+    // zeros, or the boundary values injected from the finest grid
+    for (int p = t; p < 4 * PP; p += kDeepThreads) {
+        const int i = p % P, jj = p / P % P, kp = k0 - 1 + p / PP;
+        const bool inner = i > 0 && i < 16 && jj > 0 && jj < 16 && kp > 0 && kp < 16;
+        double val = 0.0;
+        if (fmg && u64 && !inner && kp <= 16) {
+            const long long st = nfine / 16, PF = nfine + 1;
+            val = u64[i * st + PF * (jj * st + PF * (kp * st))];
+        }
+        u[p] = val;
+    }
+    for (int p = t; p < 3 * PP; p += kDeepThreads) res[p] = 0.0;
+    if (rank == 0)
+        for (int p = t; p < cube(8); p += kDeepThreads) S.u[2][p] = S.f[2][p] = 0.0;
+    cluster_sync_all();
+
+    auto sum6 = [&](int at) {
+        return (u[at + 1] + u[at - 1]) + (u[at + P] + u[at - P]) + (u[at + PP] + u[at - PP]);
+    };
+    auto set_node = [&](int c, double x, bool remote) {
+        u[o[c]] = x;
+        if (push && remote) push[o[c]] = x;
+    };
+    auto relax = [&](int c, bool zero, bool remote) {
+        if (on[c]) set_node(c, fused(-h2, fv[c], zero ? 0.0 : sum6(o[c])) * (1.0 / 6.0), remote);
+    };
+    // res on this slab, the first plane's values also as the third plane of the CTA below
+    auto set_res = [&](int c, double r) {
+        res[o[c] - PP] = r;
+        if (below) below[o[c] - PP] = r;
+    };
+    // the full weighting of res on the coarse plane rank + 1, whose fine plane is k0 + 1, into CTA 0
+    auto restrict_res = [&]() {
+        if (rank < kDeep - 1 && t < 49) {
+            const int I = t % 7 + 1, J = t / 7 + 1;
+            double acc = 0.0;
+#pragma unroll
+            for (int c = -1; c <= 1; ++c)
+#pragma unroll
+                for (int b = -1; b <= 1; ++b)
+#pragma unroll
+                    for (int a = -1; a <= 1; ++a) {
+                        const double w = 0.125 * (a == 0 ? 2 : 1) * (b == 0 ? 2 : 1) * (c == 0 ? 2 : 1) * 0.125;
+                        acc += w * res[(2 * I + a) + P * (2 * J + b) + PP * (1 + c)];
+                    }
+            cluster_map(S.f[2], 0)[I + 9 * (J + 9 * (rank + 1))] = acc;
+        }
+    };
+    // the coarse planes rank and rank + 1, copied once from CTA 0; their interpolation
+    auto fetch_coarse = [&]() {
+        if (rank != 0) {
+            if (t < 162) S.u[2][81 * rank + t] = cluster_map(S.u[2], 0)[81 * rank + t];
+            __syncthreads();
+        }
+    };
+    auto interpolated = [&](int c) {
+        const int i = o[c] % P;
+        const int I0 = i >> 1, I1 = (i + 1) >> 1, J0 = j >> 1, J1 = (j + 1) >> 1, K0 = k >> 1, K1 = (k + 1) >> 1;
+        const double* const w = S.u[2];
+        double sum = (w[I0 + 9 * (J0 + 9 * K0)] + w[I1 + 9 * (J0 + 9 * K0)])
+                   + (w[I0 + 9 * (J1 + 9 * K0)] + w[I1 + 9 * (J1 + 9 * K0)]);
+        sum += (w[I0 + 9 * (J0 + 9 * K1)] + w[I1 + 9 * (J0 + 9 * K1)])
+             + (w[I0 + 9 * (J1 + 9 * K1)] + w[I1 + 9 * (J1 + 9 * K1)]);
+        return sum * 0.125;
+    };
+
+    if (fmg) {  // the levels 2 .. 8 in CTA 0, then the first values of this one
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (on[c]) set_res(c, fv[c]);
+        cluster_sync_all();
+        restrict_res();
+        cluster_sync_all();
+        if (rank == 0) {
+            sm_restrict_down<double, 2>(S);
+            sm_inject<double, 2>(S, u64, nfine);
+            __syncthreads();
+            sm_fmg_up<double, 2>(S, h * 8.0, ncycle, npre, npost);
+        }
+        cluster_sync_all();
+        fetch_coarse();
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (on[c]) set_node(c, interpolated(c), true);
+        cluster_sync_all();
+    } else {
+        ncycle = 1;
+    }
+    for (int cycle = 0; cycle < ncycle; ++cycle) {
+        for (int q = 0; q < npre; ++q) {
+            relax(0, !fmg && q == 0, true);
+            cluster_sync_all();
+            relax(1, false, true);
+            cluster_sync_all();
+        }
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (on[c]) set_res(c, fv[c] - (sum6(o[c]) - 6.0 * u[o[c]]) * ih2);
+        cluster_sync_all();
+        restrict_res();
+        cluster_sync_all();
+        if (rank == 0) {
+            sm_fill<double, 8>(S.u[2], 0.0);
+            sm_vcycle<double, 2, true>(S, h * 2.0, npre, npost);
+        }
+        cluster_sync_all();
+        fetch_coarse();
+        if (on[1]) set_node(1, u[o[1]] + interpolated(1), true);
+        cluster_sync_all();
+        // no CTA touches another's shared memory after its last barrier
+        for (int q = 0; q < npost; ++q) {
+            relax(0, false, true);
+            cluster_sync_all();
+            const bool last = cycle == ncycle - 1 && q == npost - 1;
+            relax(1, false, !last);
+            if (!last) cluster_sync_all();
+        }
+    }
+    __syncthreads();
+    // the slab with its boundary nodes, and the planes 0 and 16
+    for (int p = t + (rank == 0 ? 0 : PP); p < 3 * PP; p += kDeepThreads) {
+        const int i = p % P, jj = p / P % P, kp = k0 - 1 + p / PP;
+        e[node_off(v, i, jj, kp)] = u[p];
+    }
+}
+
 using Vec4 = RowVec<float>;
 
 // Half a row of the 32-interval level: nodes i = 16 half + 1 .. 16 half + 16.
@@ -2271,7 +2458,14 @@ cudaError_t launch_coarse(int fmg, T* e, const T* f, const LevelView& v, double 
     case 2: coarse_kernel<T, 0><<<g, kCoarseThreads, bytes, s>>>(fmg, e, f, v, (T)h, u64, nfine, ncycle, npre, npost, act); break;
     case 4: coarse_kernel<T, 1><<<g, kCoarseThreads, bytes, s>>>(fmg, e, f, v, (T)h, u64, nfine, ncycle, npre, npost, act); break;
     case 8: coarse_kernel<T, 2><<<g, kCoarseThreads, bytes, s>>>(fmg, e, f, v, (T)h, u64, nfine, ncycle, npre, npost, act); break;
-    case 16: coarse_kernel<T, 3><<<g, kCoarseThreads, bytes, s>>>(fmg, e, f, v, (T)h, u64, nfine, ncycle, npre, npost, act); break;
+    case 16:
+        if constexpr (sizeof(T) == sizeof(double)) {
+            coarse_deep_kernel<<<kDeep * g, kDeepThreads, deep_smem_bytes(), s>>>(fmg, e, f, v, h, u64, nfine, ncycle, npre,
+                                                                                  npost, act);
+        } else {
+            coarse_kernel<T, 3><<<g, kCoarseThreads, bytes, s>>>(fmg, e, f, v, (T)h, u64, nfine, ncycle, npre, npost, act);
+        }
+        break;
     default: return cudaErrorInvalidValue;  // the coarse solver covers the levels n = 2 .. 16
     }
     return cudaSuccess;
@@ -2515,11 +2709,8 @@ cudaError_t prepare_kernels()
             cudaSuccess ||
         cudaFuncSetAttribute(vslab_kernel<256>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return cudaGetLastError();
-    cudaError_t e = cudaFuncSetAttribute(coarse_kernel<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)coarse_smem_bytes<float>(kCoarseN));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(coarse_kernel<double, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)coarse_smem_bytes<double>(kCoarseN));
+    return cudaFuncSetAttribute(coarse_kernel<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)coarse_smem_bytes<float>(kCoarseN));
 }
 
 void launch_reduce_norms(const double* partials, int nblocks, double* out, cudaStream_t s)

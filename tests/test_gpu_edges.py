@@ -191,3 +191,23 @@ def test_guess_gradients_on_all_tile_widths(q, S, tensor_path):
     for name, sl in U.layer_slices():
         assert rel_l2(got[sl], want[sl]) < 0.15, name
     g.close()
+
+
+@pytest.mark.parametrize("n,npre,npost", [(32, 1, 2), (64, 2, 1)])
+def test_fp64_coarse_levels_of_several_sets(q, n, npre, npost):
+    # one cluster of blocks per set runs the levels from n = 16 down: each set's solve as if alone, bit for bit
+    rng = np.random.default_rng(n)
+    nodes = (n + 1) ** 3
+    rhs = to_dev(rng.uniform(-1.0, 1.0, 3 * nodes))
+    kw = dict(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_FP64, bc_mode=q.QUMOND_BC_ZERO, npre=npre, npost=npost,
+              ncycle=2)
+    ctx = q.Context(nsets=3, **kw)
+    phi = torch.zeros_like(rhs)
+    ctx.qumond_solve_mond(0, rhs, None, phi)
+    ctx.close()
+    ctx = q.Context(**kw)
+    for s in range(3):
+        one = torch.zeros(nodes, dtype=torch.float64, device="cuda")
+        ctx.qumond_solve_mond(0, rhs[s * nodes:(s + 1) * nodes].clone(), None, one)
+        assert torch.equal(one, phi[s * nodes:(s + 1) * nodes])
+    ctx.close()
