@@ -262,10 +262,10 @@ __device__ __forceinline__ void restrict_node(const T* __restrict__ ef, const T*
     fc[node_off(vc, I, J, K)] = T(0.125) * centre + T(0.03125) * edge;
 }
 
-template <typename T>
+// A coarse node a thread, on small FP32 levels.
 __global__ void __launch_bounds__(kBX * kBY)
-restrict_resid_red_kernel(const T* __restrict__ ef, const T* __restrict__ ff, LevelView vf, T* __restrict__ fc,
-                          LevelView vc, T ih2, const SolveState* __restrict__ act)
+restrict_nodes_kernel(const float* __restrict__ ef, const float* __restrict__ ff, LevelView vf, float* __restrict__ fc,
+                          LevelView vc, float ih2, const SolveState* __restrict__ act)
 {
     int kz;
     const int set = set_of(vc.n - 1, kz);
@@ -275,7 +275,51 @@ restrict_resid_red_kernel(const T* __restrict__ ef, const T* __restrict__ ff, Le
     const int J = blockIdx.y * kBY + threadIdx.y + 1;
     const int K = kz + 1;
     if (I >= vc.n || J >= vc.n) return;
-    restrict_node<T>(ef + sf, ff + sf, vf, fc + sc, vc, ih2, I, J, K);
+    restrict_node<float>(ef + sf, ff + sf, vf, fc + sc, vc, ih2, I, J, K);
+}
+
+// FP64: a CTA takes 16 x 4 x 2 coarse nodes and evaluates each red residual under
+// them once into shared memory, 743 for 128 nodes.  With the 13 residuals of every
+// node evaluated anew it is bound by the two FP64 lanes a clock (a 129^3 solve of 36
+// restrictions: 785 us, 510 so, launches included); in FP32 at n = 32 and 64 it is
+// bound by latency, and the second phase costs more (33^3 solve: 398 us, 405 so).
+// The arithmetic is restrict_node's.
+constexpr int kTI = 16, kTJ = 4, kTK = 2;             // coarse nodes of a CTA
+constexpr int kTRow = kTI + 1;                        // red nodes of a fine row
+constexpr int kTRows = 2 * kTJ + 1, kTPlanes = 2 * kTK + 1;
+
+template <typename T>
+__global__ void __launch_bounds__(kTI * kTJ * kTK)
+restrict_tile_kernel(const T* __restrict__ ef, const T* __restrict__ ff, LevelView vf, T* __restrict__ fc,
+                          LevelView vc, T ih2, int zper, const SolveState* __restrict__ act)
+{
+    __shared__ T res[kTPlanes][kTRows][kTRow];
+    int zt;
+    const int set = set_of(zper, zt);
+    if (act && !act[set].cont) return;
+    ef += (long long)set * 2 * vf.cs;
+    ff += (long long)set * 2 * vf.cs;
+    fc += (long long)set * 2 * vc.cs;
+    const int I0 = blockIdx.x * kTI + 1, J0 = blockIdx.y * kTJ + 1, K0 = zt * kTK + 1;
+    const int t = (int)threadIdx.x;
+    for (int w = t; w < kTPlanes * kTRows * kTRow; w += kTI * kTJ * kTK) {
+        const int q = w % kTRow, b = w / kTRow % kTRows, c = w / (kTRow * kTRows);
+        const int j = 2 * J0 - 1 + b, k = 2 * K0 - 1 + c;
+        const int i = 2 * (I0 - 1 + q) + ((j + k) & 1);
+        if (i > 0 && i < vf.n && j < vf.n && k < vf.n) res[c][b][q] = red_residual(ef, ff, vf, i, j, k, ih2);
+    }
+    __syncthreads();
+    const int a = t % kTI, b = t / kTI % kTJ, c = t / (kTI * kTJ);
+    const int I = I0 + a, J = J0 + b, K = K0 + c;
+    if (I >= vc.n || J >= vc.n || K >= vc.n) return;
+    // the coarse node's fine row and plane; odd i = 2I -+ 1 at a and a + 1, even i = 2I at a + 1
+    const T(*p0)[kTRow] = &res[2 * c + 1][2 * b + 1];
+    const T(*pm)[kTRow] = &res[2 * c][2 * b + 1];
+    const T(*pp)[kTRow] = &res[2 * c + 2][2 * b + 1];
+    T edge = (p0[1][a + 1] + p0[1][a]) + (p0[-1][a + 1] + p0[-1][a]);
+    edge += (pp[0][a + 1] + pp[0][a]) + (pm[0][a + 1] + pm[0][a]);
+    edge += (pp[1][a + 1] + pp[-1][a + 1]) + (pm[1][a + 1] + pm[-1][a + 1]);
+    fc[node_off(vc, I, J, K)] = T(0.125) * p0[0][a + 1] + T(0.03125) * edge;
 }
 
 // The same restriction on FP32 levels without recomputation: a CTA owns a
@@ -2401,8 +2445,14 @@ void launch_restrict_resid_red(const T* ef, const T* ff, const LevelView& vf, T*
                                                            rk, zper, sets.act);
         return;
     }
-    restrict_resid_red_kernel<T><<<per_sets(inner_grid(vc.n), sets), dim3(kBX, kBY), 0, s>>>(
-        ef, ff, vf, fc, vc, (T)(1.0 / (hf * hf)), sets.act);
+    const T ih2 = (T)(1.0 / (hf * hf));
+    if constexpr (sizeof(T) == sizeof(float)) {
+        restrict_nodes_kernel<<<per_sets(inner_grid(vc.n), sets), dim3(kBX, kBY), 0, s>>>(ef, ff, vf, fc, vc, ih2, sets.act);
+    } else {
+        const int zper = (int)cdiv(vc.n - 1, kTK);
+        const dim3 grid(cdiv(vc.n - 1, kTI), cdiv(vc.n - 1, kTJ), (unsigned)(zper * sets.n));
+        restrict_tile_kernel<T><<<grid, kTI * kTJ * kTK, 0, s>>>(ef, ff, vf, fc, vc, ih2, zper, sets.act);
+    }
 }
 
 template <typename T>

@@ -211,3 +211,20 @@ def test_fp64_coarse_levels_of_several_sets(q, n, npre, npost):
         ctx.qumond_solve_mond(0, rhs[s * nodes:(s + 1) * nodes].clone(), None, one)
         assert torch.equal(one, phi[s * nodes:(s + 1) * nodes])
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [64, 128])
+def test_fp64_restriction_tiles(q, ora, n):
+    # coarse grids of 31 and 63 nodes against tiles of 16 x 4 x 2: a remainder on every side
+    rng = np.random.default_rng(n)
+    f = rng.uniform(-1.0, 1.0, (n + 1) ** 3)
+    u = rng.uniform(-1.0, 1.0, (n + 1) ** 3)
+    want = u.copy()
+    ora.fmg(n, 64.0 / n, want, f, 1, 1, 1)
+    ctx = q.Context(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_FP64, bc_mode=q.QUMOND_BC_GIVEN, npre=1, npost=1,
+                    ncycle=1)
+    phi = to_dev(u)
+    ctx.qumond_solve_mond(0, to_dev(f), None, phi)
+    # the same iterates, summed in another order
+    assert np.max(np.abs(phi.cpu().numpy() - want)) <= 1e-11 * np.max(np.abs(want))
+    ctx.close()
