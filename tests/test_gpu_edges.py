@@ -94,8 +94,8 @@ def _mond(q, src, phi0, n, box, **kw):
     return phi
 
 
-@pytest.mark.parametrize("n,sets,ncycle", [(64, 1, 2), (64, 5, 1), (128, 1, 1), (128, 3, 2), (256, 1, 1), (256, 2, 1),
-                                           (512, 1, 1)])
+@pytest.mark.parametrize("n,sets,ncycle", [(32, 1, 2), (32, 7, 1), (64, 1, 2), (64, 5, 1), (128, 1, 1), (128, 3, 2),
+                                           (256, 1, 1), (256, 2, 1), (512, 1, 1)])
 def test_whole_sweeps_give_the_bits_of_the_half_sweeps(q, n, sets, ncycle):
     # full multigrid without a tolerance: with zero boundary values by bc_mode ZERO each level's V-cycles run as whole
     # sweeps, with zeros given by the caller (GIVEN) as half-sweeps, restriction and prolongation of their own
