@@ -79,7 +79,6 @@ void launch_conv3(ConvArgs a, cudaStream_t s);
 // tcgen05 path (unet_tc.cu)
 int tc_selftest();
 bool conv3_tc_applies(const ConvArgs& a);
-size_t conv3_tc_smem_bytes(int nt);
 void prepare_conv3_tc();
 void launch_conv3_tc(ConvArgs a, cudaStream_t s);
 

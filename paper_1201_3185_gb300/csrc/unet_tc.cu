@@ -3,8 +3,8 @@
 // channels, K = 27 taps x 16 input channels per chunk, accumulated in tensor
 // memory (TMEM) and read back by the four warps for the epilogue.
 //
-// Layout trick: the input brick of a CTA is 1 x 16 x 8 voxels (z, y, x) and
-// its halo 3 x 18 x 10; the halo of a 16-channel chunk is kept in shared
+// Layout trick: the input brick of a CTA is 1 or 2 x 16 x 8 voxels (z, y, x) and
+// its halo 3 or 4 x 18 x 10; the halo of a 16-channel chunk is kept in shared
 // memory as two planes (channels 0-7 and 8-15), 16 bytes per voxel.  Eight
 // consecutive voxels of an x-row are then one 8 x 16-byte core matrix of the
 // canonical K-major layout, the sixteen y-rows are core matrices a constant
@@ -32,13 +32,13 @@ namespace unet {
 
 namespace {
 
-constexpr int kHX = 10, kHY = 18, kHZ = 3;  // halo of a 1 x 16 x 8 brick
-constexpr int kHV = kHX * kHY * kHZ;        // 540 halo voxels
-constexpr unsigned kPlaneBytes = kHV * 16;  // one channel half of the halo
+constexpr int kHX = 10, kHY = 18;  // halo of a ZP x 16 x 8 brick along x and y
+__host__ __device__ constexpr int halo_voxels(int zp) { return kHX * kHY * (zp + 2); }
+__host__ __device__ constexpr unsigned plane_bytes(int zp) { return (unsigned)halo_voxels(zp) * 16; }  // one channel half
 constexpr long long kSpinLimit = 1LL << 24;
 
-// shared memory of one chunk of 16 input channels for NT output channels: halo and weights
-__host__ __device__ constexpr unsigned conv3_tc_stage_bytes(int nt) { return 2 * kPlaneBytes + 27u * 2 * nt * 16; }
+// shared memory of one chunk of 16 input channels for NT output channels and ZP planes: halo and weights
+__host__ __device__ constexpr unsigned conv3_tc_stage_bytes(int nt, int zp) { return 2 * plane_bytes(zp) + 27u * 2 * nt * 16; }
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -198,27 +198,29 @@ __global__ void __launch_bounds__(128) tc_selftest_kernel(float* out, int* fault
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// y = act(conv(x)) on the tensor cores, a brick of 16 x 8 voxels (M = 128) and
-// NT output channels a block.  The chunks of 16 input channels come by cp.async
+// y = act(conv(x)) on the tensor cores, a brick of ZP planes of 16 x 8 voxels
+// (M = 128 each) and NT output channels a block.  The chunks of 16 input channels come by cp.async
 // into a ring of a.stages buffers; the loads of the chunks ahead and the issue
 // of the next 27 MMAs (unrolled: the descriptors are constants beside the base)
 // run while a chunk's MMAs do.  Loaded and issued in turn, a chunk took 7.5 us
 // on an otherwise idle multiprocessor (16^3, 192 -> 64 channels: 82 us), now
 // 2.4 (29 us); 16 -> 16 channels at 64^3: 28 -> 20 us.
-template <int NT>
+template <int NT, int ZP>
 __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    constexpr unsigned kStage = conv3_tc_stage_bytes(NT);  // a chunk: halo (2 planes x kHV x 8), weights (27 x 2 x NT x 8)
+    constexpr unsigned kStage = conv3_tc_stage_bytes(NT, ZP);  // a chunk: halo (2 x kHV x 8), weights (27 x 2 x NT x 8)
+    constexpr int kHV = halo_voxels(ZP);
+    constexpr unsigned kPlaneBytes = plane_bytes(ZP);
     __shared__ __align__(8) unsigned long long bar[2];  // chunk c: bar[c & 1], phase c / 2
     __shared__ unsigned slot;
-    constexpr unsigned kCols = NT <= 32 ? 32 : 64;
+    constexpr unsigned kCols = NT * ZP <= 32 ? 32 : NT * ZP <= 64 ? 64 : 128;
     constexpr unsigned kIdesc = idesc_bf16(NT, 128);
 
     const int S = a.S;
     const int nbx = S / 8, nby = S / 16;
     const int brick = blockIdx.x;
-    const int x0 = (brick % nbx) * 8, y0 = ((brick / nbx) % nby) * 16, z0 = brick / (nbx * nby);
+    const int x0 = (brick % nbx) * 8, y0 = ((brick / nbx) % nby) * 16, z0 = brick / (nbx * nby) * ZP;
     const int co0 = blockIdx.y * NT;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -277,9 +279,12 @@ __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
             for (int t = 0; t < 27; ++t) {
                 const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;  // halo offsets 0..2 of the tap
                 const unsigned aoff = (unsigned)(((dz * kHY + dy) * kHX + dx) * 16);
-                const unsigned long long ad = sdesc(hbase + aoff, kPlaneBytes, kHX * 16);
                 const unsigned long long bd = sdesc(wbase + (unsigned)(t * 2 * NT * 16), NT * 16, 128);
-                mma(taddr, ad, bd, kIdesc, (c > 0 || t > 0) ? 1 : 0);
+#pragma unroll
+                for (int zp = 0; zp < ZP; ++zp) {
+                    const unsigned long long ad = sdesc(hbase + aoff + zp * (kHX * kHY * 16), kPlaneBytes, kHX * 16);
+                    mma(taddr + zp * NT, ad, bd, kIdesc, (c > 0 || t > 0) ? 1 : 0);
+                }
             }
             commit(&bar[c & 1]);
         }
@@ -295,13 +300,13 @@ __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
     // epilogue: warp w holds TMEM lanes 32w..32w+31 = brick voxels 32w + lane
     const int m = warp * 32 + lane;
     const int ly = m / 8, lx = m % 8;
-    const long long v = ((long long)z0 * S + (y0 + ly)) * S + (x0 + lx);
 #pragma unroll
-    for (int c0 = 0; c0 < NT; c0 += 16) {
+    for (int cz = 0; cz < NT * ZP; cz += 16) {  // 16 columns: plane cz / NT, channels cz % NT ..
         float r[16];
-        tmem_ld16(taddr + ((unsigned)(warp * 32) << 16) + (unsigned)c0, r);
+        tmem_ld16(taddr + ((unsigned)(warp * 32) << 16) + (unsigned)cz, r);
         if (!ok) continue;
-        const int co = co0 + c0;
+        const long long v = ((long long)(z0 + cz / NT) * S + (y0 + ly)) * S + (x0 + lx);
+        const int co = co0 + cz % NT;
         __nv_bfloat16 h[16];
         __nv_bfloat16 mk[16];
         if (a.mask) {
@@ -326,7 +331,11 @@ __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
     if (warp == 0) tmem_dealloc(taddr, kCols);
 }
 
-size_t conv3_tc_smem_bytes(int nt) { return conv3_tc_stage_bytes(nt); }
+// Planes of a brick: two share the chunk's weights and two of their halo planes,
+// where the level leaves at least four blocks for every multiprocessor (64^3,
+// 16 -> 16 channels: 20 us with one plane, 18 with two; 48 -> 16: 54 and 47;
+// 16 -> 48: 35 and 27).
+static int conv3_tc_planes(int blocks) { return blocks >= 2 * 4 * 152 ? 2 : 1; }
 
 bool conv3_tc_applies(const ConvArgs& a)
 {
@@ -337,26 +346,40 @@ bool conv3_tc_applies(const ConvArgs& a)
            (!a.mask || (a.ld_mask % 8 == 0 && a.mask_off % 8 == 0));
 }
 
+template <int NT, int ZP>
+static void prepare_tc()
+{
+    cudaFuncSetAttribute(conv3_tc_kernel<NT, ZP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)conv3_smem_max(conv3_tc_stage_bytes(NT, ZP)));
+}
+
 void prepare_conv3_tc()
 {
-    cudaFuncSetAttribute(conv3_tc_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem_max(conv3_tc_smem_bytes(16)));
-    cudaFuncSetAttribute(conv3_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem_max(conv3_tc_smem_bytes(32)));
-    cudaFuncSetAttribute(conv3_tc_kernel<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem_max(conv3_tc_smem_bytes(48)));
-    cudaFuncSetAttribute(conv3_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem_max(conv3_tc_smem_bytes(64)));
+    prepare_tc<16, 1>(), prepare_tc<32, 1>(), prepare_tc<48, 1>(), prepare_tc<64, 1>();
+    prepare_tc<16, 2>(), prepare_tc<32, 2>(), prepare_tc<48, 2>(), prepare_tc<64, 2>();
+}
+
+template <int NT>
+static void launch_tc(ConvArgs a, int bricks, cudaStream_t s)
+{
+    const int tiles = a.cout / NT, zp = conv3_tc_planes(bricks * tiles);
+    const size_t stage = conv3_tc_stage_bytes(NT, zp);
+    const dim3 grid((unsigned)(bricks / zp), (unsigned)tiles);
+    a.stages = conv3_stages(stage, (int)(grid.x * grid.y), a.cin / 16);
+    if (zp == 2)
+        conv3_tc_kernel<NT, 2><<<grid, 128, a.stages * stage, s>>>(a);
+    else
+        conv3_tc_kernel<NT, 1><<<grid, 128, a.stages * stage, s>>>(a);
 }
 
 void launch_conv3_tc(ConvArgs a, cudaStream_t s)
 {
     const int bricks = (a.S / 8) * (a.S / 16) * a.S;
-    const int nt = conv3_tile(a.cout, bricks);
-    const dim3 grid((unsigned)bricks, (unsigned)(a.cout / nt));
-    a.stages = conv3_stages(conv3_tc_smem_bytes(nt), bricks * (a.cout / nt), a.cin / 16);
-    const size_t smem = a.stages * conv3_tc_smem_bytes(nt);
-    switch (nt) {
-    case 64: conv3_tc_kernel<64><<<grid, 128, smem, s>>>(a); break;
-    case 48: conv3_tc_kernel<48><<<grid, 128, smem, s>>>(a); break;
-    case 32: conv3_tc_kernel<32><<<grid, 128, smem, s>>>(a); break;
-    default: conv3_tc_kernel<16><<<grid, 128, smem, s>>>(a); break;
+    switch (conv3_tile(a.cout, bricks)) {
+    case 64: launch_tc<64>(a, bricks, s); break;
+    case 48: launch_tc<48>(a, bricks, s); break;
+    case 32: launch_tc<32>(a, bricks, s); break;
+    default: launch_tc<16>(a, bricks, s); break;
     }
 }
 
