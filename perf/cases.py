@@ -80,8 +80,7 @@ def draw(rng):
     if kind == "whole":
         return dict(kind=kind, n=rng.choice((64, 128)), nboxes=rng.randint(2, 3), particles=_log_int(rng, 1e5, 2e6),
                     nbins=rng.randint(20, 60), nphi=64, dc=rng.randint(2, 4))
-    # powers of two: before the bricks divided every level, 48 (levels of 24, 12 and 6) wrote past a block's shared memory
-    return dict(kind=kind, S=rng.choice((16, 32, 64)), batch=rng.randint(1, 3))
+    return dict(kind=kind, S=rng.choice((16, 32, 48, 64)), batch=rng.randint(1, 3))
 
 
 # --- inputs ---------------------------------------------------------------------------------------------------------
