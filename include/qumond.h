@@ -188,8 +188,9 @@ typedef struct qumond_ctx qumond_ctx;
 QUMOND_API void qumond_default_params(qumond_params* p);
 
 /* Validates p and allocates the context's device scratch on the current
-   device (about 12 (n+1)^3 bytes per set in QUMOND_PREC_MIXED, 20 in FP64,
-   36 in QUMOND_PREC_MIXED_FIXED).
+   device (about 10 (n+1)^3 bytes per set in QUMOND_PREC_MIXED, 20 in FP64,
+   34 in QUMOND_PREC_MIXED_FIXED; with even npre and npost the FP32 modes take
+   up to 2 more for faster sweeps, and do without where they do not fit).
    Returns INVALID_ARG, OUT_OF_MEMORY or CUDA_ERROR on failure (*out = NULL). */
 QUMOND_API qumond_status qumond_create(const qumond_params* p, qumond_ctx** out);
 

@@ -19,7 +19,7 @@ struct Level {
     LevelView v;
     void* e = nullptr;  // iterate / correction, 2 colours
     void* f = nullptr;  // right-hand side, 2 colours
-    float* t = nullptr; // second array of the black colour (FP32 levels that whole sweeps cover)
+    float* t = nullptr; // second array of the black colour (FP32 levels that run as whole sweeps)
     RbMaps maps;        // TMA descriptors of e (FP32 levels with n >= 64)
 };
 
@@ -327,13 +327,9 @@ void rb(qumond_ctx* c, int l, int colour, bool zero, double h, cudaStream_t s)
     });
 }
 
-// Whether level l's V-cycles on a zero-boundary problem run as whole sweeps:
-// the black values alternate between e and t, so both legs of the cycle take
-// an even number of sweeps (other counts go through the half-sweeps).
-inline bool whole_sweeps(const qumond_ctx* c, int l)
-{
-    return c->lev[l].t != nullptr && c->p.npre % 2 == 0 && c->p.npost % 2 == 0;  // each at least 2
-}
+// Whether level l's V-cycles on a zero-boundary problem run as whole sweeps
+// (see sweeps_run); without t through the half-sweeps.
+inline bool whole_sweeps(const qumond_ctx* c, int l) { return c->lev[l].t != nullptr; }
 
 // One red-black sweep in one pass; q: which of its leg (the even ones write t).
 void sweep(qumond_ctx* c, int l, SweepStart start, int q, SweepAfter after, double h, cudaStream_t s)
@@ -902,6 +898,158 @@ qumond_status check_phis(qumond_ctx* c, const double* const* phis, const char* w
     return QUMOND_OK;
 }
 
+// The levels that one kernel's V-cycle covers (params.persistent_vcycle): lc .. vtop, vtop -1 where there is none.
+void choose_small_levels(qumond_ctx* c)
+{
+    const qumond_params& p = c->p;
+    const int lc = c->lc, L = c->L;
+    int top = -1;  // of the levels above lc with n <= 64 below the finest
+    for (int l = lc + 1; l < L; ++l)
+        if (c->lev[l].v.n <= 64) top = l;
+    const bool some = top > lc && top - lc + 1 <= 6;
+    if (p.persistent_vcycle == 2) {
+        // levels lc+1 .. vtop as one thread-block cluster per set
+        const int cs = vcluster_size(p.precision == QUMOND_PREC_FP64);
+        if (cs >= 2 && some) {
+            c->vtop = top;
+            c->vcs = cs;
+        }
+    }
+    if (p.persistent_vcycle == 3 && c->elt == sizeof(float) && lc + 1 < L && c->lev[lc + 1].v.n == 32) {
+        // the 32-interval level (below the finest) and the levels under it in one cluster's shared memory
+        const int cs = vslab_size(p.small_cluster ? p.small_cluster : 8);
+        if (cs > 0) {
+            c->vtop = lc + 1;
+            c->vcs = cs;
+        }
+    }
+    if (p.persistent_vcycle == 1) {
+        // levels lc+1 .. vtop in one cooperative kernel
+        int dev = 0, coop = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (coop && sms > 0 && some) {
+            c->vtop = top;
+            c->vgrid = vsub_grid(sms);
+        }
+    }
+}
+
+// Whether any V-cycle of the context's solves runs level l as whole sweeps.  The black values alternate between two
+// arrays, so both legs take an even number of sweeps; the boundary values are zero: corrections, and the FMG V-cycles
+// of a box whose boundary is zero.  The level vtop is always its own kernel's.
+bool sweeps_run(const qumond_ctx* c, int l)
+{
+    const qumond_params& p = c->p;
+    if (c->elt != sizeof(float) || l <= c->lc || l == c->vtop || !sweep_level(c->lev[l].v.n)) return false;
+    if (p.npre % 2 != 0 || p.npost % 2 != 0) return false;
+    const bool fmg = !p.warm_start, refine = p.rel_tol > 0.0 && p.max_vcycles > 0;
+    if (fmg && p.bc_mode == QUMOND_BC_ZERO) return true;                    // box 0, each level's own V-cycles
+    if (l == c->L) return refine;                                           // the defect correction
+    if (l > c->vtop) return fmg || refine;                                  // corrections of the level above
+    return fmg && l + 1 < c->vtop;                                          // under vtop FMG alone comes by
+}
+
+// sweeps: with the whole sweeps' second black arrays.
+qumond_status create_ctx(const qumond_params* p, bool sweeps, qumond_ctx** out)
+{
+    qumond_ctx* c = new qumond_ctx();
+    qumond_status st = check_params(c, p);
+    if (st != QUMOND_OK) {
+        delete c;
+        return st;
+    }
+    c->p = *p;
+    c->nsets = p->nsets;
+    const size_t ns = (size_t)p->nsets;
+    c->elt = p->precision == QUMOND_PREC_FP64 ? sizeof(double) : sizeof(float);  // FIXED smooths in FP32
+    int L = 0;
+    while ((2 << L) < p->n) ++L;
+    c->L = L;
+    int lc = 0;
+    while ((2 << lc) < kCoarseN && lc < L) ++lc;
+    c->lc = lc;
+    c->lev.resize(L + 1);
+    for (int l = 0; l <= L; ++l) c->lev[l].v = make_view(2 << l);
+    bool ok = prepare_kernels() == cudaSuccess;
+    if (ok) choose_small_levels(c);
+    // every level's arrays in one zeroed allocation, each on a 256-byte boundary
+    auto place = [&](unsigned char* base) {
+        size_t used = 0;
+        auto take = [&](size_t bytes) {
+            unsigned char* at = base ? base + used : nullptr;
+            used += (bytes + 255) & ~(size_t)255;
+            return at;
+        };
+        for (int l = lc; l <= L; ++l) {
+            Level& lv = c->lev[l];
+            const size_t bytes = (size_t)(2 * lv.v.cs) * c->elt * ns;
+            lv.e = take(bytes);
+            lv.f = take(bytes);
+            if (sweeps && sweeps_run(c, l)) lv.t = reinterpret_cast<float*>(take(bytes / 2));
+        }
+        return used;
+    };
+    const size_t pool = place(nullptr);
+    ok = ok && cudaMalloc(&c->pool, pool) == cudaSuccess && cudaMemset(c->pool, 0, pool) == cudaSuccess;
+    if (ok) place(static_cast<unsigned char*>(c->pool));
+    for (int l = lc; ok && l <= L; ++l)
+        if (c->lev[l].t) ok = prepare_sweep_level(c->lev[l].v.n) == cudaSuccess;
+    if (ok) {
+        const int nrows = residual_rows_blocks(p->n > 2 ? p->n : 2);
+        const int nouter = residual_outer_blocks(p->n > 2 ? p->n : 2);
+        c->max_partials = nrows > nouter ? nrows : nouter;
+        c->pstride = 2 * (long long)(c->max_partials + 1);
+        ok = cudaMalloc(&c->partials, sizeof(double) * (size_t)c->pstride * ns) == cudaSuccess &&
+             cudaMalloc(&c->d_norms, sizeof(double) * 2) == cudaSuccess &&
+             cudaMallocHost(&c->h_norms, sizeof(double) * 2) == cudaSuccess &&
+             cudaMalloc(&c->d_state, sizeof(SolveState) * ns) == cudaSuccess &&
+             cudaMallocHost(&c->h_state, sizeof(SolveState) * ns) == cudaSuccess &&
+             cudaMemset(c->d_state, 0, sizeof(SolveState) * ns) == cudaSuccess &&
+             cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
+             cudaMalloc(&c->fault, sizeof(int)) == cudaSuccess && cudaMemset(c->fault, 0, sizeof(int)) == cudaSuccess &&
+             (p->bc_mode != QUMOND_BC_MULTIPOLE ||
+              cudaMalloc(&c->ff, sizeof(double) * far_field_scratch_doubles(p->nsets)) == cudaSuccess);
+        if (ok && c->elt == sizeof(float))
+            for (int l = lc; l <= L; ++l) {
+                make_rb_maps(static_cast<float*>(c->lev[l].e), static_cast<float*>(c->lev[l].f), c->lev[l].v,
+                             &c->lev[l].maps, (int)ns);
+                if (l > 0)
+                    make_prolong_maps(static_cast<float*>(c->lev[l - 1].e), c->lev[l - 1].v,
+                                      static_cast<float*>(c->lev[l].e), c->lev[l].v, &c->lev[l].maps, (int)ns);
+            }
+        if (ok && p->precision == QUMOND_PREC_MIXED_FIXED) {
+            const size_t nn = fixed_elems(p->n) * ns;
+            const int nfix = fixed_residual_blocks(p->n > 2 ? p->n : 2);
+            if (nfix > c->max_partials) ok = false;  // partial buffer sized above covers it
+            ok = ok && cudaMalloc(&c->Ufix, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMalloc(&c->Ufix2, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMalloc(&c->Ffix, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMemset(c->Ufix, 0, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMemset(c->Ufix2, 0, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMemset(c->Ffix, 0, nn * sizeof(int64_t)) == cudaSuccess &&
+                 cudaMalloc(&c->maxbits, sizeof(unsigned) * ns) == cudaSuccess &&
+                 cudaMemset(c->maxbits, 0, sizeof(unsigned) * ns) == cudaSuccess;
+            if (ok && c->elt == sizeof(float)) {
+                const int n = p->n;
+                const long long items = (long long)((n - 1 + 31) / 32) * ((n - 1 + 7) / 8) * ((n - 1 + 15) / 16);
+                if (items <= c->max_partials)
+                    make_fixed_maps(c->Ufix, c->Ufix2, c->Ffix, static_cast<float*>(c->lev[L].e), c->lev[L].v,
+                                    &c->fmaps, (int)ns);
+            }
+        }
+    }
+    if (ok && c->vgrid > 0) ok = cudaMalloc(&c->vbar, sizeof(unsigned)) == cudaSuccess;
+    if (!ok) {
+        (void)cudaGetLastError();
+        qumond_destroy(c);
+        return QUMOND_ERR_OUT_OF_MEMORY;
+    }
+    *out = c;
+    return QUMOND_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -938,138 +1086,9 @@ qumond_status qumond_create(const qumond_params* p, qumond_ctx** out)
 {
     if (!out) return QUMOND_ERR_INVALID_ARG;
     *out = nullptr;
-    qumond_ctx* c = new qumond_ctx();
-    qumond_status st = check_params(c, p);
-    if (st != QUMOND_OK) {
-        delete c;
-        return st;
-    }
-    c->p = *p;
-    c->nsets = p->nsets;
-    const size_t ns = (size_t)p->nsets;
-    c->elt = p->precision == QUMOND_PREC_FP64 ? sizeof(double) : sizeof(float);  // FIXED smooths in FP32
-    int L = 0;
-    while ((2 << L) < p->n) ++L;
-    c->L = L;
-    int lc = 0;
-    while ((2 << lc) < kCoarseN && lc < L) ++lc;
-    c->lc = lc;
-    c->lev.resize(L + 1);
-    // every level's arrays in one zeroed allocation, each on a 256-byte boundary
-    bool ok = true;
-    auto place = [&](unsigned char* base) {
-        size_t used = 0;
-        auto take = [&](size_t bytes) {
-            unsigned char* at = base ? base + used : nullptr;
-            used += (bytes + 255) & ~(size_t)255;
-            return at;
-        };
-        for (int l = lc; l <= L; ++l) {
-            Level& lv = c->lev[l];
-            const size_t bytes = (size_t)(2 * lv.v.cs) * c->elt * ns;
-            lv.e = take(bytes);
-            lv.f = take(bytes);
-            if (c->elt == sizeof(float) && l > lc && sweep_level(lv.v.n))
-                lv.t = reinterpret_cast<float*>(take(bytes / 2));
-        }
-        return used;
-    };
-    for (int l = 0; l <= L; ++l) c->lev[l].v = make_view(2 << l);
-    const size_t pool = place(nullptr);
-    ok = cudaMalloc(&c->pool, pool) == cudaSuccess && cudaMemset(c->pool, 0, pool) == cudaSuccess;
-    if (ok) {
-        place(static_cast<unsigned char*>(c->pool));
-        for (int l = lc; l <= L; ++l)
-            if (c->lev[l].t && prepare_sweep_level(c->lev[l].v.n) != cudaSuccess) ok = false;
-    }
-    if (ok) {
-        const int nrows = residual_rows_blocks(p->n > 2 ? p->n : 2);
-        const int nouter = residual_outer_blocks(p->n > 2 ? p->n : 2);
-        c->max_partials = nrows > nouter ? nrows : nouter;
-        c->pstride = 2 * (long long)(c->max_partials + 1);
-        ok = cudaMalloc(&c->partials, sizeof(double) * (size_t)c->pstride * ns) == cudaSuccess &&
-             cudaMalloc(&c->d_norms, sizeof(double) * 2) == cudaSuccess &&
-             cudaMallocHost(&c->h_norms, sizeof(double) * 2) == cudaSuccess &&
-             cudaMalloc(&c->d_state, sizeof(SolveState) * ns) == cudaSuccess &&
-             cudaMallocHost(&c->h_state, sizeof(SolveState) * ns) == cudaSuccess &&
-             cudaMemset(c->d_state, 0, sizeof(SolveState) * ns) == cudaSuccess &&
-             cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess &&
-             cudaMalloc(&c->fault, sizeof(int)) == cudaSuccess && cudaMemset(c->fault, 0, sizeof(int)) == cudaSuccess &&
-             (p->bc_mode != QUMOND_BC_MULTIPOLE ||
-              cudaMalloc(&c->ff, sizeof(double) * far_field_scratch_doubles(p->nsets)) == cudaSuccess) &&
-             prepare_kernels() == cudaSuccess;
-        if (ok && c->elt == sizeof(float))
-            for (int l = lc; l <= L; ++l) {
-                make_rb_maps(static_cast<float*>(c->lev[l].e), static_cast<float*>(c->lev[l].f), c->lev[l].v,
-                             &c->lev[l].maps, (int)ns);
-                if (l > 0)
-                    make_prolong_maps(static_cast<float*>(c->lev[l - 1].e), c->lev[l - 1].v,
-                                      static_cast<float*>(c->lev[l].e), c->lev[l].v, &c->lev[l].maps, (int)ns);
-            }
-        if (ok && p->precision == QUMOND_PREC_MIXED_FIXED) {
-            const size_t nn = fixed_elems(p->n) * ns;
-            const int nfix = fixed_residual_blocks(p->n > 2 ? p->n : 2);
-            if (nfix > c->max_partials) ok = false;  // partial buffer sized above covers it
-            ok = ok && cudaMalloc(&c->Ufix, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMalloc(&c->Ufix2, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMalloc(&c->Ffix, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMemset(c->Ufix, 0, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMemset(c->Ufix2, 0, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMemset(c->Ffix, 0, nn * sizeof(int64_t)) == cudaSuccess &&
-                 cudaMalloc(&c->maxbits, sizeof(unsigned) * ns) == cudaSuccess &&
-                 cudaMemset(c->maxbits, 0, sizeof(unsigned) * ns) == cudaSuccess;
-            if (ok && c->elt == sizeof(float)) {
-                const int n = p->n;
-                const long long items = (long long)((n - 1 + 31) / 32) * ((n - 1 + 7) / 8) * ((n - 1 + 15) / 16);
-                if (items <= c->max_partials)
-                    make_fixed_maps(c->Ufix, c->Ufix2, c->Ffix, static_cast<float*>(c->lev[L].e), c->lev[L].v,
-                                    &c->fmaps, (int)ns);
-            }
-        }
-    }
-    if (ok && p->persistent_vcycle == 2) {
-        // levels lc+1 .. vtop (n <= 64, below the finest) as one thread-block cluster per set
-        int top = -1;
-        for (int l = c->lc + 1; l < L; ++l)
-            if (c->lev[l].v.n <= 64) top = l;
-        const int cs = vcluster_size(p->precision == QUMOND_PREC_FP64);
-        if (cs >= 2 && top > c->lc && top - c->lc + 1 <= 6) {
-            c->vtop = top;
-            c->vcs = cs;
-        }
-    }
-    if (ok && p->persistent_vcycle == 3 && c->elt == sizeof(float) && lc + 1 < L && c->lev[lc + 1].v.n == 32) {
-        // the 32-interval level (below the finest) and the levels under it in one cluster's shared memory
-        const int cs = vslab_size(p->small_cluster ? p->small_cluster : 8);
-        if (cs > 0) {
-            c->vtop = lc + 1;
-            c->vcs = cs;
-        }
-    }
-    if (ok && p->persistent_vcycle == 1) {
-        // levels lc+1 .. vtop (n <= 64, below the finest) in one cooperative kernel
-        int dev = 0, coop = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        int top = -1;
-        for (int l = c->lc + 1; l < L; ++l)
-            if (c->lev[l].v.n <= 64) top = l;
-        if (coop && sms > 0 && top > c->lc && top - c->lc + 1 <= 6) {
-            ok = cudaMalloc(&c->vbar, sizeof(unsigned)) == cudaSuccess;
-            if (ok) {
-                c->vtop = top;
-                c->vgrid = vsub_grid(sms);
-            }
-        }
-    }
-    if (!ok) {
-        (void)cudaGetLastError();
-        qumond_destroy(c);
-        return QUMOND_ERR_OUT_OF_MEMORY;
-    }
-    *out = c;
-    return QUMOND_OK;
+    // a context that does not fit with the whole sweeps' arrays does without them: half-sweeps, the same bits
+    const qumond_status st = create_ctx(p, true, out);
+    return st == QUMOND_ERR_OUT_OF_MEMORY ? create_ctx(p, false, out) : st;
 }
 
 void qumond_destroy(qumond_ctx* c)

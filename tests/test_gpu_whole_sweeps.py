@@ -1,0 +1,76 @@
+"""Whole red-black sweeps (one pass per sweep, FP32 levels n >= 32): the memory that a context takes for them, and
+their bits against the half-sweeps over the launch shapes they are chosen for."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def q():
+    import paper_1201_3185_gb300 as q
+    return q
+
+
+def _footprint(q, n, **kw):
+    """Device bytes of a context."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    ctx = q.Context(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, **kw)
+    took = before - torch.cuda.mem_get_info()[0]
+    ctx.close()
+    return took
+
+
+def _black(n):
+    """Bytes of the black values of a level of one set: rows padded to four entries."""
+    return 4 * ((n // 2 + 1 + 3) // 4 * 4) * (n + 1) ** 2
+
+
+@pytest.mark.parametrize("n,sets,without,levels", [
+    # (the other context's parameters, the levels whose second black array it does not need)
+    (256, 2, dict(npre=1), (256, 128, 64)),                            # odd counts run half-sweeps
+    (256, 2, dict(npost=3), (256, 128, 64)),
+    (128, 16, dict(bc_mode=1, rel_tol=0.0), (128,)),                   # no correction, every finest V-cycle with
+                                                                       # boundary values: half-sweeps there
+])
+def test_second_black_arrays_only_where_whole_sweeps_run(q, n, sets, without, levels):
+    kw = dict(nsets=sets, rel_tol=1e-8)
+    _footprint(q, n, **kw)  # what the first context of a shape loads for good
+    _footprint(q, n, **{**kw, **without})
+    need = sum(_black(m) for m in levels) * sets
+    # allocations come in blocks of 2 MB
+    assert _footprint(q, n, **kw) - _footprint(q, n, **{**kw, **without}) >= need - 2 * (2 << 20)
+
+
+def test_no_second_black_array_on_the_level_that_a_cluster_runs(q):
+    # n = 32 below n = 64: its V-cycles are one kernel's (form 3) or half and whole sweeps (form 0)
+    n, sets = 64, 512
+    a = _footprint(q, n, nsets=sets, rel_tol=1e-8, persistent_vcycle=3)
+    b = _footprint(q, n, nsets=sets, rel_tol=1e-8, persistent_vcycle=0)
+    assert b - a >= _black(32) * sets - 2 * (2 << 20)
+
+
+@pytest.mark.parametrize("precision,n,sets", [(1, 256, 8), (2, 256, 16)])
+def test_a_context_without_room_for_the_second_black_arrays(q, precision, n, sets):
+    # device memory for the context but for half of those arrays: it is created all the same, and its solves give the
+    # same bits
+    assert (q.QUMOND_PREC_MIXED, q.QUMOND_PREC_MIXED_FIXED) == (1, 2)
+    kw = dict(n=n, nboxes=1, L0=64.0, precision=precision, nsets=sets, rel_tol=1e-8)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    src = torch.rand(sets * (n + 1) ** 3, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    want, got = torch.zeros_like(src), torch.zeros_like(src)
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    ctx = q.Context(**kw)
+    full = free - torch.cuda.mem_get_info()[0]
+    ctx.qumond_solve_mond(0, src, None, want)
+    ctx.close()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - full + _black(n) * sets // 2, dtype=torch.uint8, device="cuda")
+    ctx = q.Context(**kw)
+    ctx.qumond_solve_mond(0, src, None, got)
+    ctx.close()
+    del filler
+    torch.cuda.empty_cache()
+    assert torch.equal(got, want)
