@@ -610,13 +610,23 @@ struct CoarseSmem {
     T* u[kMaxCoarseLevels];
     T* f[kMaxCoarseLevels];
     T* r[kMaxCoarseLevels];
-    T* x[kMaxCoarseLevels];  // row exchange of the levels n >= 8
+    T* x[kMaxCoarseLevels];  // row exchange of the levels run by rows
 };
 
+// Levels whose V-cycle keeps rows in registers (Row below).  In FP64 the pipe (2 operations
+// a clock) bounds these levels, and more threads with a node each keep it
+// busier (17^3 V-cycle 71 us either way, 9^3 17 us against 21).
+template <typename T>
+__host__ __device__ constexpr bool rows_at(int n) { return n >= 8 && sizeof(T) == 4; }
+template <typename T, int L>
+constexpr bool by_rows() { return rows_at<T>(2 << L); }
+
 // Elements of level n in the coarse solver's shared memory: u, f, r and the row exchange.
-__host__ __device__ inline int row_exchange(int n) { return n >= 8 ? (n + 1) * (n + 2) * n : 0; }
+template <typename T>
+__host__ __device__ inline int row_exchange(int n) { return rows_at<T>(n) ? (n + 1) * (n + 2) * n : 0; }
 __host__ __device__ inline int cube4(int n) { return (cube(n) + 3) & ~3; }
-__host__ __device__ inline int coarse_elems(int n) { return 3 * cube4(n) + row_exchange(n); }
+template <typename T>
+__host__ __device__ inline int coarse_elems(int n) { return 3 * cube4(n) + row_exchange<T>(n); }
 
 template <typename T>
 __device__ __forceinline__ void coarse_layout(CoarseSmem<T>& S, T* base, int top)
@@ -626,10 +636,10 @@ __device__ __forceinline__ void coarse_layout(CoarseSmem<T>& S, T* base, int top
         if (l > top) break;
         const int c = cube4(2 << l);
         S.x[l] = base;
-        S.u[l] = base + row_exchange(2 << l);
+        S.u[l] = base + row_exchange<T>(2 << l);
         S.f[l] = S.u[l] + c;
         S.r[l] = S.f[l] + c;
-        base += coarse_elems(2 << l);
+        base += coarse_elems<T>(2 << l);
     }
 }
 
@@ -1176,12 +1186,6 @@ __device__ __forceinline__ void row_vcycle(CoarseSmem<T>& S, Row<T, (2 << L)>& r
     }
 }
 
-// Levels whose V-cycle keeps rows in registers.  In FP64 the pipe (2 operations
-// a clock) bounds these levels, and more threads with a node each keep it
-// busier (17^3 V-cycle 71 us either way, 9^3 17 us against 21).
-template <typename T, int L>
-constexpr bool by_rows() { return L >= 2 && sizeof(T) == 4; }
-
 // V(npre, npost) cycle from level L down to the 3^3 grid; the coarser levels
 // start from zero (zero boundary values), level L from what u[L] holds, or, with
 // ZERO, from zero with zero boundary values (only these are read of u[L], and
@@ -1608,7 +1612,7 @@ constexpr int kDeepPlane = 17 * 17;
 size_t deep_smem_bytes()
 {
     int elems = 7 * kDeepPlane + 1;  // u: four planes, residuals: three; kept even
-    for (int l = 0; l < 3; ++l) elems += coarse_elems(2 << l);
+    for (int l = 0; l < 3; ++l) elems += coarse_elems<double>(2 << l);
     return sizeof(double) * elems;
 }
 
@@ -2349,7 +2353,7 @@ template <typename T>
 size_t coarse_smem_bytes(int n)
 {
     size_t tot = 0;
-    for (int m = 2; m <= n; m *= 2) tot += (size_t)coarse_elems(m);
+    for (int m = 2; m <= n; m *= 2) tot += (size_t)coarse_elems<T>(m);
     return tot * sizeof(T);
 }
 
