@@ -644,26 +644,10 @@ __device__ __forceinline__ void coarse_layout(CoarseSmem<T>& S, T* base, int top
 }
 
 // Every level size is a compile-time constant (N = 2 << L), so the index
-// arithmetic below is shifts and multiplications.  Each routine is run either
-// by the whole block (W = false: stride blockDim.x, a multiple of 8, and a
-// block barrier at the end) or by warp 0 alone (W = true: the levels n <= 4,
-// at most 27 nodes a phase, stride 32 and a warp barrier), which spares the
-// smallest levels a block-wide barrier per phase; the arithmetic of every
-// node is the same either way.
-template <bool W>
-__device__ __forceinline__ int sm_stride()
-{
-    return W ? 32 : (int)blockDim.x;
-}
-
-template <bool W>
-__device__ __forceinline__ void sm_sync()
-{
-    if (W)
-        __syncwarp();
-    else
-        __syncthreads();
-}
+// arithmetic below is shifts and multiplications.  Each routine is run by the
+// whole block (stride blockDim.x, a multiple of 8) and ends with its barrier;
+// the level n = 4 has its own form in one warp (warp_vcycle4), which spares it a
+// block-wide barrier per phase.
 
 // a b + c rounded once (written out: where a product is the same in every
 // sweep, the compiler would round it on its own and keep it).
@@ -676,11 +660,11 @@ __device__ __forceinline__ double fused(double a, double b, double c) { return _
 // row (j, k) without divisions (the residual and the prolongation below do
 // the same with N lanes per row, the last one idle).
 // ZERO: every neighbour is known to be zero.
-template <typename T, int N, bool W = false, bool ZERO = false>
+template <typename T, int N, bool ZERO = false>
 __device__ void sm_relax(T* u, const T* f, T h2, int colour)
 {
     constexpr int M = N - 1, P = N + 1, H = N / 2, ROWS = M * M;
-    const int dr = sm_stride<W>() / H;  // rows advanced per pass
+    const int dr = (int)blockDim.x / H;  // rows advanced per pass
     const int dj = dr % M, dk = dr / M;
     const int sl = (int)threadIdx.x % H;
     int row = (int)threadIdx.x / H;
@@ -700,14 +684,14 @@ __device__ void sm_relax(T* u, const T* f, T h2, int colour)
             ++k;
         }
     }
-    sm_sync<W>();
+    __syncthreads();
 }
 
-template <typename T, int N, bool W = false>
+template <typename T, int N>
 __device__ void sm_residual(const T* u, const T* f, T* r, T ih2)
 {
     constexpr int M = N - 1, P = N + 1, ROWS = M * M;
-    const int dr = sm_stride<W>() / N;  // rows advanced per pass: a row is N lanes, the last one idle
+    const int dr = (int)blockDim.x / N;  // rows advanced per pass: a row is N lanes, the last one idle
     const int dj = dr % M, dk = dr / M;
     const int i = (int)threadIdx.x % N + 1;
     int row = (int)threadIdx.x / N;
@@ -725,14 +709,14 @@ __device__ void sm_residual(const T* u, const T* f, T* r, T ih2)
             ++k;
         }
     }
-    sm_sync<W>();
+    __syncthreads();
 }
 
-template <typename T, int NF, bool W = false>
+template <typename T, int NF>
 __device__ void sm_restrict(const T* fine, T* coarse)
 {
     constexpr int NC = NF / 2, MC = NC - 1, PF = NF + 1, PC = NC + 1, TOT = MC * MC * MC;
-    for (int t = threadIdx.x; t < TOT; t += sm_stride<W>()) {
+    for (int t = threadIdx.x; t < TOT; t += (int)blockDim.x) {
         const int I = t % MC + 1, J = (t / MC) % MC + 1, K = t / (MC * MC) + 1;
         T acc = T(0);
 #pragma unroll
@@ -746,14 +730,14 @@ __device__ void sm_restrict(const T* fine, T* coarse)
                 }
         coarse[I + PC * (J + PC * K)] = acc;
     }
-    sm_sync<W>();
+    __syncthreads();
 }
 
-template <typename T, int NC, bool W = false>
-__device__ void sm_prolong(const T* coarse, T* fine, bool add)
+template <typename T, int NC>
+__device__ void sm_prolong(const T* coarse, T* fine)
 {
     constexpr int NF = 2 * NC, M = NF - 1, PF = NF + 1, PC = NC + 1, ROWS = M * M;
-    const int dr = sm_stride<W>() / NF;  // rows advanced per pass: a row is NF lanes, the last one idle
+    const int dr = (int)blockDim.x / NF;  // rows advanced per pass: a row is NF lanes, the last one idle
     const int dj = dr % M, dk = dr / M;
     const int i = (int)threadIdx.x % NF + 1;
     int row = (int)threadIdx.x / NF;
@@ -767,7 +751,7 @@ __device__ void sm_prolong(const T* coarse, T* fine, bool add)
                  + (coarse[I0 + PC * (J1 + PC * K1)] + coarse[I1 + PC * (J1 + PC * K1)]);
             sum *= T(0.125);
             const int o = i + PF * (j + PF * k);
-            fine[o] = add ? fine[o] + sum : sum;
+            fine[o] = sum;
         }
         j += dj;
         k += dk;
@@ -776,7 +760,7 @@ __device__ void sm_prolong(const T* coarse, T* fine, bool add)
             ++k;
         }
     }
-    sm_sync<W>();
+    __syncthreads();
 }
 
 // The correction of the black nodes alone (the red half-sweep after it does not
@@ -803,23 +787,23 @@ __device__ void sm_correct(const T* coarse, T* fine)
     __syncthreads();
 }
 
-template <typename T, int N, bool W = false>
+template <typename T, int N>
 __device__ void sm_fill(T* a, T val)
 {
     constexpr int TOT = (N + 1) * (N + 1) * (N + 1);
-    for (int t = threadIdx.x; t < TOT; t += sm_stride<W>()) a[t] = val;
-    sm_sync<W>();
+    for (int t = threadIdx.x; t < TOT; t += (int)blockDim.x) a[t] = val;
+    __syncthreads();
 }
 
 // The single unknown of the 3^3 grid (Section 2): u = (sum of 6 nbrs - h^2 f)/6.
-template <typename T, bool W = false>
+template <typename T>
 __device__ void sm_coarsest(T* u, const T* f, T h)
 {
     if (threadIdx.x == 0) {
         const T sum = (u[14] + u[12]) + (u[16] + u[10]) + (u[22] + u[4]);
         u[13] = (sum - h * h * f[13]) * (T(1) / T(6));
     }
-    sm_sync<W>();
+    __syncthreads();
 }
 
 // --- the levels n = 8 and 16 with a row of nodes per thread ---------------------------------------------------------
@@ -1213,7 +1197,7 @@ __device__ void sm_vcycle(CoarseSmem<T>& S, T h, int npre, int npost)
         row.store_u(S.u[L]);
     } else {
         for (int q = 0; q < npre; ++q) {
-            if (ZERO && q == 0) sm_relax<T, N, false, true>(S.u[L], S.f[L], h * h, 0);
+            if (ZERO && q == 0) sm_relax<T, N, true>(S.u[L], S.f[L], h * h, 0);
             else sm_relax<T, N>(S.u[L], S.f[L], h * h, 0);
             sm_relax<T, N>(S.u[L], S.f[L], h * h, 1);
         }
@@ -1279,7 +1263,7 @@ __device__ void sm_fmg_up(CoarseSmem<T>& S, T h0, int ncycle, int npre, int npos
     } else {
         sm_fmg_up<T, L - 1>(S, h0, ncycle, npre, npost);
         const T h = h0 / T(1 << L);
-        sm_prolong<T, (2 << (L - 1))>(S.u[L - 1], S.u[L], false);
+        sm_prolong<T, (2 << (L - 1))>(S.u[L - 1], S.u[L]);
         for (int c = 0; c < ncycle; ++c) sm_vcycle<T, L>(S, h, npre, npost);
     }
 }
