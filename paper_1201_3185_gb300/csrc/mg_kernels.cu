@@ -594,7 +594,9 @@ __global__ void set_boundary_kernel(T* __restrict__ e, LevelView v, const double
 //  fmg = 1: full multigrid from 3^3 up to `top` (boundary values injected
 //           from u64, or zero), ncycle V-cycles per level;
 //  fmg = 0: one V-cycle from a zero initial guess with zero boundary values.
-// The result (all nodes, boundary included) is written to e.
+// With fmg = 1 all nodes of e are written, boundary values included; with
+// fmg = 0 the boundary entries of e must be zero on entry and stay so (the
+// prolongation that reads e next reads them too), the interior is written.
 // The shared-memory routines below stride over their nodes by the block's
 // size: the coarse-grid kernel runs them with kCoarseThreads, the cooperative
 // and cluster V-cycle kernels with kVsubThreads.  (1024 threads for the

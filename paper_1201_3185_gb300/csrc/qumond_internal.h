@@ -110,6 +110,8 @@ int vcluster_size(bool fp64);
 cudaError_t launch_vslab(float* e, const float* f, const LevelView& v, double h, double hc, int zero_top, int npre,
                          int npost, int csize, cudaStream_t s, const Sets& sets);
 int vslab_size(int want);
+// The levels n <= 16 in one block per set: fmg = 1 full multigrid with boundary values from u64 (zero without it), all
+// nodes of e written; fmg = 0 one V-cycle from zero, the boundary entries of e zero on entry and left so.
 template <typename T> cudaError_t launch_coarse(int fmg, T* e, const T* f, const LevelView& v, double h,
                                                 const double* u64, int nfine, int ncycle, int npre, int npost,
                                                 cudaStream_t s, const Sets& sets = Sets());

@@ -1,5 +1,6 @@
 """Whole red-black sweeps (one pass per sweep, FP32 levels n >= 32): the memory that a context takes for them, and
-their bits against the half-sweeps over the launch shapes they are chosen for."""
+their bits against the half-sweeps over the launch shapes they are chosen for; the corrections that follow an FMG with
+boundary values on the same context."""
 import pytest
 import torch
 
@@ -74,3 +75,29 @@ def test_a_context_without_room_for_the_second_black_arrays(q, precision, n, set
     del filler
     torch.cuda.empty_cache()
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("n", [4, 8, 16, 32, 64, 128])
+def test_corrections_after_an_fmg_with_boundary_values(q, precision, n):
+    # FMG leaves boundary values on its way up every level, and the corrections after it read zeros there: on the same
+    # context the same bits as on one that never ran an FMG, from the same start
+    g = torch.Generator(device="cuda").manual_seed(n)
+    src = torch.rand((n + 1) ** 3, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    given = torch.rand_like(src) + 1.0
+    kw = dict(n=n, nboxes=1, L0=64.0, precision=precision, bc_mode=q.QUMOND_BC_GIVEN, ncycle=1)
+    tol = dict(rel_tol=1e-6, max_vcycles=60)
+    ctx = q.Context(**kw)
+    start = given.clone()
+    ctx.qumond_solve_mond(0, src, None, start)
+    ctx.close()
+    ctx = q.Context(**kw, **tol)
+    for _ in range(2):  # the second solve also follows the first's corrections
+        a = given.clone()
+        ctx.qumond_solve_mond(0, src, None, a)
+    ctx.close()
+    ctx = q.Context(**kw, **tol, warm_start=1)
+    b = start.clone()
+    ctx.qumond_solve_mond(0, src, None, b)
+    ctx.close()
+    assert torch.equal(a, b)
