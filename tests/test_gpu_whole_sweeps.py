@@ -101,3 +101,56 @@ def test_corrections_after_an_fmg_with_boundary_values(q, precision, n):
     ctx.qumond_solve_mond(0, src, None, b)
     ctx.close()
     assert torch.equal(a, b)
+
+
+def _two_cycles(q, src, n, sets, **kw):
+    """Two V-cycles on src from zero, on the finest level as: the FMG's own ones with zero boundary values (whole sweeps
+    where they apply, from black values that are zero), the FMG's own ones with boundary values given (half-sweeps), and
+    one step of the defect correction from zero (whole sweeps whose first starts from zero)."""
+    kw = dict(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, nsets=sets, **kw)
+    out = []
+    for case in (dict(ncycle=2), dict(ncycle=2, bc_mode=q.QUMOND_BC_GIVEN),
+                 dict(warm_start=1, dc_vcycles=2, max_vcycles=2, rel_tol=0.9)):
+        ctx = q.Context(**kw, **case)
+        phi = torch.zeros_like(src)
+        ctx.qumond_solve_mond(0, src, None, phi)
+        ctx.close()
+        out.append(phi)
+    return out
+
+
+# sets: the launches of n = 32, 64, 128 take their large tiles from 2^20 groups of four entries in all sets on (273, 34
+# and 5 sets), those of n = 256 with any; from n = 512 the tiles run along the rows too (2 and 4 of them)
+@pytest.mark.parametrize("npre,npost", [(2, 2), (4, 2), (1, 2), (3, 1)])  # odd ones: the fallback
+@pytest.mark.parametrize("n,sets", [(32, 1), (32, 280), (64, 1), (64, 34), (128, 1), (128, 8), (256, 1), (256, 2),
+                                    (512, 1), (512, 2), (1024, 1)])
+def test_sweeps_from_zero_give_the_bits_of_the_half_sweeps(q, n, sets, npre, npost):
+    # a source that alternates along x: its full weighting is exactly zero, so FMG brings a zero to the finest level and
+    # the V-cycles there start from zero in all three runs.  The coarser levels' corrections are the same launches in
+    # all three, so each level's launches are compared where it is the finest
+    if n == 1024 and (npre, npost) != (2, 2):
+        pytest.skip("one size of four tiles along a row is enough")
+    g = torch.Generator(device="cuda").manual_seed(n + sets)
+    src = torch.rand(sets, n + 1, n + 1, 1, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    src = (src * (1.0 - 2.0 * (torch.arange(n + 1, device="cuda") % 2))).reshape(-1)
+    own, given, corrected = _two_cycles(q, src, n, sets, npre=npre, npost=npost)
+    assert torch.equal(own, given)
+    assert torch.equal(corrected, given)
+    assert torch.all(torch.isfinite(own)) and torch.any(own != 0.0)
+
+
+@pytest.mark.parametrize("npre,npost", [(1, 1), (1, 2), (3, 1)])
+def test_odd_counts_to_a_tolerance_give_the_bits_of_the_solve_without_allocation(q, npre, npost):
+    # the half-sweeps that odd counts run, first sweeps from zero in one launch among them
+    n = 64
+    g = torch.Generator(device="cuda").manual_seed(npre + npost)
+    src = torch.rand((n + 1) ** 3, dtype=torch.float64, device="cuda", generator=g) - 0.5
+    kw = dict(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, npre=npre, npost=npost, ncycle=1, rel_tol=1e-9,
+              max_vcycles=60, dc_vcycles=2)
+    ctx = q.Context(**kw)
+    a = torch.zeros_like(src)
+    ctx.qumond_solve_mond(0, src, None, a)
+    ctx.close()
+    b = torch.zeros_like(src)
+    q.qumond.qumond_solve_mond_noalloc(q.default_params(**kw), 0, src, None, b)
+    assert torch.equal(a, b)
