@@ -168,6 +168,7 @@ void conv(qumond_guess* g, int l, cudaStream_t s)
     a.out = w.out, a.ld_out = w.ld_out, a.out_off = w.out_off, a.cout = kLayers[l].cout;
     a.relu = 1;
     a.S = g->S >> kLayers[l].level;
+    a.sms = g->sms;
     a.use_tc = g->use_tc;
     a.fault = g->fault;
     launch_conv3(a, s);
@@ -220,6 +221,7 @@ void backward(qumond_guess* g, const __nv_bfloat16* target, float k, float loss_
         ConvArgs a{};
         a.in = g->G[l], a.ld_in = cout, a.in_off = 0, a.cin = cout;
         a.w = g->wd[l], a.bias = nullptr, a.relu = 0, a.cout = cin, a.S = S;
+        a.sms = g->sms;
         a.use_tc = g->use_tc;
         a.fault = g->fault;
         const bool from_pool = (l == 2 || l == 4 || l == 6);

@@ -26,6 +26,7 @@ struct ConvArgs {
     int ld_mask, mask_off;
     int relu;
     int S;
+    int sms;      // multiprocessors of the device
     Brick brick;  // set by the launcher
     int stages;   // set by the launcher: chunks of input channels in flight
     int use_tc;   // 1: the convolution may run on the tcgen05 path (where conv3_tc_applies); 0: mma.sync
@@ -63,10 +64,10 @@ __device__ __forceinline__ void cp_async_wait(int pending)
 
 Brick brick_for(int S);
 size_t conv3_smem_bytes(int cout_tile);
-int conv3_tile(int cout, int bricks);  // output channels of a block
+int conv3_tile(int cout, int bricks, int sms);  // output channels of a block
 constexpr size_t kConvSmem = 226 * 1024;  // of a multiprocessor, for the chunk rings of its blocks
 constexpr int kConvStages = 4;
-int conv3_stages(size_t stage_bytes, int blocks, int chunks);
+int conv3_stages(size_t stage_bytes, int blocks, int chunks, int sms);
 // the most that conv3_stages gives a block
 inline size_t conv3_smem_max(size_t stage_bytes)
 {

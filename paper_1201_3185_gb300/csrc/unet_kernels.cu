@@ -218,20 +218,20 @@ size_t conv3_smem_bytes(int cout_tile)
 // channels at 16^3: 101 us, 82 us with 16; 128 -> 128 at 8^3: 73 us, 43 us; before
 // the ring of chunks).  An
 // output channel's sums do not depend on the tile.
-int conv3_tile(int cout, int bricks)
+int conv3_tile(int cout, int bricks, int sms)
 {
     const int tiles[3] = {64, 48, 32};
     for (int t : tiles)
-        if (cout % t == 0 && (long long)bricks * (cout / t) >= 152) return t;
+        if (cout % t == 0 && (long long)bricks * (cout / t) >= sms) return t;
     return 16;
 }
 
 // Buffers of a chunk ring: the shared memory of a multiprocessor divided among
 // the blocks it gets, at least one buffer each (many blocks hide one another's
 // loads; a single block needs its next chunks in flight), at most four.
-int conv3_stages(size_t stage_bytes, int blocks, int chunks)
+int conv3_stages(size_t stage_bytes, int blocks, int chunks, int sms)
 {
-    const int per_sm = (blocks + 151) / 152;
+    const int per_sm = (blocks + sms - 1) / sms;
     int stages = (int)(kConvSmem / (per_sm * (stage_bytes + 2048)));  // 1 KB a block is the system's; static arrays
     if (stages > chunks) stages = chunks;
     if (stages > kConvStages) stages = kConvStages;
@@ -243,7 +243,7 @@ static void launch_conv3_t(ConvArgs a, int bricks, cudaStream_t s)
 {
     const int nt = NTILES * 8;
     const int blocks = bricks * (a.cout / nt);
-    a.stages = conv3_stages(conv3_smem_bytes(nt), blocks, a.cin / 16);
+    a.stages = conv3_stages(conv3_smem_bytes(nt), blocks, a.cin / 16, a.sms);
     conv3_kernel<NTILES><<<dim3(bricks, a.cout / nt), 256, a.stages * conv3_smem_bytes(nt), s>>>(a);
 }
 
@@ -267,7 +267,7 @@ void launch_conv3(ConvArgs a, cudaStream_t s)
     }
     a.brick = brick_for(a.S);
     const int bricks = (a.S / a.brick.bx) * (a.S / a.brick.by) * (a.S / a.brick.bz);
-    switch (conv3_tile(a.cout, bricks)) {
+    switch (conv3_tile(a.cout, bricks, a.sms)) {
     case 64: launch_conv3_t<8>(a, bricks, s); break;
     case 48: launch_conv3_t<6>(a, bricks, s); break;
     case 32: launch_conv3_t<4>(a, bricks, s); break;

@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
 // where the level leaves at least four blocks for every multiprocessor (64^3,
 // 16 -> 16 channels: 20 us with one plane, 18 with two; 48 -> 16: 54 and 47;
 // 16 -> 48: 35 and 27).
-static int conv3_tc_planes(int blocks) { return blocks >= 2 * 4 * 152 ? 2 : 1; }
+static int conv3_tc_planes(int blocks, int sms) { return blocks >= 2 * 4 * sms ? 2 : 1; }
 
 bool conv3_tc_applies(const ConvArgs& a)
 {
@@ -362,10 +362,10 @@ void prepare_conv3_tc()
 template <int NT>
 static void launch_tc(ConvArgs a, int bricks, cudaStream_t s)
 {
-    const int tiles = a.cout / NT, zp = conv3_tc_planes(bricks * tiles);
+    const int tiles = a.cout / NT, zp = conv3_tc_planes(bricks * tiles, a.sms);
     const size_t stage = conv3_tc_stage_bytes(NT, zp);
     const dim3 grid((unsigned)(bricks / zp), (unsigned)tiles);
-    a.stages = conv3_stages(stage, (int)(grid.x * grid.y), a.cin / 16);
+    a.stages = conv3_stages(stage, (int)(grid.x * grid.y), a.cin / 16, a.sms);
     if (zp == 2)
         conv3_tc_kernel<NT, 2><<<grid, 128, a.stages * stage, s>>>(a);
     else
@@ -375,7 +375,7 @@ static void launch_tc(ConvArgs a, int bricks, cudaStream_t s)
 void launch_conv3_tc(ConvArgs a, cudaStream_t s)
 {
     const int bricks = (a.S / 8) * (a.S / 16) * a.S;
-    switch (conv3_tile(a.cout, bricks)) {
+    switch (conv3_tile(a.cout, bricks, a.sms)) {
     case 64: launch_tc<64>(a, bricks, s); break;
     case 48: launch_tc<48>(a, bricks, s); break;
     case 32: launch_tc<32>(a, bricks, s); break;
