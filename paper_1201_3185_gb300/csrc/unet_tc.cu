@@ -334,7 +334,12 @@ __global__ void __launch_bounds__(128) conv3_tc_kernel(ConvArgs a)
 // Planes of a brick: two share the chunk's weights and two of their halo planes,
 // where the level leaves at least four blocks for every multiprocessor (64^3,
 // 16 -> 16 channels: 20 us with one plane, 18 with two; 48 -> 16: 54 and 47;
-// 16 -> 48: 35 and 27).
+// 16 -> 48: 35 and 27).  Whole networks, one plane everywhere and this rule in
+// turn (each side within 0.4 %, the same bits): gradients of a batch of two at
+// 64^3 2029 and 1983 us; of one at 48^3 814 and 812, at 80^3 1600 and 1543, at
+// 96^3 2155 and 2018, at 128^3 4038 and 3618; an inference at 128^3 1454 and
+// 1213.  With the line at eight blocks 64^3 and 96^3 lose (1017, 2036); at two
+// 48^3 and 96^3 take 803 and 1950 and nothing is slower, so it may lie lower.
 static int conv3_tc_planes(int blocks, int sms) { return blocks >= 2 * 4 * sms ? 2 : 1; }
 
 bool conv3_tc_applies(const ConvArgs& a)
