@@ -334,7 +334,10 @@ QUMOND_API qumond_status qumond_set_barrier_poll_limit(qumond_ctx* ctx, int64_t 
 
 /* Per-kernel-class counters of a context since it was created or last reset. */
 typedef struct {
-    const char* name;     /* kernel class, e.g. "rb_half_finest" (static storage) */
+    const char* name;     /* kernel class (static storage), e.g. "rb_half_finest",
+                             red-black half-sweeps of the finest level, or
+                             "sweep_finest", whole sweeps of it, with the
+                             correction or the restriction that some include */
     int64_t launches;     /* kernels of this class launched */
     double bytes;         /* algorithmic HBM bytes of those launches (the minimum
                              each kernel must read and write) */

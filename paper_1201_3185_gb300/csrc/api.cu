@@ -27,13 +27,14 @@ struct Level {
 enum Kind {
     K_DEPOSIT, K_FIXED_TO_RHO, K_BOUNDARY, K_CONVERT_RHS, K_RESTRICT_FULL, K_COARSE, K_RB_FINEST, K_RB_COARSER,
     K_RESTRICT_RESID, K_PROLONG, K_SET_BOUNDARY, K_ASSIGN_OUTER, K_RESIDUAL_OUTER, K_REDUCE, K_SOURCE, K_FORCES,
-    K_ROTATION_CURVE, K_FIXED_SETUP, K_FIXED_OUTPUT, K_CHI2, K_PROFILE, K_VSUB, K_FAR_FIELD, K_COUNT
+    K_ROTATION_CURVE, K_FIXED_SETUP, K_FIXED_OUTPUT, K_CHI2, K_PROFILE, K_VSUB, K_FAR_FIELD, K_SWEEP_FINEST,
+    K_SWEEP_COARSER, K_COUNT
 };
 const char* const kKindNames[K_COUNT] = {
     "cic_deposit", "fixed_to_rho", "boundary_fill", "convert_rhs", "restrict_full", "coarse_solver",
     "rb_half_finest", "rb_half_coarser", "restrict_resid_red", "prolong_black", "set_boundary", "update_outer",
     "residual_outer", "reduce_norms", "qumond_source", "forces", "rotation_curve", "fixed_setup", "fixed_output", "chi2", "profile", "vcycle_small_levels",
-    "far_field",
+    "far_field", "sweep_finest", "sweep_coarser",
 };
 constexpr int kMaxTimed = 32768;
 
@@ -339,7 +340,7 @@ void sweep(qumond_ctx* c, int l, SweepStart start, int q, SweepAfter after, doub
     const double words = 1.5 + (start == SweepStart::kZero ? 0.0 : 0.5) +
                          (start == SweepStart::kCorrected ? 0.125 : 0.0) +
                          (after == SweepAfter::kRed ? 0.5 : after == SweepAfter::kRestrict ? 0.125 : 0.0);
-    run(c, l == c->L ? K_RB_FINEST : K_RB_COARSER, words * cube(n) * sizeof(float), s, [&] {
+    run(c, l == c->L ? K_SWEEP_FINEST : K_SWEEP_COARSER, words * cube(n) * sizeof(float), s, [&] {
         launch_sweep(E<float>(c, l), c->lev[l].t, F<float>(c, l), c->lev[l].v, start, q % 2 == 0, after,
                      E<float>(c, l - 1), F<float>(c, l - 1), c->lev[l - 1].v, h, s, sets_of(c));
     });

@@ -154,3 +154,33 @@ def test_odd_counts_to_a_tolerance_give_the_bits_of_the_solve_without_allocation
     b = torch.zeros_like(src)
     q.qumond.qumond_solve_mond_noalloc(q.default_params(**kw), 0, src, None, b)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("npre,npost,bc,whole", [(2, 2, 0, True), (2, 4, 0, True), (1, 2, 0, False), (2, 2, 1, False)])
+def test_whole_sweeps_have_a_tracer_class_of_their_own(q, npre, npost, bc, whole):
+    # full multigrid on levels 128, 64, 32 (per-step form): its V-cycles, ncycle on each level, visit every level under
+    # it; the restriction and the correction of a whole sweep are not counted in the classes of their own launches.
+    # With boundary values given (bc 1) each level's own V-cycles are half-sweeps, the corrections under it whole ones
+    n, ncycle = 128, 2
+    ctx = q.Context(n=n, nboxes=1, L0=64.0, precision=q.QUMOND_PREC_MIXED, npre=npre, npost=npost, ncycle=ncycle,
+                    bc_mode=bc, persistent_vcycle=0, use_graphs=0)
+    src = torch.ones((n + 1) ** 3, dtype=torch.float64, device="cuda")
+    phi = torch.zeros_like(src)
+    ctx.qumond_trace_read(reset=True)
+    ctx.qumond_solve_mond(0, src, None, phi)
+    st, _, cells = ctx.qumond_trace_read(reset=True)
+    ctx.close()
+    count = {k: v.launches for k, v in st.items()}
+    sweeps = npre + npost
+    if whole:
+        assert count["sweep_finest"] == ncycle * sweeps
+        assert count["sweep_coarser"] == ncycle * sweeps * (2 + 3)  # 64 for itself and 128; 32 for itself, 64 and 128
+        assert count["rb_half_finest"] == count["rb_half_coarser"] == count["restrict_resid_red"] == 0
+        assert count["prolong_black"] == 3  # FMG's own, one a level
+    elif bc == 0:
+        assert count["sweep_finest"] == count["sweep_coarser"] == 0
+        assert count["rb_half_finest"] > 0 and count["rb_half_coarser"] > 0
+    else:
+        assert count["sweep_finest"] == 0
+        assert count["rb_half_finest"] == ncycle * 2 * sweeps
+        assert count["sweep_coarser"] == ncycle * sweeps * (1 + 2)  # 64 for 128; 32 for 64 and 128
