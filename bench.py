@@ -244,6 +244,21 @@ def solve_roofline(pipe1, ctx1, step, steps, peak, barrier, max_over_ranks):
                       "one chain (no concurrent solve); bytes = the algorithmic bytes of the solve kernels" % steps}
 
 
+def replay_one_chain(ctxs, run, times):
+    """Per-class statistics of `times` runs with every kernel launched on its own between two CUDA events."""
+    import torch
+    ctxs.qumond_trace_timing(True)
+    run()
+    torch.cuda.synchronize()
+    ctxs.qumond_trace_read(reset=True)
+    for _ in range(times):
+        run()
+    torch.cuda.synchronize()
+    st, _, _ = ctxs.qumond_trace_read(reset=True)
+    ctxs.qumond_trace_timing(False)
+    return st
+
+
 class Contexts:
     """The contexts of a pipeline, read and driven as one (tracer counters merged)."""
 
@@ -527,12 +542,16 @@ def run_ours(args):
     # --- kernels timed live: the same steps with one chain (no concurrent solve sharing
     # the GPU), the graphs carrying event-record nodes around each run of consecutive
     # launches of one kernel class in the FMG part of every solve.  The three classes
-    # with the most replay time are timed this way (one timed region each); the
-    # dominant kernel is the one with the most live time per step. ----------------------
+    # with the most replay time are timed this way (one timed region each); a class that
+    # has no launch there (the defect correction's whole sweeps: its loop is a conditional
+    # body, where event records cannot go) keeps its times from one-by-one launches with one
+    # chain.  The dominant kernel is the one with the most time per step. ---------------
     pipe1 = q.Pipeline(ctx.ctxs[0], dev)
     ctx1 = Contexts(ctx.ctxs[:1])
     candidates = [k.name for k in sorted(kstats.values(), key=lambda k: -k.ms)[:3]]
     live_by = {}
+    timed_in = {}
+    replay1 = None
     one_chain_ms = None
     for name in candidates:
         ctx1.qumond_trace_timing(True, only=name)
@@ -550,9 +569,15 @@ def run_ours(args):
         one_chain_ms = ms1 if one_chain_ms is None else min(one_chain_ms, ms1)
         st1, _, _ = ctx1.qumond_trace_read(reset=True)
         ctx1.qumond_trace_timing(False)
-        k = st1[name]
+        k, steps_k = st1[name], args.steps
+        timed_in[name] = "graphs"
+        if not k.timed:
+            if replay1 is None:
+                replay1 = replay_one_chain(ctx1, lambda: step(pipe1), min(args.steps, 5))
+            k, steps_k = replay1[name], min(args.steps, 5)
+            timed_in[name] = "launches"
         per_launch = k.ms / k.timed if k.timed else 0.0
-        live_by[name] = (k, per_launch * k.launches / args.steps)
+        live_by[name] = (k, per_launch * k.launches / steps_k)
     dom_name = max(live_by, key=lambda nm: live_by[nm][1])
     live = {dom_name: live_by[dom_name][0]}
     live_ms_per_step = {nm: v[1] for nm, v in live_by.items()}
@@ -570,11 +595,16 @@ def run_ours(args):
                 "algorithmic_bytes_per_launch": bytes_per_launch,
                 "avg_launch_ms": avg_ms, "timed_launches": dom.timed,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)" if peaks else "fallback 6.8 TB/s",
-                "timing": "CUDA event-record nodes around each run of consecutive launches of this kernel class in "
-                          "the FMG part of each solve's graph (e.g. the four half-sweeps of a pre-smoothing), read "
-                          "after each solve, over %d timed steps of the same workload run with one chain; achieved = "
-                          "algorithmic bytes of the timed launches / their time" % args.steps,
-                "live_ms_per_step_of_candidates": live_ms_per_step}
+                "timing": ("CUDA event-record nodes around each run of consecutive launches of this kernel class in "
+                           "the FMG part of each solve's graph (e.g. the four half-sweeps of a pre-smoothing), read "
+                           "after each solve, over %d timed steps of the same workload run with one chain; achieved "
+                           "= algorithmic bytes of the timed launches / their time" % args.steps)
+                if timed_in[dom_name] == "graphs" else
+                          ("CUDA events around every launch of this class, the kernels launched one by one over %d "
+                           "steps of the same workload run with one chain (the class runs in the defect correction's "
+                           "conditional loop, where event records cannot go); achieved = algorithmic bytes of the "
+                           "launches / their time, which includes a launch's start" % min(args.steps, 5)),
+                "live_ms_per_step_of_candidates": live_ms_per_step, "candidates_timed_in": timed_in}
     # --- the solve-level roofline: every FMG solve of the step (boundary values, FMG and the defect correction
     # to the tolerance) bracketed by CUDA events on its stream, with one chain so that no two solves overlap;
     # achieved = the algorithmic bytes of the solves' kernels / the solves' summed event time ----------------
@@ -757,15 +787,18 @@ def run_sweep(args):
     value = ws * w["sets"] * args.steps / (ms_total / 1000.0)
 
     # kernel classes timed live inside the batched graphs (the tuned batch, one lane): event-record nodes
-    # around each run of consecutive launches of the class in the FMG part of every solve
+    # around each run of consecutive launches of the class in the FMG part of every solve; a class that has no
+    # launch there, in the replay of one-by-one launches
     one = q.FitSweep(params(prec, choice["tile_small"], choice["persistent_vcycle"], choice["dc_vcycles"]),
                      batch=choice["batch"], lanes=1, **kw)
     c1 = Contexts(one.ctxs)
     nsub = choice["batch"]
     sub = tuple(a[:nsub * (a.numel() // w["sets"])] for a in sets)
     live = {}
-    for name in ("rb_half_finest", "rb_half_coarser", "restrict_resid_red", "prolong_black", "residual_outer",
-                 "coarse_solver"):
+    timed_in = {}
+    replay1 = replay_one_chain(c1, lambda: one.run(sub, dist[:nsub], v_obs, sigma), 1)
+    for name in ("sweep_finest", "sweep_coarser", "rb_half_finest", "rb_half_coarser", "restrict_resid_red",
+                 "prolong_black", "residual_outer", "coarse_solver"):
         c1.qumond_trace_timing(True, only=name)
         one.run(sub, dist[:nsub], v_obs, sigma)
         c1.qumond_trace_read(reset=True)
@@ -773,7 +806,8 @@ def run_sweep(args):
         torch.cuda.synchronize()
         st1, _, _ = c1.qumond_trace_read(reset=True)
         c1.qumond_trace_timing(False)
-        k = st1[name]
+        k = st1[name] if st1[name].timed else replay1[name]
+        timed_in[name] = "graphs" if st1[name].timed else "launches"
         if k.timed:
             live[name] = (k, k.ms / k.timed * k.launches / nsub)
     one.close()
@@ -787,8 +821,12 @@ def run_sweep(args):
                 "algorithmic_bytes_per_launch": dom.timed_bytes / dom.timed, "avg_launch_ms": dom.ms / dom.timed,
                 "timed_launches": dom.timed,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)" if peaks else "fallback 6.8 TB/s",
-                "timing": "CUDA event-record nodes around runs of this class's launches in the FMG part of each "
-                          "solve's graph; one context holding %d sets (every launch covers all of them)" % nsub,
+                "timing": ("CUDA event-record nodes around runs of this class's launches in the FMG part of each "
+                           "solve's graph" if timed_in[dom_name] == "graphs" else
+                           "CUDA events around every launch of this class, the kernels launched one by one (it runs "
+                           "in the defect correction's conditional loop, where event records cannot go)") +
+                          "; one context holding %d sets (every launch covers all of them)" % nsub,
+                "classes_timed_in": timed_in,
                 "live_ms_per_set": {nm: v[1] for nm, v in live.items()},
                 "live_GBps": {nm: v[0].timed_bytes / v[0].ms / 1e6 for nm, v in live.items() if v[0].ms}}
 
@@ -1208,10 +1246,10 @@ def run_reference(args):
 
 
 def profile_case(args):
-    """One box of the workload solved once, then a single V-cycle of defect
-    correction from that solution with every kernel launched on its own,
-    between cudaProfilerStart and cudaProfilerStop: the launches ncu sees
-    with --profile-from-start off are the finest-level ones first."""
+    """One box of the workload solved once, then one step of the defect
+    correction (two V-cycles) from that solution with every kernel launched on
+    its own, between cudaProfilerStart and cudaProfilerStop: the launches ncu
+    sees with --profile-from-start off are the finest-level ones first."""
     import torch
 
     import paper_1201_3185_gb300 as q
@@ -1220,8 +1258,8 @@ def profile_case(args):
     p = make_particles()
     dev = torch.device("cuda", 0)
     x, y, z, m = (torch.from_numpy(a).to(dev) for a in (p.x, p.y, p.z, p.m))
-    common = dict(n=w["n"], nboxes=1, L0=w["L0"], npre=w["npre"], npost=w["npost"], ncycle=w["ncycle"],
-                  precision=prec, use_graphs=0)
+    common = dict(n=w["n"], nboxes=1, L0=w["L0"], npre=args.smoothing or w["npre"],
+                  npost=args.smoothing or w["npost"], ncycle=w["ncycle"], precision=prec, use_graphs=0)
     ctx = q.Context(rel_tol=w["rel_tol"], max_vcycles=w["max_vcycles"], **common)
     nodes = ctx.nodes
     qf = torch.empty(nodes, dtype=torch.int64, device=dev)
@@ -1240,7 +1278,7 @@ def profile_case(args):
     torch.cuda.profiler.stop()
     ctx.close()
     ctx2.close()
-    print(json.dumps({"profile_case": "box 0 of the workload, one warm-start V-cycle", "n": w["n"],
+    print(json.dumps({"profile_case": "box 0 of the workload, one warm-start correction step", "n": w["n"],
                       "precision": args.precision}))
 
 
@@ -1278,7 +1316,10 @@ def main():
     ap.add_argument("--small-cluster", type=int, choices=[0, 4, 8, 16], default=0,
                     help="CTAs per cluster of --persistent-vcycle 3 (0: 8)")
     ap.add_argument("--profile-case", action="store_true",
-                    help="run one profiled V-cycle on one box instead of the benchmark (for ncu)")
+                    help="run one profiled correction step on one box instead of the benchmark (for ncu)")
+    ap.add_argument("--smoothing", type=int, default=0,
+                    help="--profile-case: pre- and post-smoothing sweeps of its V-cycles (an odd number runs the "
+                         "half-sweeps, restriction and correction of their own; 0: the workload's)")
     args = ap.parse_args()
     WORKLOAD.clear()
     WORKLOAD.update(WORKLOADS[args.workload])
