@@ -975,10 +975,16 @@ qumond_status create_ctx(const qumond_params* p, bool sweeps, qumond_ctx** out)
     for (int l = 0; l <= L; ++l) c->lev[l].v = make_view(2 << l);
     bool ok = prepare_kernels() == cudaSuccess;
     if (ok) choose_small_levels(c);
-    // every level's arrays in one zeroed allocation, each on a 256-byte boundary
+    // every level's arrays in one zeroed allocation, each on a 256-byte boundary, those of a megabyte and more on one of
+    // 2 MB, as allocations of their own would lie.  Which pages they share is worth a percent of a 129^3 solve with FP64
+    // corrections: one after another with the array t of the level n = 32 among them 1097, 1106 and 1111 us on three
+    // GPUs, without it 1107 on the first (also with the levels in the other order, or on 64 KB boundaries), so 1097,
+    // 1107 and 1104.
+    constexpr size_t kPage = (size_t)2 << 20;
     auto place = [&](unsigned char* base) {
         size_t used = 0;
         auto take = [&](size_t bytes) {
+            if (bytes >= kPage / 2) used = (used + kPage - 1) & ~(kPage - 1);
             unsigned char* at = base ? base + used : nullptr;
             used += (bytes + 255) & ~(size_t)255;
             return at;
