@@ -279,7 +279,8 @@ restrict_nodes_kernel(const float* __restrict__ ef, const float* __restrict__ ff
 }
 
 // FP64: a CTA takes 16 x 4 x 2 coarse nodes and evaluates each red residual under
-// them once into shared memory, 743 for 128 nodes.  With the 13 residuals of every
+// them once into shared memory, 765 for 128 nodes (the first of the even ones of
+// a row, 23 of them, belong to the tile beside).  With the 13 residuals of every
 // node evaluated anew it is bound by the two FP64 lanes a clock (a 129^3 solve of 36
 // restrictions: 785 us, 510 so, launches included); in FP32 at n = 32 and 64 it is
 // bound by latency, and the second phase costs more (33^3 solve: 398 us, 405 so).
